@@ -1,0 +1,263 @@
+// FP64 diagonal block of the partial Cholesky (step (b) of factor.cu): L_kk L_kk^T =
+// P[k:k+w, k:k+w] (w <= NB) written back, L_kk^-1 to Dinv.
+//
+// The FP64 pipe bounds it: an SM retires 1.65 FP64 FMAs per clock and a warp's FMA takes
+// 65 clocks, so the block's 0.7M FMAs are over 200 us on one SM whatever the schedule, and
+// a level near the root has few fronts.  A cluster of CL CTAs therefore takes one front:
+//   - the 32 x 32 diagonal sub-block is factored and inverted by every CTA (redundantly:
+//     cheaper than handing it on), one column per step, lane = row, the columns spread
+//     over the eight warps;
+//   - CTA q owns the block's rows congruent to q mod CL: their part of the panel
+//     L_IJ = A_IJ X_JJ^T, stored into every CTA's copy of L through distributed shared
+//     memory, and of the trailing update; the rows of the next diagonal sub-block go to
+//     every CTA the same way;
+//   - the inverse is spread by columns (four adjacent ones to a CTA), which needs no
+//     exchange: X_JK = -X_JJ sum_M L_JM X_MK.
+// Measured: one 128-block per launch 0.57 ms before (one CTA, the block in registers, two
+// barriers and a reciprocal square root per column for the factor and again for the
+// inverse), 0.14 ms on 8 CTAs; 64 fronts on 2 CTAs each 0.19 ms.
+// L fills the lower triangle of a 128 x 129 array, X (transposed, one column further
+// right) its upper triangle.
+#include <algorithm>
+
+#include "cluster.cuh"
+#include "rsd_internal.cuh"
+
+namespace rsd {
+namespace {
+
+constexpr int DT = 256, DW = DT / 32;    // threads, warps
+constexpr int SBK = 32;                  // sub-block
+constexpr int LD = NB + 1;               // row stride of L / X (odd: lanes over rows hit distinct banks)
+constexpr int SLD = SBK + 1;
+constexpr size_t DIAG_SMEM = sizeof(double) * ((size_t)NB * LD + 2 * SBK * SLD + 2 * SBK + 2);
+
+__device__ __forceinline__ void cl_st_f64(uint32_t a, double v) {
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+}
+
+// Cholesky of the 32 x 32 block in D (lower part) and its inverse, all eight warps: thread
+// (lane, warp) holds row `lane` of columns warp + 8 q of both.  On return D holds L and Y
+// the inverse (both with zeros above the diagonal).  Returns 1 on a pivot that is not
+// positive or not finite (replaced by 1; 1 / inf would hide an infinite pivot behind zeros).
+__device__ int chol_inv32(double* __restrict__ D, double* __restrict__ Y, double* __restrict__ col, double* __restrict__ dinv,
+                          int lane, int warp) {
+    double a[4], y[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int c = warp + DW * q;
+        a[q] = c <= lane ? D[lane * SLD + c] : 0.0;
+        y[q] = c == lane ? 1.0 : 0.0;
+    }
+    int bad = 0;
+#pragma unroll
+    for (int jb = 0; jb < 4; ++jb) {
+#pragma unroll 1
+        for (int jj = 0; jj < DW; ++jj) {
+            const int j = DW * jb + jj;
+            double* cj = col + (j & 1) * SBK;
+            if (warp == jj) {
+                double d = __shfl_sync(0xffffffffu, a[jb], j);
+                if (!(d > 0.0 && d <= 1.7976931348623157e308)) { bad = 1; d = 1.0; }
+                const double inv = rsqrt(d);
+                const double l = lane > j ? a[jb] * inv : (lane == j ? d * inv : 0.0);
+                a[jb] = l;
+                cj[lane] = l;
+                if (lane == 0) dinv[j & 1] = inv;
+            }
+            __syncthreads();
+            const double li = cj[lane];
+            // the next pivot's column first, then the rest right of column j
+#pragma unroll
+            for (int q = jb; q < 4; ++q)
+                if (warp + DW * q > j) a[q] -= li * cj[warp + DW * q];
+            // row j of the inverse, then the rows below it
+            const double inv = dinv[j & 1];
+#pragma unroll
+            for (int q = 0; q <= jb; ++q) {
+                if (warp + DW * q > j) continue;
+                const double xj = __shfl_sync(0xffffffffu, y[q], j) * inv;
+                y[q] = lane == j ? xj : (lane > j ? y[q] - li * xj : y[q]);
+            }
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int c = warp + DW * q;
+        D[lane * SLD + c] = c <= lane ? a[q] : 0.0;
+        Y[lane * SLD + c] = c <= lane ? y[q] : 0.0;
+    }
+    __syncthreads();
+    return bad;
+}
+
+template <int CL>
+__device__ __forceinline__ void cluster_or_cta_sync() {
+    if constexpr (CL > 1) cl_sync(); else __syncthreads();
+}
+
+template <int CL>
+__global__ void __launch_bounds__(DT, 1) k_chol_diag_f64(const FrontDesc* __restrict__ fronts, int k, int* __restrict__ err,
+                                                       int* __restrict__ bad_front) {
+    extern __shared__ __align__(16) unsigned char diag_smem[];
+    double* Lf = (double*)diag_smem;             // NB x LD
+    double* D = Lf + NB * LD;                    // 32 x SLD: the diagonal sub-block
+    double* Y = D + SBK * SLD;                   // 32 x SLD: its inverse
+    double* col = Y + SBK * SLD;                 // two columns
+    double* dinv = col + 2 * SBK;                // two reciprocal pivots
+    const FrontDesc f = fronts[blockIdx.x / CL];
+    if (f.s <= k) return;                        // the whole cluster
+    const int w = min(NB, f.s - k), nJ = (w + SBK - 1) / SBK;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int rank = CL > 1 ? (int)cl_rank() : 0;
+    double* P = (double*)f.P + (int64_t)k * f.ldp + k;
+    double* Dg = (double*)f.Dinv + (int64_t)(k / NB) * NB * NB;
+    // this CTA's rows, and the first diagonal sub-block (every CTA); identity past the front
+    for (int r = rank + CL * warp; r < nJ * SBK; r += CL * DW)
+        for (int c = lane; c <= r; c += 32) Lf[r * LD + c] = r < w ? P[(int64_t)r * f.ldp + c] : (r == c ? 1.0 : 0.0);
+    for (int e = tid; e < SBK * SBK; e += DT) {
+        const int r = e / SBK, c = e % SBK;
+        D[r * SLD + c] = c <= r ? (r < w ? P[(int64_t)r * f.ldp + c] : (r == c ? 1.0 : 0.0)) : 0.0;
+    }
+    __syncthreads();
+    int bad = 0;
+    for (int J = 0; J < nJ; ++J) {
+        const int o = SBK * J, below = SBK * (J + 1), rows = nJ * SBK;
+        if (J > 0) cluster_or_cta_sync<CL>();          // the sub-block's rows are in D
+        bad |= chol_inv32(D, Y, col, dinv, lane, warp);
+        // L_JJ out (one CTA), X_JJ into the columns this CTA owns
+        if (rank == J % CL)
+            for (int e = tid; e < SBK * SBK; e += DT) {
+                const int r = e / SBK, c = e % SBK;
+                if (c <= r && o + r < w) P[(int64_t)(o + r) * f.ldp + o + c] = D[r * SLD + c];
+            }
+        for (int e = tid; e < SBK * SBK; e += DT) {
+            const int c = e / SBK, r = e % SBK;
+            if (r >= c && ((o + c) >> 2) % CL == rank) Lf[(o + c) * LD + o + r + 1] = Y[r * SLD + c];
+        }
+        // panel: this CTA's rows below, L_rc = sum_m A_rm Y_cm
+        constexpr int UP = (96 / CL + DW - 1) / DW;
+        const int r_first = below + ((rank - below) % CL + CL) % CL;      // first own row >= below
+        double pv[UP];
+#pragma unroll
+        for (int u = 0; u < UP; ++u) {
+            const int r = r_first + CL * (warp + DW * u);
+            double s = 0.0;
+            if (r < rows)
+#pragma unroll 8
+                for (int m = 0; m < SBK; ++m) s += Lf[r * LD + o + m] * Y[lane * SLD + m];
+            pv[u] = s;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < UP; ++u) {
+            const int r = r_first + CL * (warp + DW * u);
+            if (r >= rows) continue;
+            double* dst = Lf + r * LD + o + lane;
+            *dst = pv[u];
+            if constexpr (CL > 1)
+                for (int q = 1; q < CL; ++q) cl_st_f64(cl_map(dst, (uint32_t)((rank + q) % CL)), pv[u]);
+            if (r < w) P[(int64_t)r * f.ldp + o + lane] = pv[u];
+        }
+        if (J + 1 < nJ) {
+            cluster_or_cta_sync<CL>();                 // the panel is complete in every CTA
+            // trailing update of this CTA's rows; a warp takes a row and 32 of its columns, the
+            // next diagonal sub-block (first column block of rows below .. below + 31) first,
+            // whose results go to every CTA
+            int it = 0;
+            for (int r = r_first; r < rows; r += CL) {
+                const int rb = r / SBK;
+                for (int cb = J + 1; cb <= rb; ++cb, ++it) {
+                    if (it % DW != warp) continue;
+                    const int c = cb * SBK + lane;
+                    double s = 0.0;
+#pragma unroll 8
+                    for (int m = 0; m < SBK; ++m) s += Lf[r * LD + o + m] * Lf[c * LD + o + m];
+                    if (c > r) continue;
+                    const double v = Lf[r * LD + c] - s;
+                    Lf[r * LD + c] = v;
+                    if (rb == J + 1) {
+                        double* dst = D + (r - below) * SLD + lane;
+                        *dst = v;
+                        if constexpr (CL > 1)
+                            for (int q = 1; q < CL; ++q) cl_st_f64(cl_map(dst, (uint32_t)((rank + q) % CL)), v);
+                    }
+                }
+            }
+        } else {
+            __syncthreads();
+        }
+        // block row J of the inverse, this CTA's columns: a warp takes a column c, lane = row;
+        // T = sum over blocks M of L_JM X_M,c, then X_J,c = -X_JJ T
+        int ic = 0;
+        for (int c0 = 4 * rank; c0 < o; c0 += 4 * CL)
+            for (int cc = 0; cc < 4; ++cc, ++ic) {
+                if (ic % DW != warp) continue;
+                const int c = c0 + cc, m0 = c & ~(SBK - 1);
+                const double* Lr = Lf + (o + lane) * LD;
+                const double* Xc = Lf + c * LD + 1;     // Xc[m] = X[m][c], m >= c
+                double t0 = 0.0, t1 = 0.0;
+#pragma unroll 4
+                for (int m = m0; m < o; m += 2) {
+                    t0 += Lr[m] * (m >= c ? Xc[m] : 0.0);
+                    t1 += Lr[m + 1] * (m + 1 >= c ? Xc[m + 1] : 0.0);
+                }
+                const double t = t0 + t1;
+                double x = 0.0;
+#pragma unroll 8
+                for (int m = 0; m < SBK; ++m) x -= Y[lane * SLD + m] * __shfl_sync(0xffffffffu, t, m);
+                Lf[c * LD + 1 + o + lane] = x;
+            }
+    }
+    __syncthreads();
+    // the inverse's columns of this CTA (zero above the diagonal and past the front)
+    for (int e = tid; e < NB * (NB / CL); e += DT) {
+        const int r = e / (NB / CL), q = e % (NB / CL);
+        const int c = (q >> 2) * 4 * CL + 4 * rank + (q & 3);
+        Dg[r * NB + c] = (r >= c && r < w) ? Lf[c * LD + 1 + r] : 0.0;
+    }
+    if (bad && rank == 0 && lane == 0) {
+        atomicExch(&err[ERR_NOT_SPD], 1);
+        atomicMin(&err[ERR_NOT_SPD_NODE], f.node);
+        bad_front[f.node] = 1;
+    }
+}
+
+template <int CL>
+int launch_cl(const FrontDesc* d_fronts, int nf, int k, int* err, int* bad_front, cudaStream_t st) {
+    RSD_CUDA_TRY(cudaFuncSetAttribute(k_chol_diag_f64<CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DIAG_SMEM));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(nf * CL));
+    cfg.blockDim = dim3(DT);
+    cfg.dynamicSmemBytes = DIAG_SMEM;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = CL;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    RSD_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_chol_diag_f64<CL>, d_fronts, k, err, bad_front));
+    count_launch();
+    return RSD_OK;
+}
+
+}  // namespace
+
+// The largest cluster that still gives every front with rows past k SMs of its own: the
+// FP64 pipes it adds are worth more than anything else to a lone block (see above), and
+// past one wave a larger cluster only queues.
+int launch_chol_diag_f64(Handle& h, int li, int k, cudaStream_t st) {
+    Level& L = h.levels[li];
+    int alive = 0;
+    for (auto& f : L.fronts) alive += f.s > k;
+    if (!alive) return RSD_OK;
+    const int nf = (int)L.fronts.size();
+    if (alive * 8 <= h.num_sms) return launch_cl<8>(L.d_fronts, nf, k, h.d_err, h.d_front_bad, st);
+    if (alive * 4 <= h.num_sms) return launch_cl<4>(L.d_fronts, nf, k, h.d_err, h.d_front_bad, st);
+    if (alive * 2 <= h.num_sms) return launch_cl<2>(L.d_fronts, nf, k, h.d_err, h.d_front_bad, st);
+    return launch_cl<1>(L.d_fronts, nf, k, h.d_err, h.d_front_bad, st);
+}
+
+}  // namespace rsd

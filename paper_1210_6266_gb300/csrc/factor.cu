@@ -263,153 +263,9 @@ __global__ void __launch_bounds__(256) k_gemm_simt(const GemmTask* __restrict__ 
 }
 
 // ---------------------------------------------------------------------------------
-// Diagonal block: Cholesky of P[k:k+w, k:k+w] (w <= NB), written back to P, and its
-// inverse stored as Dinv_k (NB x NB, zero padded).  One CTA per front whose interface
-// extends past k.  The block lives in registers, distributed over a 16 x 16 thread grid:
-// thread (tr, tc) holds e[a][b] = A[16a + tr][16b + tc].  The factorisation takes NB
-// right-looking column steps (the owners of column j broadcast it through shared memory,
-// every thread updates its 8 x 8 elements); the inverse takes NB right-looking row steps
-// of X = L^-1 on the identity.  Entries above the diagonal of the broadcast vectors are
-// zero, so the full-square updates leave finished columns intact; the upper triangle of
-// the register block is never read back.  Beyond w the block is padded with the identity.
-// ---------------------------------------------------------------------------------
-constexpr int DLD = NB + 1;     // shared-memory row stride of L
-
-template <typename T> __device__ __forceinline__ T rsqrt_t(T x);
-template <> __device__ __forceinline__ float rsqrt_t(float x) { return rsqrtf(x); }
-template <> __device__ __forceinline__ double rsqrt_t(double x) { return 1.0 / sqrt(x); }
-
-template <typename T>
-__device__ __forceinline__ T store_round(T x, bool rnd);
-template <>
-__device__ __forceinline__ double store_round(double x, bool) { return x; }
-template <>
-__device__ __forceinline__ float store_round(float x, bool rnd) {
-    if (!rnd) return x;
-    uint32_t r;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-    return __uint_as_float(r);
-}
-
-template <typename T>
-__global__ void __launch_bounds__(256) k_potrf_diag(const FrontDesc* __restrict__ fronts, int k,
-                                                   int* __restrict__ err, int round_tf32, int* __restrict__ bad_front) {
-    extern __shared__ unsigned char smem_raw[];
-    T* A = (T*)smem_raw;                 // L after the factorisation (upper part zero)
-    T* vb = A + NB * DLD;                // two broadcast vectors
-    const FrontDesc f = fronts[blockIdx.x];
-    if (f.s <= k) return;
-    const int w = min(NB, f.s - k);
-    const int tid = threadIdx.x, tr = tid >> 4, tc = tid & 15;
-    T* P = (T*)f.P;
-    T e[8][8];
-#pragma unroll
-    for (int a = 0; a < 8; ++a)
-#pragma unroll
-        for (int b = 0; b < 8; ++b) {
-            const int i = 16 * a + tr, c = 16 * b + tc;
-            e[a][b] = (i < w && c <= i) ? P[(int64_t)(k + i) * f.ldp + (k + c)] : (i == c ? (T)1 : (T)0);
-        }
-    int bad = 0;
-    // ---- Cholesky ----
-#pragma unroll
-    for (int jb = 0; jb < 8; ++jb) {
-#pragma unroll 1
-        for (int jj = 0; jj < 16; ++jj) {
-            const int j = 16 * jb + jj;
-            T* col = vb + (j & 1) * NB;
-            T own[8];
-            if (tc == jj) {
-#pragma unroll
-                for (int a = 0; a < 8; ++a) {
-                    own[a] = e[a][jb];
-                    col[16 * a + tr] = (16 * a + tr >= j) ? own[a] : (T)0;
-                }
-            }
-            __syncthreads();
-            T d = col[j];
-            if (!(d > (T)0)) { bad = 1; d = (T)1; }
-            const T inv = rsqrt_t(d), inv2 = inv * inv;
-            // rows and columns before block jb see a zero column entry, and entries right
-            // of the diagonal block (b > a) are never read: update the rest only
-            T ci[8], ck[8];
-#pragma unroll
-            for (int a = jb; a < 8; ++a) ci[a] = col[16 * a + tr] * inv2;
-#pragma unroll
-            for (int b = jb; b < 8; ++b) ck[b] = col[16 * b + tc];
-#pragma unroll
-            for (int a = jb; a < 8; ++a)
-#pragma unroll
-                for (int b = jb; b <= a; ++b) e[a][b] -= ci[a] * ck[b];
-            if (tc == jj) {
-#pragma unroll
-                for (int a = 0; a < 8; ++a) {
-                    const int i = 16 * a + tr;
-                    e[a][jb] = i > j ? own[a] * inv : (i == j ? d * inv : own[a]);
-                }
-            }
-        }
-    }
-    if (bad) {
-        atomicExch(&err[ERR_NOT_SPD], 1);
-        atomicMin(&err[ERR_NOT_SPD_NODE], f.node);
-        bad_front[f.node] = 1;
-    }
-#pragma unroll
-    for (int a = 0; a < 8; ++a)
-#pragma unroll
-        for (int b = 0; b < 8; ++b) {
-            const int i = 16 * a + tr, c = 16 * b + tc;
-            A[i * DLD + c] = c <= i ? e[a][b] : (T)0;
-            if (i < w && c <= i) P[(int64_t)(k + i) * f.ldp + (k + c)] = store_round(e[a][b], round_tf32 != 0);
-        }
-    // ---- inverse X = L^-1 ----
-#pragma unroll
-    for (int a = 0; a < 8; ++a)
-#pragma unroll
-        for (int b = 0; b < 8; ++b) e[a][b] = (16 * a + tr == 16 * b + tc) ? (T)1 : (T)0;
-    __syncthreads();
-#pragma unroll
-    for (int rb = 0; rb < 8; ++rb) {
-#pragma unroll 1
-        for (int rr = 0; rr < 16; ++rr) {
-            const int r = 16 * rb + rr;
-            T* row = vb + (r & 1) * NB;
-            const T ir = (T)1 / A[r * DLD + r];
-            if (tr == rr) {
-#pragma unroll
-                for (int b = 0; b < 8; ++b) {
-                    e[rb][b] *= ir;
-                    row[16 * b + tc] = e[rb][b];
-                }
-            }
-            __syncthreads();
-            // X[i][c] -= L[i][r] X[r][c] touches rows i > r (blocks a >= rb) and columns
-            // c <= r (blocks b <= rb) only
-            T li[8], xr[8];
-#pragma unroll
-            for (int a = rb; a < 8; ++a) li[a] = (16 * a + tr > r) ? A[(16 * a + tr) * DLD + r] : (T)0;
-#pragma unroll
-            for (int b = 0; b <= rb; ++b) xr[b] = row[16 * b + tc];
-#pragma unroll
-            for (int a = rb; a < 8; ++a)
-#pragma unroll
-                for (int b = 0; b <= rb; ++b) e[a][b] -= li[a] * xr[b];
-        }
-    }
-    T* D = (T*)f.Dinv + (int64_t)(k / NB) * NB * NB;
-#pragma unroll
-    for (int a = 0; a < 8; ++a)
-#pragma unroll
-        for (int b = 0; b < 8; ++b) {
-            const int i = 16 * a + tr, c = 16 * b + tc;
-            D[i * NB + c] = (i < w && c <= i) ? store_round(e[a][b], round_tf32 != 0) : (T)0;
-        }
-}
-
-// ---------------------------------------------------------------------------------
-// FP32 diagonal block, blocked by 32: the same result as k_potrf_diag (Cholesky of
-// P[k:k+w, k:k+w] written back, its inverse to Dinv_k) with a short critical path.
+// FP32 diagonal block, blocked by 32: Cholesky of P[k:k+w, k:k+w] (w <= NB) written back,
+// its inverse to Dinv_k (NB x NB, zero padded), one CTA per front whose interface extends
+// past k (FP64 blocks: diag_f64.cu), with a short critical path.
 // Shared memory holds the block A (L in its lower triangle), the inverse X, the current
 // 32-column panel transposed (LT[m][r] = L[r][32J + m]), the current diagonal inverse
 // transposed (XT[c][r] = X_JJ[r][c]) and the columns of L_JJ, rotated so that row j
@@ -1535,13 +1391,11 @@ int run_factor_level(Handle& h, int li) {
     // task buffer for this level: one slot per front per launch kind
     GemmTask* d_tasks = nullptr;
     RSD_CUDA_TRY(cudaMallocAsync((void**)&d_tasks, sizeof(GemmTask) * L.fronts.size() * 2 + 64, h.stream));
-    const size_t potrf_smem = f64 ? (size_t)NB * DLD * es + (size_t)2 * NB * es : POTRF_BLK_SMEM;
     const size_t trsm_smem = (size_t)NB * NB * es + (size_t)TR_ROWS * (NB + 1) * es;
     if (f64) {
-        RSD_CUDA_TRY(cudaFuncSetAttribute(k_potrf_diag<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)potrf_smem));
         RSD_CUDA_TRY(cudaFuncSetAttribute(k_trsm_simt<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)trsm_smem));
     } else {
-        RSD_CUDA_TRY(cudaFuncSetAttribute(k_potrf_diag_blk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)potrf_smem));
+        RSD_CUDA_TRY(cudaFuncSetAttribute(k_potrf_diag_blk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)POTRF_BLK_SMEM));
         RSD_CUDA_TRY(cudaFuncSetAttribute(k_trsm_simt<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)trsm_smem));
     }
     std::vector<GemmTask> tasks;
@@ -1603,9 +1457,13 @@ int run_factor_level(Handle& h, int li) {
         for (auto& f : L.fronts)
             if (f.s > k) { const double w = std::min(NB, f.s - k); pf += 2.0 * w * w * w / 3.0; pb += (2.0 * w * w + NB * NB) * es; }
         const int ppi = prof_begin(h, K_POTRF);
-        if (f64) k_potrf_diag<double><<<(unsigned)L.fronts.size(), 256, potrf_smem, h.stream>>>(L.d_fronts, k, h.d_err, 0, h.d_front_bad);
-        else k_potrf_diag_blk<<<(unsigned)L.fronts.size(), 256, potrf_smem, h.stream>>>(L.d_fronts, k, h.d_err, tc ? 1 : 0, h.d_front_bad);
-        count_launch();
+        if (f64) {
+            rc = launch_chol_diag_f64(h, li, k, h.stream);
+            if (rc != RSD_OK) break;
+        } else {
+            k_potrf_diag_blk<<<(unsigned)L.fronts.size(), 256, POTRF_BLK_SMEM, h.stream>>>(L.d_fronts, k, h.d_err, tc ? 1 : 0, h.d_front_bad);
+            count_launch();
+        }
         prof_end(h, ppi, pf, pb);
         if (cudaGetLastError() != cudaSuccess) { rc = RSD_ERR_CUDA; break; }
         // (c) panel solve below the diagonal block

@@ -353,6 +353,8 @@ int launch_assemble_fronts(Handle& h, int li, const int64_t* rowptr, const int* 
                            const int* tin, const int* tout);
 int launch_extend_add(Handle& h, int li);
 int run_factor_level(Handle& h, int li);
+// FP64 diagonal block factor + inverse at column k of every front of level li (diag_f64.cu)
+int launch_chol_diag_f64(Handle& h, int li, int k, cudaStream_t st);
 // nonsymmetric fronts: assembly, extend-add and LU partial factorisation of level li
 int launch_assemble_fronts_lu(Handle& h, int li, const int64_t* rowptr, const int* col, const double* val,
                               const int* owner, const int* rank, const int* tin, const int* tout);
