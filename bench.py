@@ -581,7 +581,9 @@ def form_record(res, ms, t_setup, t_solve, n_dof, steps, pk, peak_rec, form, pro
     tc_classes = [k for k in ("gemm_tcgen05_f16", "gemm_tcgen05") if classes.get(k, {}).get("launches")]
     if tc_classes:
         bf = pk["bf16_tflops_sustained"]
-        cls_peak = {"gemm_tcgen05": bf * NOMINAL_TF32 / NOMINAL_BF16, "gemm_tcgen05_f16": bf}
+        # an FP64 front's products are split into 36 exact FP16 ones each
+        parts = 36 if form == "fp64" else 1
+        cls_peak = {"gemm_tcgen05": bf * NOMINAL_TF32 / NOMINAL_BF16, "gemm_tcgen05_f16": bf / parts}
         counted = sum(classes[k]["flops"] for k in tc_classes)
         per_cls, t_min, t_act = {}, 0.0, 0.0
         for k in tc_classes:
@@ -597,11 +599,12 @@ def form_record(res, ms, t_setup, t_solve, n_dof, steps, pk, peak_rec, form, pro
         roof = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "peak_source": (f"measured BF16 sustained {bf} TFLOP/s for the kind::f16 launches (FP16 and BF16 "
                                 f"share the dense rate), x {NOMINAL_TF32}/{NOMINAL_BF16} (nominal ratio) for the "
-                                f"kind::tf32 launches; the peak is the flop-weighted combination"),
+                                f"kind::tf32 launches; the peak is the flop-weighted combination"
+                                + (f"; {parts} FP16 products per FP64 product" if parts > 1 else "")),
                 "classes": per_cls}
         if peak_rec:
             own = {"gemm_tcgen05": peak_rec["tf32_tcgen05"]["sustained"],
-                   "gemm_tcgen05_f16": peak_rec["fp16_tcgen05"]["sustained"]}
+                   "gemm_tcgen05_f16": peak_rec["fp16_tcgen05"]["sustained"] / parts}
             t_own = sum(per_cls[k]["algorithmic_flops"] / (own[k] * 1e12) for k in tc_classes)
             roof["frac_of_own_kernel_peak"] = t_own / t_act
         gemm_cls = "+".join(tc_classes)

@@ -44,7 +44,10 @@ extern "C" {
 #define RSD_ERR_NOCONV     (-7)  /* Krylov solve hit maxit; x and stats still filled */
 
 /* ---- precisions of the stored factors and the arithmetic on them ----------------- */
-#define RSD_PREC_FP64  0   /* FP64 storage, FP64 arithmetic on CUDA cores                */
+#define RSD_PREC_FP64  0   /* FP64 storage and accuracy: the factorisation's products are split
+                              into exact FP16 products on tcgen05 tensor cores and rounded to
+                              FP64 once; diagonal blocks and sweeps (and nonsymmetric fronts)
+                              in FP64 on CUDA cores                                      */
 #define RSD_PREC_FP32  1   /* FP32 storage, FP32 arithmetic on CUDA cores                */
 #define RSD_PREC_TF32  2   /* FP32 storage; GEMM/TRSM updates on tcgen05 tensor cores in
                               TF32 with FP32 accumulation; diagonal blocks in FP32       */
@@ -168,7 +171,7 @@ typedef struct {
  * (the entries the sweeps read), 11 inner GMRES of paper mode with gamma > 0: its Arnoldi
  * steps (start vector, modified Gram-Schmidt, least-squares finish) of one interface
  * level, 12 tcgen05 GEMM on 16-bit operand copies (kind::f16; class 2 is then the
- * kind::tf32 launches only), 13 the leaf-coupling products of paper mode's S-MatVecs
+ * kind::tf32 launches only; FP64 levels' split products, whose splitting counts in class 10), 13 the leaf-coupling products of paper mode's S-MatVecs
  * (bytes = the X rows streamed), 14 the interface part of those S-MatVecs (K_II x less
  * the coupling terms).                                                                  */
 #define RSD_PROFILE_CLASSES 15

@@ -1036,13 +1036,30 @@ static int build_handle(Handle& h, Analysis& a, const int64_t* rowptr, const int
     const size_t o_err = take(sizeof(int) * ERR_SLOTS);
     const size_t o_bad = take(sizeof(int) * a.n_nodes);
     const size_t o_ticket = take(sizeof(int) * 2 * nl + 16);
-    h.arena_bytes = off;
+    // FP64 fronts factored on the tensor cores: the digits of one panel, last in the arena
+    // (levels are factored one after another and share it); without room for it the FP64
+    // levels run on the FP64 pipe as before
+    size_t f64_ws = 0;
+    if (!h.lu)
+        for (int d = 0; d < nl; ++d) {
+            if (!is_fp64(h.levels[d].prec) || !h.levels[d].factored) continue;
+            std::vector<int> rows;
+            for (int t : h.levels[d].nodes) rows.push_back(a.I_off[t + 1] - a.I_off[t] + beff(t));
+            f64_ws = std::max(f64_ws, f64_tc_workspace(rows));
+        }
+    const size_t o_f64 = off;
+    h.arena_bytes = off + f64_ws;
     {
         int dev = 0;
         cudaGetDevice(&dev);
         h.device = dev;
         size_t got = 0;
         h.arena = arena_take(h.arena_bytes, dev, &got);
+        if (!h.arena && f64_ws) {
+            f64_ws = 0;
+            h.arena_bytes = off;
+            h.arena = arena_take(h.arena_bytes, dev, &got);
+        }
         if (!h.arena) {
             set_last_error("device arena of " + std::to_string(h.arena_bytes) + " bytes");
             return RSD_ERR_NOMEM;
@@ -1050,6 +1067,10 @@ static int build_handle(Handle& h, Analysis& a, const int64_t* rowptr, const int
         h.arena_capacity = got;
     }
     char* A = h.arena;
+    if (f64_ws) {
+        h.f64_ws = A + o_f64;
+        h.f64_ws_bytes = f64_ws;
+    }
     h.d_rowptr = (int64_t*)(A + o_rowptr);
     h.d_col = (int*)(A + o_col);
     h.d_val = (double*)(A + o_val);

@@ -36,6 +36,21 @@ __device__ __forceinline__ void cl_st_f64(uint32_t a, double v) {
     asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
 }
 
+// 1 / sqrt(d) for d > 0: an FP32 estimate y of the reduced argument (2^-21) and one
+// third-order Householder step, y + y e (1/2 + 3/8 e) with e = 1 - d y^2: four FMAs deep on the
+// chain from pivot to pivot (about 320 clocks; rsqrt() takes 358, 1 / sqrt(d) 960).
+__device__ __forceinline__ double rsqrt_chain(double d) {
+    const long long b = __double_as_longlong(d);
+    const int ex = (int)(b >> 52) - 1023;
+    if (ex < -1000 || ex > 1000) return 1.0 / sqrt(d);
+    const int q = ex >> 1;                                         // d = f 4^q, f in [1, 4)
+    const float f = __int_as_float(((ex - 2 * q + 127) << 23) | (int)((b >> 29) & 0x7fffff));
+    const int yb = __float_as_int(rsqrtf(f));
+    const double y = __longlong_as_double(((long long)((yb >> 23) - 127 + 1023 - q) << 52) | ((long long)(yb & 0x7fffff) << 29));
+    const double e = fma(-(d * y), y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
 // Cholesky of the 32 x 32 block in D (lower part) and its inverse, all eight warps: thread
 // (lane, warp) holds row `lane` of columns warp + 8 q of both.  On return D holds L and Y
 // the inverse (both with zeros above the diagonal).  Returns 1 on a pivot that is not
@@ -59,7 +74,7 @@ __device__ int chol_inv32(double* __restrict__ D, double* __restrict__ Y, double
             if (warp == jj) {
                 double d = __shfl_sync(0xffffffffu, a[jb], j);
                 if (!(d > 0.0 && d <= 1.7976931348623157e308)) { bad = 1; d = 1.0; }
-                const double inv = rsqrt(d);
+                const double inv = rsqrt_chain(d);
                 const double l = lane > j ? a[jb] * inv : (lane == j ? d * inv : 0.0);
                 a[jb] = l;
                 cj[lane] = l;
@@ -248,16 +263,27 @@ int launch_cl(const FrontDesc* d_fronts, int nf, int k, int* err, int* bad_front
 // The largest cluster that still gives every front with rows past k SMs of its own: the
 // FP64 pipes it adds are worth more than anything else to a lone block (see above), and
 // past one wave a larger cluster only queues.
-int launch_chol_diag_f64(Handle& h, int li, int k, cudaStream_t st) {
+int launch_chol_diag_f64(Handle& h, int li, int f0, int nf, int k, cudaStream_t st) {
     Level& L = h.levels[li];
     int alive = 0;
-    for (auto& f : L.fronts) alive += f.s > k;
+    double flops = 0, bytes = 0;
+    for (int q = f0; q < f0 + nf; ++q) {
+        if (L.fronts[q].s <= k) continue;
+        const double w = std::min(NB, L.fronts[q].s - k);
+        ++alive;
+        flops += 2.0 * w * w * w / 3.0;
+        bytes += (2.0 * w * w + NB * NB) * 8;
+    }
     if (!alive) return RSD_OK;
-    const int nf = (int)L.fronts.size();
-    if (alive * 8 <= h.num_sms) return launch_cl<8>(L.d_fronts, nf, k, h.d_err, h.d_front_bad, st);
-    if (alive * 4 <= h.num_sms) return launch_cl<4>(L.d_fronts, nf, k, h.d_err, h.d_front_bad, st);
-    if (alive * 2 <= h.num_sms) return launch_cl<2>(L.d_fronts, nf, k, h.d_err, h.d_front_bad, st);
-    return launch_cl<1>(L.d_fronts, nf, k, h.d_err, h.d_front_bad, st);
+    const FrontDesc* fr = L.d_fronts + f0;
+    const int pi = prof_begin(h, K_POTRF, st);
+    int rc;
+    if (alive * 8 <= h.num_sms) rc = launch_cl<8>(fr, nf, k, h.d_err, h.d_front_bad, st);
+    else if (alive * 4 <= h.num_sms) rc = launch_cl<4>(fr, nf, k, h.d_err, h.d_front_bad, st);
+    else if (alive * 2 <= h.num_sms) rc = launch_cl<2>(fr, nf, k, h.d_err, h.d_front_bad, st);
+    else rc = launch_cl<1>(fr, nf, k, h.d_err, h.d_front_bad, st);
+    prof_end(h, pi, flops, bytes, st);
+    return rc;
 }
 
 }  // namespace rsd

@@ -1387,6 +1387,7 @@ int run_factor_level(Handle& h, int li) {
     if (L.fronts.empty()) return RSD_OK;
     const bool f64 = is_fp64(L.prec);
     const bool tc = tc_level(L);
+    if (f64 && h.f64_ws) return factor_level_f64_tc(h, li);
     const size_t es = f64 ? 8 : 4;
     // task buffer for this level: one slot per front per launch kind
     GemmTask* d_tasks = nullptr;
@@ -1456,15 +1457,15 @@ int run_factor_level(Handle& h, int li) {
         double pf = 0, pb = 0;
         for (auto& f : L.fronts)
             if (f.s > k) { const double w = std::min(NB, f.s - k); pf += 2.0 * w * w * w / 3.0; pb += (2.0 * w * w + NB * NB) * es; }
-        const int ppi = prof_begin(h, K_POTRF);
         if (f64) {
-            rc = launch_chol_diag_f64(h, li, k, h.stream);
+            rc = launch_chol_diag_f64(h, li, 0, (int)L.fronts.size(), k, h.stream);
             if (rc != RSD_OK) break;
         } else {
+            const int ppi = prof_begin(h, K_POTRF);
             k_potrf_diag_blk<<<(unsigned)L.fronts.size(), 256, POTRF_BLK_SMEM, h.stream>>>(L.d_fronts, k, h.d_err, tc ? 1 : 0, h.d_front_bad);
             count_launch();
+            prof_end(h, ppi, pf, pb);
         }
-        prof_end(h, ppi, pf, pb);
         if (cudaGetLastError() != cudaSuccess) { rc = RSD_ERR_CUDA; break; }
         // (c) panel solve below the diagonal block
         if (tc) {

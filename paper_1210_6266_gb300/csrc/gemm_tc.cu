@@ -30,12 +30,12 @@
 #include <vector>
 
 #include "rsd_internal.cuh"
+#include "tcgen05.cuh"
 
 namespace rsd {
 
 namespace {
 
-constexpr int BM = 128;
 constexpr int BK = 32;                       // FP32 elements per 128-byte swizzle row
 // Operand formats: TF32 (FP32 storage, kind::tf32, 8 K per MMA) or a 16-bit copy (FP16
 // or BF16, kind::f16, 16 K per MMA).  A K block is one 128-byte swizzle row either way:
@@ -49,7 +49,6 @@ constexpr int TC_THREADS = 192;
 // TMEM lane quadrant, each taking 1 / TCP_SPLIT of the tile's columns)
 constexpr int TCP_SPLIT = 2;
 constexpr int TCP_THREADS = 64 + 128 * TCP_SPLIT;
-constexpr long long TC_WAIT_CYCLES = 2000000000LL;   // ~1 s
 constexpr int SPLIT_MIN_KB = 16;             // at least 16 x 32 K per split-K slice
 constexpr int TILE_BAND = 16;                // row blocks per band of a wide output's tile order
 
@@ -87,66 +86,6 @@ __device__ __forceinline__ void prefetch_c_row(const float* crow, int c_lo, int 
     for (int c = c_lo; c < c_hi; c += 32) asm volatile("prefetch.global.L2 [%0];" ::"l"(crow + c));
 }
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-    return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-// Bounded wait; returns false (and raises the error flag) on timeout.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* err) {
-    if (mbar_try(bar, parity)) return true;
-    const long long t0 = clock64();
-    while (!mbar_try(bar, parity)) {
-        if (clock64() - t0 > TC_WAIT_CYCLES || *(volatile int*)&err[ERR_TIMEOUT]) {
-            atomicExch(&err[ERR_TIMEOUT], 1);
-            return false;
-        }
-    }
-    return true;
-}
-
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-        ::"r"(dst), "l"((uint64_t)map), "r"(x), "r"(y), "r"(bar)
-        : "memory");
-}
-
-// Shared-memory matrix descriptor: K-major operand, 128-byte swizzle, 8-row groups 1024 B apart.
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
-    uint64_t d = 0;
-    d |= (uint64_t)((addr & 0x3FFFF) >> 4);          // start address
-    d |= (uint64_t)0 << 16;                           // leading byte offset (unused, swizzled K-major)
-    d |= (uint64_t)(1024 >> 4) << 32;                 // stride byte offset
-    d |= (uint64_t)1 << 46;                           // descriptor version
-    d |= (uint64_t)2 << 61;                           // 128-byte swizzle
-    return d;
-}
-
-// Instruction descriptor: D = F32, A = B of format fmt (TF32 2; F16 0; BF16 1), both
-// K-major, M = 128, N = bn.
-__host__ __device__ constexpr uint32_t idesc_of(uint32_t fmt, int bn) {
-    return (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(bn >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
-}
-__host__ __device__ constexpr uint32_t idesc_tf32(int bn) { return idesc_of(2u, bn); }
-
 __device__ __forceinline__ void mma_tf32(uint32_t tmem, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc) {
     asm volatile(
         "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
@@ -155,22 +94,10 @@ __device__ __forceinline__ void mma_tf32(uint32_t tmem, uint64_t da, uint64_t db
         : "memory");
 }
 
-__device__ __forceinline__ void mma_f16(uint32_t tmem, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc) {
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-        ::"r"(tmem), "l"(da), "l"(db), "r"(idesc), "r"(acc)
-        : "memory");
-}
-
 template <int OP>
 __device__ __forceinline__ void mma_op(uint32_t tmem, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc) {
     if constexpr (OP == TC_OP_TF32) mma_tf32(tmem, da, db, idesc, acc);
     else mma_f16(tmem, da, db, idesc, acc);
-}
-
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {

@@ -222,6 +222,10 @@ struct Handle {
     size_t arena_bytes = 0;
     size_t arena_capacity = 0;          // bytes of the block actually held (cache reuse)
     int device = 0;
+    // digits of FP64 fronts on the tensor cores (gemm_f64_tc.cu), in the arena; null when
+    // the arena only fits without it (those fronts then run on the FP64 pipe)
+    char* f64_ws = nullptr;
+    size_t f64_ws_bytes = 0;
     int* d_err = nullptr;
     int* d_front_bad = nullptr;          // per node: a pivot of its factorisation failed
     int promoted = 0;                    // fronts re-factored one precision up at setup
@@ -353,8 +357,13 @@ int launch_assemble_fronts(Handle& h, int li, const int64_t* rowptr, const int* 
                            const int* tin, const int* tout);
 int launch_extend_add(Handle& h, int li);
 int run_factor_level(Handle& h, int li);
-// FP64 diagonal block factor + inverse at column k of every front of level li (diag_f64.cu)
-int launch_chol_diag_f64(Handle& h, int li, int k, cudaStream_t st);
+// FP64 diagonal block factor + inverse at column k of fronts [f0, f0 + nf) of level li
+// (diag_f64.cu)
+int launch_chol_diag_f64(Handle& h, int li, int f0, int nf, int k, cudaStream_t st);
+// FP64 level on the tensor cores (gemm_f64_tc.cu): workspace for fronts of the given row
+// counts, and the partial Cholesky of the level (needs the handle's f64_ws)
+size_t f64_tc_workspace(const std::vector<int>& rows);
+int factor_level_f64_tc(Handle& h, int li);
 // nonsymmetric fronts: assembly, extend-add and LU partial factorisation of level li
 int launch_assemble_fronts_lu(Handle& h, int li, const int64_t* rowptr, const int* col, const double* val,
                               const int* owner, const int* rank, const int* tin, const int* tout);

@@ -132,3 +132,24 @@ def test_fp64_fronts_of_a_badly_scaled_matrix(rsd):
     got = h.front_factor(1)[:300] / scale[:300, None]
     assert (np.abs(got - L) / np.sqrt(np.diag(B)[:300])[:, None]).max() <= 40 * 301 * 2.2e-16
     h.close()
+
+
+def test_fp64_fronts_in_several_groups_match_one_at_a_time(rsd):
+    """Enough leaf rows that the digit workspace holds only part of the level's fronts at
+    once (over 10 GB for all): the same applications as each problem alone."""
+    n, count = 33, 32
+    kinds = [rsd.grid_problem(n, 1, np.exp(synth.normal(500 + q, (n - 1) ** 3)), synth.uniform(600 + q, (n - 2) ** 3))
+             for q in range(2)]
+    p = rsd.RSD_PREC_FP64
+    ref = []
+    for k in kinds:
+        h = rsd.RSD.setup(k["rowptr"], k["col"], k["val"], k["dof_node"], k["parent"], prec_leaf=p, prec_mid=p, prec_root=p)
+        ref.append(h.apply(k["b"]))
+        h.close()
+    probs = [kinds[(q // 3) % 2] for q in range(count)]
+    h = rsd.RSD.setup_batched(probs, prec_leaf=p, prec_mid=p, prec_root=p)
+    z = h.apply(torch.cat([q["b"] for q in probs])).reshape(count, -1)
+    h.close()
+    for q in range(count):
+        r = ref[(q // 3) % 2]
+        assert float((z[q] - r).abs().max()) <= 1e-13 * float(r.abs().max()), q
