@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(DT, 1) k_chol_diag_f64(const FrontDesc* __rest
         const int r = e / SBK, c = e % SBK;
         D[r * SLD + c] = c <= r ? (r < w ? P[(int64_t)r * f.ldp + c] : (r == c ? 1.0 : 0.0)) : 0.0;
     }
-    __syncthreads();
+    cluster_or_cta_sync<CL>();                   // every CTA has read the block before one writes L over it
     int bad = 0;
     for (int J = 0; J < nJ; ++J) {
         const int o = SBK * J, below = SBK * (J + 1), rows = nJ * SBK;
