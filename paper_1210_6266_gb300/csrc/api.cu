@@ -1040,13 +1040,12 @@ static int build_handle(Handle& h, Analysis& a, const int64_t* rowptr, const int
     // (levels are factored one after another and share it); without room for it the FP64
     // levels run on the FP64 pipe as before
     size_t f64_ws = 0;
-    if (!h.lu)
-        for (int d = 0; d < nl; ++d) {
-            if (!is_fp64(h.levels[d].prec) || !h.levels[d].factored) continue;
-            std::vector<int> rows;
-            for (int t : h.levels[d].nodes) rows.push_back(a.I_off[t + 1] - a.I_off[t] + beff(t));
-            f64_ws = std::max(f64_ws, f64_tc_workspace(rows));
-        }
+    for (int d = 0; d < nl; ++d) {
+        if (!is_fp64(h.levels[d].prec) || !h.levels[d].factored) continue;
+        std::vector<int> rows;
+        for (int t : h.levels[d].nodes) rows.push_back(a.I_off[t + 1] - a.I_off[t] + beff(t));
+        f64_ws = std::max(f64_ws, f64_tc_workspace(rows, h.lu));
+    }
     const size_t o_f64 = off;
     h.arena_bytes = off + f64_ws;
     {

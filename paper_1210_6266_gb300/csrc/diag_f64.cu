@@ -1,4 +1,4 @@
-// FP64 diagonal block of the partial Cholesky (step (b) of factor.cu): L_kk L_kk^T =
+// FP64 diagonal blocks.  Partial Cholesky (step (b) of factor.cu): L_kk L_kk^T =
 // P[k:k+w, k:k+w] (w <= NB) written back, L_kk^-1 to Dinv.
 //
 // The FP64 pipe bounds it: an SM retires 1.65 FP64 FMAs per clock and a warp's FMA takes
@@ -239,21 +239,228 @@ __global__ void __launch_bounds__(DT, 1) k_chol_diag_f64(const FrontDesc* __rest
     }
 }
 
+// ---- nonsymmetric fronts ---------------------------------------------------------------
+// LU without pivoting of the block (lower part from P, upper part from PU transposed), the
+// same division of work: L (unit) to P, U^T to PU, L^-1 to Dinv, (U^T)^-1 to DinvU.  A row of
+// the next diagonal sub-block goes to every CTA with all its columns, the block row of U
+// is formed by columns (CTA q those congruent to q mod CL).  The two inverses double the
+// FP64 work; they live in Dinv and DinvU themselves (each CTA reads back only the columns it
+// wrote).  Measured on a 37^3 convection-diffusion system: 0.80 ms a launch before (one CTA,
+// three barriers a column, one thread a column of the inverses), 0.24 ms.
+
+// LU and the inverses of L and U^T of the 32 x 32 block at A (row stride LD), all eight warps,
+// thread (lane, warp) holding row `lane` of columns warp + 8 q; A keeps L and U, YL = L^-1, YW =
+// (U^T)^-1 (lower, zeros above).  Returns 1 on a pivot that is zero or not finite (replaced by 1).
+__device__ int lu_inv32(double* __restrict__ A, double* __restrict__ YL, double* __restrict__ YW, double* __restrict__ col,
+                        double* __restrict__ rowu, double* __restrict__ dinv, int lane, int warp) {
+    double a[4], yl[4], yw[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int c = warp + DW * q;
+        a[q] = A[lane * LD + c];
+        yl[q] = yw[q] = c == lane ? 1.0 : 0.0;
+    }
+    int bad = 0;
+#pragma unroll
+    for (int jb = 0; jb < 4; ++jb) {
+#pragma unroll 1
+        for (int jj = 0; jj < DW; ++jj) {
+            const int j = DW * jb + jj;
+            double* cj = col + (j & 1) * SBK;
+            double* rj = rowu + (j & 1) * SBK;
+            if (warp == jj) {
+                double d = __shfl_sync(0xffffffffu, a[jb], j);
+                if (!(d != 0.0) || !(fabs(d) <= 1.7976931348623157e308)) {
+                    bad = 1;
+                    d = 1.0;
+                    if (lane == j) a[jb] = 1.0;
+                }
+                const double inv = 1.0 / d;
+                if (lane > j) a[jb] *= inv;
+                cj[lane] = lane > j ? a[jb] : 0.0;
+                if (lane == 0) dinv[j & 1] = inv;
+            }
+            if (lane == j) {
+#pragma unroll
+                for (int q = jb; q < 4; ++q) rj[warp + DW * q] = a[q];
+            }
+            __syncthreads();
+            const double li = cj[lane];
+#pragma unroll
+            for (int q = jb; q < 4; ++q)
+                if (warp + DW * q > j) a[q] -= li * rj[warp + DW * q];
+            const double inv = dinv[j & 1], ui = lane > j ? rj[lane] : 0.0;
+#pragma unroll
+            for (int q = 0; q <= jb; ++q) {
+                if (warp + DW * q > j) continue;
+                const double xl = __shfl_sync(0xffffffffu, yl[q], j);
+                const double xw = __shfl_sync(0xffffffffu, yw[q], j) * inv;
+                yl[q] = lane > j ? yl[q] - li * xl : yl[q];
+                yw[q] = lane == j ? xw : (lane > j ? yw[q] - ui * xw : yw[q]);
+            }
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int c = warp + DW * q;
+        A[lane * LD + c] = a[q];
+        YL[lane * SLD + c] = c <= lane ? yl[q] : 0.0;
+        YW[lane * SLD + c] = c <= lane ? yw[q] : 0.0;
+    }
+    __syncthreads();
+    return bad;
+}
+
+constexpr size_t LU_SMEM = sizeof(double) * ((size_t)NB * LD + 2 * SBK * SLD + 4 * SBK + 2);
+
 template <int CL>
-int launch_cl(const FrontDesc* d_fronts, int nf, int k, int* err, int* bad_front, cudaStream_t st) {
-    RSD_CUDA_TRY(cudaFuncSetAttribute(k_chol_diag_f64<CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DIAG_SMEM));
+__global__ void __launch_bounds__(DT, 1) k_lu_diag_f64(const FrontDesc* __restrict__ fronts, int k, int* __restrict__ err,
+                                                     int* __restrict__ bad_front) {
+    extern __shared__ __align__(16) unsigned char diag_smem[];
+    double* A = (double*)diag_smem;              // NB x LD: L below the diagonal, U on and above it
+    double* YL = A + NB * LD;                    // 32 x SLD: L_JJ^-1
+    double* YW = YL + SBK * SLD;                 // 32 x SLD: (U_JJ^T)^-1
+    double* col = YW + SBK * SLD;
+    double* rowu = col + 2 * SBK;
+    double* dinv = rowu + 2 * SBK;
+    const FrontDesc f = fronts[blockIdx.x / CL];
+    if (f.s <= k) return;                        // the whole cluster
+    const int w = min(NB, f.s - k), nJ = (w + SBK - 1) / SBK, rows = nJ * SBK;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int rank = CL > 1 ? (int)cl_rank() : 0;
+    double* P = (double*)f.P + (int64_t)k * f.ldp + k;
+    double* PU = (double*)f.PU + (int64_t)k * f.ldp + k;
+    double* Dg = (double*)f.Dinv + (int64_t)(k / NB) * NB * NB;
+    double* DUg = (double*)f.DinvU + (int64_t)(k / NB) * NB * NB;
+    // this CTA's rows and the first block row; identity past the front
+    for (int r = warp; r < rows; r += DW) {
+        if (r >= SBK && r % CL != rank) continue;
+        for (int c = lane; c < rows; c += 32)
+            A[r * LD + c] = (r < w && c < w) ? (c <= r ? P[(int64_t)r * f.ldp + c] : PU[(int64_t)c * f.ldp + r]) : (r == c ? 1.0 : 0.0);
+    }
+    cluster_or_cta_sync<CL>();                   // read everywhere before L and U are written over it
+    int bad = 0;
+    for (int J = 0; J < nJ; ++J) {
+        const int o = SBK * J, below = SBK * (J + 1);
+        if (J > 0) cluster_or_cta_sync<CL>();          // the block row is here
+        bad |= lu_inv32(A + o * LD + o, YL, YW, col, rowu, dinv, lane, warp);
+        for (int e = tid; e < SBK * SBK; e += DT) {
+            const int c = e % SBK, r = e / SBK;
+            if (((o + c) >> 2) % CL == rank) {
+                Dg[(o + r) * NB + o + c] = YL[r * SLD + c];
+                DUg[(o + r) * NB + o + c] = YW[r * SLD + c];
+            }
+        }
+        // own rows below: L_rc = sum_m A_rm W_cm; own columns to the right: U_ic = sum_m X_im A_mc
+        constexpr int UP = (96 / CL + DW - 1) / DW;
+        const int first = below + ((rank - below) % CL + CL) % CL;        // first own row or column >= below
+        double pl[UP], pu[UP];
+#pragma unroll
+        for (int u = 0; u < UP; ++u) {
+            const int r = first + CL * (warp + DW * u);
+            double s = 0.0, t = 0.0;
+            if (r < rows)
+#pragma unroll 8
+                for (int m = 0; m < SBK; ++m) {
+                    s += A[r * LD + o + m] * YW[lane * SLD + m];
+                    t += A[(o + m) * LD + r] * YL[lane * SLD + m];
+                }
+            pl[u] = s;
+            pu[u] = t;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < UP; ++u) {
+            const int r = first + CL * (warp + DW * u);
+            if (r >= rows) continue;
+            double* dl = A + r * LD + o + lane;
+            double* du = A + (o + lane) * LD + r;
+            *dl = pl[u];
+            *du = pu[u];
+            if constexpr (CL > 1)
+                for (int q = 1; q < CL; ++q) {
+                    cl_st_f64(cl_map(dl, (uint32_t)((rank + q) % CL)), pl[u]);
+                    cl_st_f64(cl_map(du, (uint32_t)((rank + q) % CL)), pu[u]);
+                }
+        }
+        if (J + 1 < nJ) {
+            cluster_or_cta_sync<CL>();                 // panel and block row are complete in every CTA
+            int it = 0;
+            for (int r = first; r < rows; r += CL)
+                for (int cb = J + 1; cb < nJ; ++cb, ++it) {
+                    if (it % DW != warp) continue;
+                    const int c = cb * SBK + lane;
+                    double s = 0.0;
+#pragma unroll 8
+                    for (int m = 0; m < SBK; ++m) s += A[r * LD + o + m] * A[(o + m) * LD + c];
+                    double* dst = A + r * LD + c;
+                    const double v = *dst - s;
+                    *dst = v;
+                    if constexpr (CL > 1)
+                        if (r < below + SBK)
+                            for (int q = 1; q < CL; ++q) cl_st_f64(cl_map(dst, (uint32_t)((rank + q) % CL)), v);
+                }
+        } else {
+            __syncthreads();
+        }
+        // block row J of both inverses, this CTA's columns: a warp takes a column, lane = row
+        int ic = 0;
+        for (int c0 = 4 * rank; c0 < o; c0 += 4 * CL)
+            for (int cc = 0; cc < 4; ++cc, ++ic) {
+                if (ic % DW != warp) continue;
+                const int c = c0 + cc, m0 = c & ~(SBK - 1);
+                double tl = 0.0, tw = 0.0;
+#pragma unroll 4
+                for (int m = m0; m < o; ++m) {
+                    tl += A[(o + lane) * LD + m] * Dg[m * NB + c];
+                    tw += A[m * LD + o + lane] * DUg[m * NB + c];
+                }
+                double xl = 0.0, xw = 0.0;
+#pragma unroll 8
+                for (int m = 0; m < SBK; ++m) {
+                    xl -= YL[lane * SLD + m] * __shfl_sync(0xffffffffu, tl, m);
+                    xw -= YW[lane * SLD + m] * __shfl_sync(0xffffffffu, tw, m);
+                }
+                Dg[(o + lane) * NB + c] = xl;
+                DUg[(o + lane) * NB + c] = xw;
+            }
+    }
+    __syncthreads();
+    // L (unit) and U^T, this CTA's rows; the inverses' zeros above the diagonal and past the front
+    for (int r = rank + CL * warp; r < w; r += CL * DW)
+        for (int c = lane; c <= r; c += 32) {
+            P[(int64_t)r * f.ldp + c] = c < r ? A[r * LD + c] : 1.0;
+            PU[(int64_t)r * f.ldp + c] = A[c * LD + r];
+        }
+    for (int e = tid; e < NB * (NB / CL); e += DT) {
+        const int r = e / (NB / CL), q = e % (NB / CL);
+        const int c = (q >> 2) * 4 * CL + 4 * rank + (q & 3);
+        if (r < c || r >= w || c >= w) Dg[r * NB + c] = DUg[r * NB + c] = 0.0;
+    }
+    if (bad && rank == 0 && lane == 0) {
+        atomicExch(&err[ERR_NOT_SPD], 1);
+        atomicMin(&err[ERR_NOT_SPD_NODE], f.node);
+        bad_front[f.node] = 1;
+    }
+}
+
+using DiagKernel = void (*)(const FrontDesc*, int, int*, int*);
+
+int launch_cl(DiagKernel kern, int CL, size_t smem, const FrontDesc* d_fronts, int nf, int k, int* err, int* bad_front, cudaStream_t st) {
+    RSD_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(nf * CL));
     cfg.blockDim = dim3(DT);
-    cfg.dynamicSmemBytes = DIAG_SMEM;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = CL;
+    at[0].val.clusterDim.x = (unsigned)CL;
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    RSD_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_chol_diag_f64<CL>, d_fronts, k, err, bad_front));
+    RSD_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, d_fronts, k, err, bad_front));
     count_launch();
     return RSD_OK;
 }
@@ -263,7 +470,7 @@ int launch_cl(const FrontDesc* d_fronts, int nf, int k, int* err, int* bad_front
 // The largest cluster that still gives every front with rows past k SMs of its own: the
 // FP64 pipes it adds are worth more than anything else to a lone block (see above), and
 // past one wave a larger cluster only queues.
-int launch_chol_diag_f64(Handle& h, int li, int f0, int nf, int k, cudaStream_t st) {
+int launch_diag_f64(Handle& h, int li, int f0, int nf, int k, cudaStream_t st) {
     Level& L = h.levels[li];
     int alive = 0;
     double flops = 0, bytes = 0;
@@ -271,17 +478,16 @@ int launch_chol_diag_f64(Handle& h, int li, int f0, int nf, int k, cudaStream_t 
         if (L.fronts[q].s <= k) continue;
         const double w = std::min(NB, L.fronts[q].s - k);
         ++alive;
-        flops += 2.0 * w * w * w / 3.0;
-        bytes += (2.0 * w * w + NB * NB) * 8;
+        flops += (h.lu ? 4.0 : 2.0) * w * w * w / 3.0;
+        bytes += (2.0 * w * w + NB * NB) * (h.lu ? 16 : 8);
     }
     if (!alive) return RSD_OK;
     const FrontDesc* fr = L.d_fronts + f0;
     const int pi = prof_begin(h, K_POTRF, st);
-    int rc;
-    if (alive * 8 <= h.num_sms) rc = launch_cl<8>(fr, nf, k, h.d_err, h.d_front_bad, st);
-    else if (alive * 4 <= h.num_sms) rc = launch_cl<4>(fr, nf, k, h.d_err, h.d_front_bad, st);
-    else if (alive * 2 <= h.num_sms) rc = launch_cl<2>(fr, nf, k, h.d_err, h.d_front_bad, st);
-    else rc = launch_cl<1>(fr, nf, k, h.d_err, h.d_front_bad, st);
+    static constexpr DiagKernel chol[4] = {k_chol_diag_f64<1>, k_chol_diag_f64<2>, k_chol_diag_f64<4>, k_chol_diag_f64<8>};
+    static constexpr DiagKernel lu[4] = {k_lu_diag_f64<1>, k_lu_diag_f64<2>, k_lu_diag_f64<4>, k_lu_diag_f64<8>};
+    const int lg = alive * 8 <= h.num_sms ? 3 : alive * 4 <= h.num_sms ? 2 : alive * 2 <= h.num_sms ? 1 : 0;
+    const int rc = launch_cl((h.lu ? lu : chol)[lg], 1 << lg, h.lu ? LU_SMEM : DIAG_SMEM, fr, nf, k, h.d_err, h.d_front_bad, st);
     prof_end(h, pi, flops, bytes, st);
     return rc;
 }

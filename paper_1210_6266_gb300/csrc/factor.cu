@@ -1458,7 +1458,7 @@ int run_factor_level(Handle& h, int li) {
         for (auto& f : L.fronts)
             if (f.s > k) { const double w = std::min(NB, f.s - k); pf += 2.0 * w * w * w / 3.0; pb += (2.0 * w * w + NB * NB) * es; }
         if (f64) {
-            rc = launch_chol_diag_f64(h, li, 0, (int)L.fronts.size(), k, h.stream);
+            rc = launch_diag_f64(h, li, 0, (int)L.fronts.size(), k, h.stream);
             if (rc != RSD_OK) break;
         } else {
             const int ppi = prof_begin(h, K_POTRF);

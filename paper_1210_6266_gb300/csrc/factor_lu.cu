@@ -13,7 +13,8 @@
 // Before factorisation F is spread over P (entries on or below the diagonal of F_II, and
 // F_BI) and PU (entries above it, transposed, and F_IB transposed).
 //
-// Left-looking by NB-column blocks k (CUDA cores, FP64 or FP32):
+// FP64 levels run in gemm_f64_tc.cu (and diag_f64.cu) unless the arena had no room for its
+// workspace.  Here, left-looking by NB-column blocks k (CUDA cores, FP32 or FP64):
 //   (a) P[k:N, blk]    -= P[k:N, 0:k]    PU[blk, 0:k]^T   (L and X columns, with the
 //                                                          diagonal block's lower part)
 //   (b) PU[k:N, blk]   -= PU[k:N, 0:k]   P[blk, 0:k]^T    (U^T and Y^T columns, with the
@@ -233,6 +234,7 @@ int run_factor_level_lu(Handle& h, int li) {
     Level& L = h.levels[li];
     if (L.fronts.empty()) return RSD_OK;
     const bool f64 = is_fp64(L.prec);
+    if (f64 && h.f64_ws) return factor_level_f64_tc(h, li);
     const size_t es = f64 ? 8 : 4;
     const size_t smem = (size_t)NB * (NB + 1) * es;
     if (f64) RSD_CUDA_TRY(cudaFuncSetAttribute(k_getrf_diag<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));

@@ -1,5 +1,5 @@
 // FP64 fronts on the tensor cores: every product of the blocked partial Cholesky (the
-// updates C -= X X^T, the panel solve X = A L_kk^-T) split into exact FP16 products
+// updates C -= X X^T, the panel solve X = A L_kk^-T) or LU (C -= X Y) split into exact FP16 products
 // (Ozaki, Ogita, Oishi, Rump, "Error-free transformations of matrix multiplication by
 // using fast routines of matrix multiplication", 2012).
 //
@@ -71,7 +71,7 @@ constexpr int F64_SMEM = 2 * GROUP + A_ST * A_BYTES + 1024 + 256;
 struct F64Task {
     const char *A, *B;
     const int *ea, *eb;                      // exponents by row of A and of B
-    const int* sq;                           // per row: sum of digit 4 squared (updates)
+    const int* sq;                           // per row: sum of digit 4 squared (C -= X X^T; else null)
     double *P, *U;                           // C: columns below s in P, the rest in U
     int a_nrt, b_nrt;                        // row tiles per K block
     int ldp, ldu, s;
@@ -82,8 +82,9 @@ struct F64Task {
     int tile_begin;
 };
 
-struct F64Front {                            // workspace of one front
-    char *XS, *AS, *DS;                      // digits: the panel's X, the block column's A, Dinv
+// Workspace of one front's panel [L; X] (of [U^T; Y^T] too, for a nonsymmetric front)
+struct F64Front {
+    char *XS, *AS, *DS;                      // digits: the panel's X, the block column's A, Dinv_k
     int *ex, *aex, *dex;                     // row exponents of X, A and Dinv_k
     int* sq;                                 // per row of X: sum of digit 4 squared
     float* n2;                               // per row of X: sum of (x 2^-ex)^2
@@ -240,6 +241,7 @@ __device__ __forceinline__ int store_digits(const double (&x)[8], const int (&e)
 // Operands of the panel solve at block column k: A_ij 2^-s_j (rows below the diagonal
 // block) and Dinv_cj 2^s_j, s_j the exponent of L_jj (a row's entries then compare across
 // columns of different scale).  blockIdx.x < na: SA_ROWS rows of A, else of Dinv.
+// Nonsymmetric fronts, blockIdx.z = 0: P against (U_kk^T)^-1, s_j of U_jj; 1: PU against L_kk^-1.
 constexpr int SA_ROWS = 64;
 __global__ void __launch_bounds__(256) k_split_a(const FrontDesc* __restrict__ fronts, const F64Front* __restrict__ wk, int k,
                                                 int na, int* __restrict__ err, int* __restrict__ bad_front) {
@@ -250,15 +252,18 @@ __global__ void __launch_bounds__(256) k_split_a(const FrontDesc* __restrict__ f
     const bool isA = (int)blockIdx.x < na;
     const int r0 = isA ? k + w + (int)blockIdx.x * SA_ROWS : ((int)blockIdx.x - na) * SA_ROWS;
     if (isA && r0 >= f.N) return;
-    const F64Front wf = wk[blockIdx.y];
-    const double* P = (const double*)f.P;
+    const F64Front wf = wk[gridDim.z * blockIdx.y + blockIdx.z];
+    const bool lu = gridDim.z == 2, upper = blockIdx.z == 1;
+    const double* P = (const double*)(upper ? f.PU : f.P);
+    const double* diag = (const double*)(lu && !upper ? f.PU : f.P);
+    const double* Dk = (const double*)(lu && !upper ? f.DinvU : f.Dinv) + (int64_t)(k / NB) * NB * NB;
     int ok = 1;
-    if (threadIdx.x < NB) sj[threadIdx.x] = (int)threadIdx.x < w ? exp_above(P[(int64_t)(k + threadIdx.x) * f.ldp + k + threadIdx.x], &ok) : 0;
+    if (threadIdx.x < NB) sj[threadIdx.x] = (int)threadIdx.x < w ? exp_above(diag[(int64_t)(k + threadIdx.x) * f.ldp + k + threadIdx.x], &ok) : 0;
     __syncthreads();
 #pragma unroll 1
     for (int r = r0 + (threadIdx.x >> 4); r < r0 + SA_ROWS; r += 16) {
         const bool in = isA ? r < f.N : r < w;
-        const double* src = (isA ? P + (int64_t)r * f.ldp + k : (const double*)f.Dinv + (int64_t)(k / NB) * NB * NB + r * NB) + j0;
+        const double* src = (isA ? P + (int64_t)r * f.ldp + k : Dk + r * NB) + j0;
         int top = E_NONE, e[8];
         double x[8];
 #pragma unroll
@@ -287,12 +292,12 @@ __global__ void __launch_bounds__(256) k_split_x(const FrontDesc* __restrict__ f
                                                 int K0, int* __restrict__ err, int* __restrict__ bad_front) {
     const FrontDesc f = fronts[blockIdx.y];
     if (f.s <= k) return;
-    const F64Front wf = wk[blockIdx.y];
+    const F64Front wf = wk[gridDim.z * blockIdx.y + blockIdx.z];
     const int w = min(NB, f.s - k), ch = threadIdx.x & 15, j0 = ch * 8;
     if (k + w + (int)blockIdx.x * 16 >= f.N) return;
     const int r = k + w + (int)blockIdx.x * 16 + (threadIdx.x >> 4);
     const bool in = r < f.N;
-    const double* src = (const double*)f.P + (int64_t)r * f.ldp + j0;
+    const double* src = (const double*)(blockIdx.z ? f.PU : f.P) + (int64_t)r * f.ldp + j0;
     int ok = 1, top = E_NONE;
     double x[8];
 #pragma unroll
@@ -514,7 +519,7 @@ k_gemm_f64_tc(const F64Task* __restrict__ tasks, int ntask, int n_tiles, int* __
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(acc_empty) : "memory");
             if (!in) continue;
-            if (!SOLVE && t.lower && gr >= c_base && gr < c_base + CW) {       // C's diagonal
+            if (!SOLVE && t.sq && gr >= c_base && gr < c_base + CW) {       // C's diagonal
                 const uint32_t add = (uint32_t)(t.sq[gr] + 64) >> 7;
 #pragma unroll
                 for (int c = 0; c < CW; ++c)
@@ -582,45 +587,49 @@ int64_t tiles_of(const F64Task& t) {
 // Workspace of a level: the digits of one 512-wide panel of every front at once where that
 // fits the cap (groups of fronts then take turns), of one front at least.  The cap is far
 // above what fills the chip: 4 GiB hold over 100 fronts of 4000 rows, thousands of tiles.
-size_t f64_tc_workspace(const std::vector<int>& rows) {
+size_t f64_tc_workspace(const std::vector<int>& rows, bool lu) {
     const size_t cap = (size_t)4 << 30;
     size_t sum = 0, most = 0;
-    for (int N : rows) { sum += front_bytes(N); most = std::max(most, front_bytes(N)); }
+    for (int N : rows) { sum += (lu ? 2 : 1) * front_bytes(N); most = std::max(most, (lu ? 2 : 1) * front_bytes(N)); }
     return std::min(sum, std::max(cap, most));
 }
 
-// Partial Cholesky of every FP64 front of level li (all steps of factor.cu), 512-wide
-// panels: per 128-wide block column the update by the panel's earlier columns, the
-// diagonal block, the split and the solve of the rows below; per panel the update of
-// everything right of it (P and U), K = the panel's width.
+// Partial Cholesky (all steps of factor.cu) or LU (of factor_lu.cu) of every FP64 front of
+// level li, 512-wide panels: per 128-wide block column the update by the panel's earlier
+// columns, the diagonal block, the split and the solve of the rows below; per panel the
+// update of everything right of it (P and U; PU), K = the panel's width.  Nonsymmetric
+// fronts run every step on [L; X] and [U^T; Y^T] (side 0 and 1) in one launch:
+// P -= P PU^T, PU -= PU P^T, U -= X Y.
 int factor_level_f64_tc(Handle& h, int li) {
     Level& L = h.levels[li];
     cudaStream_t st = h.stream;
-    const int nf_all = (int)L.fronts.size();
+    const int nf_all = (int)L.fronts.size(), sides = h.lu ? 2 : 1;
     struct Launch { size_t off; int n, tiles, solve; double flops, bytes; };
     struct Group { int f0, nf, max_s; };
     std::vector<Group> groups;
-    std::vector<F64Front> wk(nf_all);
+    std::vector<F64Front> wk((size_t)nf_all * sides);
     for (int f0 = 0; f0 < nf_all;) {
         Group g{f0, 0, 0};
         size_t off = 0;
         while (f0 + g.nf < nf_all) {
             const FrontDesc& f = L.fronts[f0 + g.nf];
             const size_t need = front_bytes(f.N);
-            if (g.nf && off + need > h.f64_ws_bytes) break;
-            if (need > h.f64_ws_bytes) return RSD_ERR_ARG;
-            F64Front& w = wk[f0 + g.nf];
-            char* p = h.f64_ws + off;
-            w.nrt = row_tiles(f.N);
-            w.XS = p; p += (size_t)(WP / KB) * w.nrt * GROUP;
-            w.AS = p; p += (size_t)2 * w.nrt * GROUP;
-            w.DS = p; p += (size_t)4 * GROUP;
-            w.ex = (int*)p; p += al(sizeof(int) * (size_t)f.N);
-            w.sq = (int*)p; p += al(sizeof(int) * (size_t)f.N);
-            w.n2 = (float*)p; p += al(sizeof(float) * (size_t)f.N);
-            w.aex = (int*)p; p += al(sizeof(int) * (size_t)f.N);
-            w.dex = (int*)p;
-            off += need;
+            if (g.nf && off + sides * need > h.f64_ws_bytes) break;
+            if (sides * need > h.f64_ws_bytes) return RSD_ERR_ARG;
+            for (int sd = 0; sd < sides; ++sd) {
+                F64Front& w = wk[(size_t)(f0 + g.nf) * sides + sd];
+                char* p = h.f64_ws + off;
+                w.nrt = row_tiles(f.N);
+                w.XS = p; p += (size_t)(WP / KB) * w.nrt * GROUP;
+                w.AS = p; p += (size_t)2 * w.nrt * GROUP;
+                w.DS = p; p += (size_t)4 * GROUP;
+                w.ex = (int*)p; p += al(sizeof(int) * (size_t)f.N);
+                w.sq = (int*)p; p += al(sizeof(int) * (size_t)f.N);
+                w.n2 = (float*)p; p += al(sizeof(float) * (size_t)f.N);
+                w.aex = (int*)p; p += al(sizeof(int) * (size_t)f.N);
+                w.dex = (int*)p;
+                off += need;
+            }
             g.max_s = std::max(g.max_s, f.s);
             ++g.nf;
         }
@@ -636,8 +645,8 @@ int factor_level_f64_tc(Handle& h, int li) {
         t.tile_begin = l.tiles;
         l.tiles += (int)tiles_of(t);
         ++l.n;
-        const double m = t.r_hi - t.r_lo, c = t.lower ? (t.c_hi > t.r_lo ? 0.5 * m * (m + 1) - 0.5 * std::max(0, t.r_hi - t.c_hi) * (t.r_hi - t.c_hi + 1.0) : 0)
-                                                       : m * (t.c_hi - t.c_lo);
+        const double m = t.r_hi - t.r_lo, n = t.c_hi - t.c_lo;
+        const double c = t.lower ? m * n - 0.5 * n * (n - 1) : m * n;
         l.flops += 2.0 * c * t.nkb * KB;
         l.bytes += 16.0 * c + 16.0 * m * t.nkb * KB;
         tasks.push_back(t);
@@ -645,70 +654,75 @@ int factor_level_f64_tc(Handle& h, int li) {
     for (const Group& g : groups) {
         for (int k = 0; k < g.max_s; k += NB) {
             const int K0 = k / WP * WP;
-            auto base = [&](int q) {
+            // rows [r0, N) and columns [c0, c1) of front q (side sd): C -= X X^T, X Y^T or Y X^T
+            auto update = [&](int q, int sd, int r0, int c0, int c1, int nkb, bool lower) {
                 const FrontDesc& f = L.fronts[g.f0 + q];
-                const F64Front& w = wk[g.f0 + q];
+                const F64Front& a = wk[(size_t)(g.f0 + q) * sides + sd];
+                const F64Front& b = wk[(size_t)(g.f0 + q) * sides + (sides - 1 - sd)];
                 F64Task t{};
-                t.A = t.B = w.XS;
-                t.a_nrt = t.b_nrt = w.nrt;
-                t.ea = t.eb = w.ex;
-                t.sq = w.sq;
-                t.P = (double*)f.P; t.U = (double*)f.U;
+                t.A = a.XS; t.B = b.XS;
+                t.a_nrt = t.b_nrt = a.nrt;
+                t.ea = a.ex; t.eb = b.ex;
+                t.sq = sides == 1 ? a.sq : nullptr;
+                t.P = (double*)(sd ? f.PU : f.P); t.U = (double*)f.U;
                 t.ldp = f.ldp; t.ldu = f.ldu; t.s = f.s;
-                t.r_hi = f.N;
-                t.lower = 1;
-                return t;
+                t.r_lo = r0; t.r_hi = f.N; t.c_lo = c0; t.c_hi = c1;
+                t.tm0 = r0 / BM; t.ntm = (f.N + BM - 1) / BM - t.tm0;
+                t.tn0 = c0 / TN; t.ntn = (c1 + TN - 1) / TN - t.tn0;
+                t.nkb = nkb;
+                t.lower = lower;
+                add(t);
             };
             if (k > K0) {                                  // the block column from the panel's earlier ones
                 begin(0);
                 for (int q = 0; q < g.nf; ++q) {
                     const FrontDesc& f = L.fronts[g.f0 + q];
                     if (f.s <= k) continue;
-                    F64Task t = base(q);
-                    t.r_lo = t.c_lo = k; t.c_hi = std::min(k + NB, f.s);
-                    t.tm0 = k / BM; t.ntm = (f.N + BM - 1) / BM - t.tm0;
-                    t.tn0 = k / TN; t.ntn = (t.c_hi - k + TN - 1) / TN;
-                    t.nkb = (k - K0) / KB;
+                    for (int sd = 0; sd < sides; ++sd) update(q, sd, k, k, std::min(k + NB, f.s), (k - K0) / KB, true);
+                }
+            }
+            begin(1);                                      // the rows below the diagonal block
+            for (int q = 0; q < g.nf; ++q) {
+                const FrontDesc& f = L.fronts[g.f0 + q];
+                const int wd = std::min(NB, f.s - k);
+                if (f.s <= k || f.N <= k + wd) continue;
+                for (int sd = 0; sd < sides; ++sd) {
+                    const F64Front& w = wk[(size_t)(g.f0 + q) * sides + sd];
+                    F64Task t{};
+                    t.A = w.AS; t.B = w.DS;
+                    t.a_nrt = w.nrt; t.b_nrt = 2;
+                    t.ea = w.aex; t.eb = w.dex;
+                    t.P = (double*)(sd ? f.PU : f.P); t.U = (double*)f.U;
+                    t.ldp = f.ldp; t.ldu = f.ldu; t.s = f.s;
+                    t.r_lo = k + wd; t.r_hi = f.N; t.c_lo = k; t.c_hi = k + wd;
+                    t.tm0 = t.r_lo / BM; t.ntm = (f.N + BM - 1) / BM - t.tm0;
+                    t.tn0 = k / TN; t.ntn = (wd + TN - 1) / TN;
+                    t.b_rt0 = k / TN;
+                    t.nkb = (wd + KB - 1) / KB;
                     add(t);
                 }
             }
-            begin(1);                                // the rows below the diagonal block
-            for (int q = 0; q < g.nf; ++q) {
-                const FrontDesc& f = L.fronts[g.f0 + q];
-                const F64Front& w = wk[g.f0 + q];
-                const int wd = std::min(NB, f.s - k);
-                if (f.s <= k || f.N <= k + wd) continue;
-                F64Task t = base(q);
-                t.A = w.AS; t.B = w.DS; t.b_nrt = 2;
-                t.ea = w.aex; t.eb = w.dex;
-                t.r_lo = k + wd; t.c_lo = k; t.c_hi = k + wd;
-                t.tm0 = t.r_lo / BM; t.ntm = (f.N + BM - 1) / BM - t.tm0;
-                t.tn0 = k / TN; t.ntn = (wd + TN - 1) / TN;
-                t.b_rt0 = k / TN;
-                t.nkb = (wd + KB - 1) / KB;
-                t.lower = 0;
-                add(t);
-            }
             if (k + NB < std::min(K0 + WP, g.max_s)) continue;
-            begin(0);                                // everything right of the panel
+            begin(0);                                      // everything right of the panel
             for (int q = 0; q < g.nf; ++q) {
                 const FrontDesc& f = L.fronts[g.f0 + q];
-                const int c0 = std::min(K0 + WP, f.s);
+                const int c0 = std::min(K0 + WP, f.s), nkb = (c0 - K0 + KB - 1) / KB;
                 if (f.s <= K0 || f.N <= c0) continue;
-                F64Task t = base(q);
-                t.r_lo = t.c_lo = c0; t.c_hi = f.N;
-                t.tm0 = c0 / BM; t.ntm = (f.N + BM - 1) / BM - t.tm0;
-                t.tn0 = c0 / TN; t.ntn = (f.N + TN - 1) / TN - t.tn0;
-                t.nkb = (c0 - K0 + KB - 1) / KB;
-                add(t);
+                if (sides == 1) {
+                    update(q, 0, c0, c0, f.N, nkb, true);
+                    continue;
+                }
+                if (f.s > c0)
+                    for (int sd = 0; sd < 2; ++sd) update(q, sd, c0, c0, f.s, nkb, true);
+                if (f.b) update(q, 0, f.s, f.s, f.N, nkb, false);
             }
         }
     }
-    const size_t o_tasks = al(sizeof(F64Front) * (size_t)nf_all), total = o_tasks + sizeof(F64Task) * tasks.size();
+    const size_t o_tasks = al(sizeof(F64Front) * wk.size()), total = o_tasks + sizeof(F64Task) * tasks.size();
     char* meta = nullptr;
     RSD_CUDA_TRY(cudaMallocAsync((void**)&meta, total, st));
     struct Free { char* p; cudaStream_t s; ~Free() { cudaFreeAsync(p, s); } } fr{meta, st};
-    RSD_CUDA_TRY(cudaMemcpyAsync(meta, stage_host(h, wk.data(), sizeof(F64Front) * nf_all), sizeof(F64Front) * nf_all, cudaMemcpyHostToDevice, st));
+    RSD_CUDA_TRY(cudaMemcpyAsync(meta, stage_host(h, wk.data(), sizeof(F64Front) * wk.size()), sizeof(F64Front) * wk.size(), cudaMemcpyHostToDevice, st));
     if (!tasks.empty())
         RSD_CUDA_TRY(cudaMemcpyAsync(meta + o_tasks, stage_host(h, tasks.data(), sizeof(F64Task) * tasks.size()),
                                      sizeof(F64Task) * tasks.size(), cudaMemcpyHostToDevice, st));
@@ -735,7 +749,7 @@ int factor_level_f64_tc(Handle& h, int li) {
         for (int k = 0; k < g.max_s; k += NB) {
             const int K0 = k / WP * WP;
             if (k > K0) RSD_TRY(run());
-            RSD_TRY(launch_chol_diag_f64(h, li, g.f0, g.nf, k, st));
+            RSD_TRY(launch_diag_f64(h, li, g.f0, g.nf, k, st));
             double bytes = 0;
             int rows = 0;                                   // below the diagonal block, at most
             for (int q = 0; q < g.nf; ++q) {
@@ -743,14 +757,14 @@ int factor_level_f64_tc(Handle& h, int li) {
                 if (f.s <= k) continue;
                 const int wd = std::min(NB, f.s - k);
                 rows = std::max(rows, f.N - k - wd);
-                bytes += 24.0 * (f.N - k - wd) * wd;
+                bytes += 24.0 * sides * (f.N - k - wd) * wd;
             }
             auto split = [&](bool x) -> int {
                 if (!rows) return RSD_OK;
                 const int pi = prof_begin(h, K_COPY16, st);
-                if (x) k_split_x<<<dim3((unsigned)((rows + 15) / 16), (unsigned)g.nf), 256, 0, st>>>(d_fr, d_wk + g.f0, k, K0, h.d_err, h.d_front_bad);
-                else k_split_a<<<dim3((unsigned)((rows + SA_ROWS - 1) / SA_ROWS + NB / SA_ROWS), (unsigned)g.nf), 256, 0, st>>>(
-                         d_fr, d_wk + g.f0, k, (rows + SA_ROWS - 1) / SA_ROWS, h.d_err, h.d_front_bad);
+                if (x) k_split_x<<<dim3((unsigned)((rows + 15) / 16), (unsigned)g.nf, (unsigned)sides), 256, 0, st>>>(d_fr, d_wk + (size_t)g.f0 * sides, k, K0, h.d_err, h.d_front_bad);
+                else k_split_a<<<dim3((unsigned)((rows + SA_ROWS - 1) / SA_ROWS + NB / SA_ROWS), (unsigned)g.nf, (unsigned)sides), 256, 0, st>>>(
+                         d_fr, d_wk + (size_t)g.f0 * sides, k, (rows + SA_ROWS - 1) / SA_ROWS, h.d_err, h.d_front_bad);
                 count_launch();
                 prof_end(h, pi, 0.0, bytes, st);
                 RSD_CUDA_TRY(cudaGetLastError());

@@ -357,12 +357,12 @@ int launch_assemble_fronts(Handle& h, int li, const int64_t* rowptr, const int* 
                            const int* tin, const int* tout);
 int launch_extend_add(Handle& h, int li);
 int run_factor_level(Handle& h, int li);
-// FP64 diagonal block factor + inverse at column k of fronts [f0, f0 + nf) of level li
-// (diag_f64.cu)
-int launch_chol_diag_f64(Handle& h, int li, int f0, int nf, int k, cudaStream_t st);
+// FP64 diagonal block factor + inverse (Cholesky, or LU and both inverses) at column k of
+// fronts [f0, f0 + nf) of level li (diag_f64.cu)
+int launch_diag_f64(Handle& h, int li, int f0, int nf, int k, cudaStream_t st);
 // FP64 level on the tensor cores (gemm_f64_tc.cu): workspace for fronts of the given row
-// counts, and the partial Cholesky of the level (needs the handle's f64_ws)
-size_t f64_tc_workspace(const std::vector<int>& rows);
+// counts, and the partial Cholesky or LU of the level (needs the handle's f64_ws)
+size_t f64_tc_workspace(const std::vector<int>& rows, bool lu);
 int factor_level_f64_tc(Handle& h, int li);
 // nonsymmetric fronts: assembly, extend-add and LU partial factorisation of level li
 int launch_assemble_fronts_lu(Handle& h, int li, const int64_t* rowptr, const int* col, const double* val,

@@ -6,6 +6,7 @@ import numpy as np
 import pytest
 
 import synth
+from oracle.rsd_exact import lu_nopivot
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -153,3 +154,60 @@ def test_fp64_fronts_in_several_groups_match_one_at_a_time(rsd):
     for q in range(count):
         r = ref[(q // 3) % 2]
         assert float((z[q] - r).abs().max()) <= 1e-13 * float(r.abs().max()), q
+
+
+@pytest.mark.parametrize("count,edge,s_root", [(1, 1, 3), (1, 33, 129), (2, 128, 31), (3, 130, 200), (2, 600, 90),
+                                               (1, 1030, 140), (20, 129, 65), (40, 97, 64), (80, 131, 33)])
+def test_fp64_lu_of_arrow_fronts(rsd, count, edge, s_root):
+    """Nonsymmetric fronts: L, U, the couplings and L_kk^-1 against LU without pivoting."""
+    sizes = [max(1, edge - (c % 3)) for c in range(count)]
+    A, owner, parent = _arrow(sizes, s_root, 5000 + 7 * edge)
+    skew = synth.uniform(5100 + edge, A.size).reshape(A.shape) * 0.5 * np.abs(A)
+    skew[np.arange(len(A)), np.arange(len(A))] = 0.0
+    A = A + np.triu(skew, 1) - np.triu(skew, 1).T
+    A[np.arange(len(A)), np.arange(len(A))] = 1.25 * (np.abs(A).sum(1) + 1.0)
+    p = rsd.RSD_PREC_FP64
+    h = rsd.RSD.setup(*_csr(A), torch.as_tensor(owner, device="cuda"), parent, prec_leaf=p, prec_mid=p, prec_root=p,
+                      nonsymmetric=True)
+    n, r0 = A.shape[0], A.shape[0] - s_root
+    S = A[r0:, r0:].copy()
+    off = 0
+    for c, s in enumerate(sizes):
+        L, U = lu_nopivot(A[off:off + s, off:off + s])
+        X = np.linalg.solve(U.T, A[r0:, off:off + s].T).T
+        Y = np.linalg.solve(L, A[off:off + s, r0:])
+        gl, gu = h.front_factor(1 + c), h.front_factor_upper(1 + c)
+        tol = 40 * (s + 1) * 2.2e-16                          # (s + 1) eps of each factor's scale, times the condition
+        d = np.abs(U).max()
+        assert np.abs(gl[:s] - L).max() <= tol and np.abs(gl[s:] - X).max() <= tol, c
+        assert np.abs(gu[:s] - U.T).max() <= tol * d and np.abs(gu[s:] - Y.T).max() <= tol * d, c
+        for k, D in enumerate(h.front_dinv(1 + c)):
+            w = min(128, s - 128 * k)
+            assert np.abs(D[:w, :w] @ L[128 * k:128 * k + w, 128 * k:128 * k + w] - np.eye(w)).max() <= tol
+            assert not D[w:].any() and not D[:, w:].any() and not np.triu(D, 1).any()
+        S -= X @ Y
+        off += s
+    L, U = lu_nopivot(S)
+    tol = 40 * (max(sizes) + s_root) * 2.2e-16
+    assert np.abs(h.front_factor(0) - L).max() <= tol
+    assert np.abs(h.front_factor_upper(0) - U.T).max() <= tol * np.abs(U).max()
+    f = synth.uniform(5200 + edge, n)
+    u, st = h.solve(torch.as_tensor(f, device="cuda"), tol=1e-12)
+    assert st["iterations"] == 1
+    x = np.linalg.solve(A, f)
+    assert np.abs(u.cpu().numpy() - x).max() <= 1e-12 * np.abs(x).max()
+    h.close()
+
+
+@pytest.mark.parametrize("where", ["diag", "below", "coupling"])
+def test_fp64_lu_front_refuses_values_that_are_not_finite(rsd, where):
+    A, owner, parent = _arrow([200, 40], 150, 77)
+    i, j = {"diag": (3, 3), "below": (190, 5), "coupling": (A.shape[0] - 2, 7)}[where]
+    rp, cl, vl = _csr(A)
+    row = torch.repeat_interleave(torch.arange(A.shape[0], device="cuda"), rp[1:] - rp[:-1])
+    vl[(row == i) & (cl == j)] = float("nan")
+    p = rsd.RSD_PREC_FP64
+    with pytest.raises(rsd.RSDError) as e:
+        rsd.RSD.setup(rp, cl, vl, torch.as_tensor(owner, device="cuda"), parent, prec_leaf=p, prec_mid=p, prec_root=p,
+                      nonsymmetric=True)
+    assert e.value.code == -3
