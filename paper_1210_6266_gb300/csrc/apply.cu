@@ -102,8 +102,12 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_al
 // Wait until *flag >= target; returns the last value seen.  Thread 0 polls, the block syncs.
 // After `limit` clock cycles (the handle's wait bound) the wait gives up, raises
 // ERR_TIMEOUT and returns as if the target had been reached; once the flag is raised,
-// every later wait of the launch returns at once.
-__device__ int wait_flag(const int* flag, int target, int* err, int* s_val, long long limit) {
+// every later wait of the launch returns at once.  The value goes through two shared slots
+// in turn (*turn): thread 0 may be at its next wait before the slowest warp has read this one's.
+struct FlagSlots { int v[2]; };
+__device__ int wait_flag(const int* flag, int target, int* err, FlagSlots* slots, int* turn, long long limit) {
+    int* s_val = &slots->v[*turn];
+    *turn ^= 1;
     if (threadIdx.x == 0) {
         int v = ld_volatile(flag);
         if (v < target) {
@@ -197,7 +201,9 @@ __global__ void __launch_bounds__(AT, GD == 1 ? 2 : 1) k_fwd_sweep(const FrontDe
     constexpr int VW = Vec<T>::W;
     constexpr int PASSES = NB / (32 * VW);
     constexpr int RPW = NB / AW;                 // rows per warp and block
-    __shared__ int s_item, s_flag;
+    __shared__ int s_item;
+    __shared__ FlagSlots s_flag;
+    int turn = 0;
     __shared__ __align__(16) A s_t[GD * NB];
     __shared__ __align__(16) A s_y[NB];
     __shared__ float s_ri[H ? GD * NB : 1];      // row factors of the item's rows (FP16 copy)
@@ -249,7 +255,7 @@ __global__ void __launch_bounds__(AT, GD == 1 ? 2 : 1) k_fwd_sweep(const FrontDe
                                                                   : make_uint4(0u, 0u, 0u, 0u);
                     }
                 const int need = min(cb + 2, ncb);
-                if (seen < need) seen = wait_flag(&f.flag[0], need, err, &s_flag, wait);
+                if (seen < need) seen = wait_flag(&f.flag[0], need, err, &s_flag, &turn, wait);
                 float y[8];
 #pragma unroll
                 for (int e = 0; e < 8; ++e) y[e] = (cl + e < cw) ? ld_cg(v + c0 + cl + e) : 0.f;
@@ -279,7 +285,7 @@ __global__ void __launch_bounds__(AT, GD == 1 ? 2 : 1) k_fwd_sweep(const FrontDe
                         const int row = r0 + g * NB + warp + AW * u;
                         l[g][u] = (g < nb && row < r1 && cl < cw) ? __ldg((const V*)(P + (int64_t)row * f.ldp + c0 + cl)) : V{};
                     }
-                if (ps == 0 && seen < cb + 1) seen = wait_flag(&f.flag[0], cb + 1, err, &s_flag, wait);
+                if (ps == 0 && seen < cb + 1) seen = wait_flag(&f.flag[0], cb + 1, err, &s_flag, &turn, wait);
                 A y[VW];
 #pragma unroll
                 for (int e = 0; e < VW; ++e) y[e] = (cl + e < cw) ? ld_cg(v + c0 + cl + e) : (A)0;
@@ -421,7 +427,9 @@ __global__ void __launch_bounds__(AT, GD == 1 ? 2 : 1) k_bwd_sweep(const FrontDe
     constexpr int VW = Vec<T>::W;
     constexpr int PASSES = NB / (32 * VW);
     constexpr int RB = 16 / PASSES;              // rows per warp per batch (a whole row block for FP32)
-    __shared__ int s_item, s_flag;
+    __shared__ int s_item;
+    __shared__ FlagSlots s_flag;
+    int turn = 0;
     __shared__ A s_red[AW][GD * NB];
     __shared__ A s_t[GD * NB];
     __shared__ A s_x[NB];
@@ -488,7 +496,7 @@ __global__ void __launch_bounds__(AT, GD == 1 ? 2 : 1) k_bwd_sweep(const FrontDe
                     l[u] = (in && cl < cw) ? __ldg((const uint4*)(P + (int64_t)row * f.ldp + c0 + cl)) : make_uint4(0u, 0u, 0u, 0u);
                     rsc[u] = in ? f.ri[row] : 0.f;
                 }
-                if (seen < need) seen = wait_flag(&f.flag[1], need, err, &s_flag, wait);
+                if (seen < need) seen = wait_flag(&f.flag[1], need, err, &s_flag, &turn, wait);
 #pragma unroll
                 for (int u = 0; u < RB; ++u) {
                     const int row = rlo + (warp + AW * u) * HW + sub;
@@ -537,7 +545,7 @@ __global__ void __launch_bounds__(AT, GD == 1 ? 2 : 1) k_bwd_sweep(const FrontDe
                             l[u][g][ps] = (row < g1 && cl < cw) ? __ldg((const V*)(P + (int64_t)row * f.ldp + c0 + cl)) : V{};
                         }
                 }
-                if (base == g0 && seen < need) seen = wait_flag(&f.flag[1], need, err, &s_flag, wait);
+                if (base == g0 && seen < need) seen = wait_flag(&f.flag[1], need, err, &s_flag, &turn, wait);
                 A x[RB];
 #pragma unroll
                 for (int u = 0; u < RB; ++u) {
@@ -770,7 +778,9 @@ __device__ __forceinline__ void cl_issue_tile(unsigned char* stage, const FrontD
 __global__ void __cluster_dims__(SWEEP_CL, 1, 1) __launch_bounds__(AT, 1)
 k_fwd_sweep_cl(const FrontDesc* __restrict__ fronts, const int* __restrict__ items, int n_items,
                int* __restrict__ ticket, int* __restrict__ err, long long wait) {
-    __shared__ int s_item, s_it, s_flag;
+    __shared__ int s_item, s_it;
+    __shared__ FlagSlots s_flag;
+    int turn = 0;
     __shared__ int s_got[SWEEP_CL];                  // epoch of the block pushed by each earlier CTA
     __shared__ __align__(16) float s_in[SWEEP_CL][NB];   // the blocks pushed by the earlier CTAs
     __shared__ __align__(16) float s_t[NB];
@@ -825,7 +835,7 @@ k_fwd_sweep_cl(const FrontDesc* __restrict__ fronts, const int* __restrict__ ite
             float4 y;
             if (i < g0) {
                 const bool yin = (ymask >> (i % CL_RING)) & 1u;
-                if (!yin && seen < i + 1) seen = wait_flag(&f.flag[0], i + 1, err, &s_flag, wait);
+                if (!yin && seen < i + 1) seen = wait_flag(&f.flag[0], i + 1, err, &s_flag, &turn, wait);
                 __syncthreads();                      // the stage of step i is in place
                 y = yin ? reinterpret_cast<const float4*>(stg + NB * NB * 2)[lane]
                         : __ldcg(reinterpret_cast<const float4*>(v + i * NB) + lane);
@@ -893,7 +903,9 @@ k_fwd_sweep_cl(const FrontDesc* __restrict__ fronts, const int* __restrict__ ite
 __global__ void __cluster_dims__(SWEEP_CL, 1, 1) __launch_bounds__(AT, 1)
 k_bwd_sweep_cl(const FrontDesc* __restrict__ fronts, const int* __restrict__ items, int n_items,
                int* __restrict__ ticket, int* __restrict__ err, double* __restrict__ z, long long wait) {
-    __shared__ int s_item, s_it, s_flag;
+    __shared__ int s_item, s_it;
+    __shared__ FlagSlots s_flag;
+    int turn = 0;
     __shared__ int s_got[SWEEP_CL];                  // epoch of the block pushed by each earlier CTA
     __shared__ __align__(16) float s_in[SWEEP_CL][NB];   // ri x of the blocks pushed by the earlier CTAs
     __shared__ __align__(16) float s_c[2][NB];       // ri x of the step's row block
@@ -957,7 +969,7 @@ k_bwd_sweep_cl(const FrontDesc* __restrict__ fronts, const int* __restrict__ ite
                     sc = xs + NB;
                 } else {
                     const int need = f.nd - rb;
-                    if (seen < need) seen = wait_flag(&f.flag[1], need, err, &s_flag, wait);
+                    if (seen < need) seen = wait_flag(&f.flag[1], need, err, &s_flag, &turn, wait);
                     if (tid < NB) {
                         const int row = rb * NB + tid;
                         s_c[i & 1][tid] = row < f.s ? __ldcg(v + row) * f.ri[row] : 0.f;
@@ -1017,6 +1029,240 @@ k_bwd_sweep_cl(const FrontDesc* __restrict__ fronts, const int* __restrict__ ite
     }
 }
 
+
+// ---- FP64 sweeps on clusters (levels of few fronts) --------------------------------------
+// The FP64 pipe (1.65 FMAs per clock and SM, 65 clocks a warp instruction) makes a block's
+// own steps the cost of the chain: the product with the previous block, two warp-sum
+// reductions and the product with Dinv keep one SM busy for about 20 us a block.  Here a
+// cluster of F64_CL CTAs takes a block, NB / F64_CL rows (forward) or as many rows of every
+// row block (backward) each, so that each SM has an eighth of that; t goes to every CTA
+// of the cluster through distributed shared memory.  The progress counter counts CTAs: a
+// block is done at F64_CL per block (a CTA finishes block k + 1 only after all of block k).
+// Work items, their order and the waits are those of the per-CTA kernels.
+constexpr int F64_CL = 8;
+constexpr int F64_R = NB / F64_CL;               // rows per CTA of a block
+constexpr int F64_CL_FRONTS = 16;               // levels of at most this many fronts
+constexpr int F64_AHEAD = 4;                     // blocks whose factor entries are loaded before their wait
+static_assert(F64_R == 2 * AW, "two rows per warp");
+
+__device__ __forceinline__ void cl_st_remote64(uint32_t a, double v) {
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+}
+
+// Sum of a over the warp into lanes 0..15, of b into lanes 16..31 (every lane of a half gets it).
+__device__ __forceinline__ double warp_sum_pair(double a, double b, int lane) {
+    const double give = lane < 16 ? b : a, keep = lane < 16 ? a : b;
+    double s = keep + __shfl_xor_sync(0xffffffffu, give, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+}
+
+// This CTA's part of a block is in global memory: count it
+__device__ __forceinline__ void f64_publish(int* flag, bool wrote) {
+    if (wrote) __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) atomicAdd(flag, 1);
+}
+
+__global__ void __cluster_dims__(F64_CL, 1, 1) __launch_bounds__(AT, 2)
+k_fwd_sweep_f64(const FrontDesc* __restrict__ fronts, const int* __restrict__ items, int n_items,
+                int* __restrict__ ticket, int* __restrict__ err, long long wait) {
+    __shared__ int s_item, s_it;
+    __shared__ FlagSlots s_flag;
+    int turn = 0;
+    __shared__ __align__(16) double s_t[NB];
+    __shared__ __align__(16) double s_D[F64_R * NB];          // this CTA's rows of Dinv
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t rank = cl_rank();
+    if (tid == 0) s_item = 0;
+    for (;;) {
+        const int it = cl_ticket(&s_item, &s_it, ticket, rank);
+        if (it >= n_items) return;
+        const int slot = items[it] >> 16, blk = items[it] & 0xffff;
+        const FrontDesc f = fronts[slot];
+        const bool diag = blk < f.nd;
+        const double* P = (const double*)f.P;
+        double* v = (double*)f.vec;
+        const int rb = diag ? blk * NB : f.s + (blk - f.nd) * NB, re = diag ? min(rb + NB, f.s) : min(rb + NB, f.N);
+        const int row0 = rb + (int)rank * F64_R + 2 * warp;        // this warp's two rows
+        if (diag)
+            prefetch_rows(s_D, (const double*)f.Dinv + (int64_t)blk * NB * NB + (int)rank * F64_R * NB, NB, F64_R);
+        cp_async_commit();
+        const int my_row = row0 + (lane >> 4);
+        const double vr = my_row < re ? ld_cg(v + my_row) : 0.0;
+        const int ncb = diag ? blk : f.nd;
+        double acc[2] = {0.0, 0.0};
+        int seen = 0;
+        for (int cb0 = 0; cb0 < ncb; cb0 += F64_AHEAD) {
+            double2 l[F64_AHEAD][2][2];
+#pragma unroll
+            for (int a = 0; a < F64_AHEAD; ++a)
+#pragma unroll
+                for (int u = 0; u < 2; ++u)
+#pragma unroll
+                    for (int ps = 0; ps < 2; ++ps) {
+                        const int c = (cb0 + a) * NB + ps * 64 + lane * 2;
+                        l[a][u][ps] = (cb0 + a < ncb && row0 + u < re && c < f.s)
+                                          ? __ldg((const double2*)(P + (int64_t)(row0 + u) * f.ldp + c)) : make_double2(0.0, 0.0);
+                    }
+#pragma unroll
+            for (int a = 0; a < F64_AHEAD; ++a) {
+                const int cb = cb0 + a;
+                if (cb >= ncb) break;
+                if (seen < F64_CL * (cb + 1)) seen = wait_flag(&f.flag[0], F64_CL * (cb + 1), err, &s_flag, &turn, wait);
+#pragma unroll
+                for (int ps = 0; ps < 2; ++ps) {
+                    const int c = cb * NB + ps * 64 + lane * 2;
+                    const double y0 = c < f.s ? ld_cg(v + c) : 0.0, y1 = c + 1 < f.s ? ld_cg(v + c + 1) : 0.0;
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        acc[u] = fma(l[a][u][ps].x, y0, acc[u]);
+                        acc[u] = fma(c + 1 < f.s ? l[a][u][ps].y : 0.0, y1, acc[u]);
+                    }
+                }
+            }
+        }
+        const double t = vr - warp_sum_pair(acc[0], acc[1], lane);
+        if (!diag) {
+            if ((lane & 15) == 0 && my_row < re) __stcg(v + my_row, t);
+            continue;
+        }
+        if ((lane & 15) < F64_CL)
+            cl_st_remote64(cl_map(&s_t[my_row - rb], (uint32_t)(lane & 15)), my_row < re ? t : 0.0);
+        cp_async_wait();
+        cl_sync();                                     // t is complete in every CTA
+        double part[2] = {0.0, 0.0};
+#pragma unroll
+        for (int ps = 0; ps < 2; ++ps) {
+            const int c = ps * 64 + lane * 2;
+            const double2 tt = *reinterpret_cast<const double2*>(s_t + c);
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const double2 d = *reinterpret_cast<const double2*>(s_D + (2 * warp + u) * NB + c);
+                part[u] = fma(d.x, tt.x, part[u]);
+                part[u] = fma(d.y, tt.y, part[u]);
+            }
+        }
+        const double y = warp_sum_pair(part[0], part[1], lane);
+        const bool wrote = (lane & 15) == 0 && my_row < re;
+        if (wrote) __stcg(v + my_row, y);
+        f64_publish(&f.flag[0], wrote);
+    }
+}
+
+// Backward: a CTA sums its F64_R rows of every row block below over all 128 columns; the
+// eight partial sums of a column meet in the CTA that owns it (16 columns each), which
+// hands t on and forms x = Dinv^T t for its columns.
+__global__ void __cluster_dims__(F64_CL, 1, 1) __launch_bounds__(AT, 2)
+k_bwd_sweep_f64(const FrontDesc* __restrict__ fronts, const int* __restrict__ items, int n_items,
+                int* __restrict__ ticket, int* __restrict__ err, double* __restrict__ z, long long wait) {
+    __shared__ int s_item, s_it;
+    __shared__ FlagSlots s_flag;
+    int turn = 0;
+    __shared__ __align__(16) double s_red[AW][NB];
+    __shared__ __align__(16) double s_part[NB];               // this CTA's rows' sums
+    __shared__ __align__(16) double s_t[NB];
+    __shared__ __align__(16) double s_D[NB * F64_R];          // Dinv, this CTA's columns
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t rank = cl_rank();
+    if (tid == 0) s_item = 0;
+    for (;;) {
+        const int it = cl_ticket(&s_item, &s_it, ticket, rank);
+        if (it >= n_items) return;
+        const int slot = items[it] >> 16, hi = items[it] & 0xffff;
+        const FrontDesc f = fronts[slot];
+        const double* P = (const double*)f.P;
+        double* v = (double*)f.vec;
+        const int c0 = hi * NB, wc = min(NB, f.s - c0), col0 = (int)rank * F64_R;
+        {
+            const double* D = (const double*)f.Dinv + (int64_t)hi * NB * NB + col0;
+            const uint32_t d0 = (uint32_t)__cvta_generic_to_shared(s_D);
+            for (int e = tid; e < NB * (F64_R / 2); e += AT) {
+                const int r = e / (F64_R / 2), q = e % (F64_R / 2);
+                cp16(d0 + (uint32_t)(r * F64_R + 2 * q) * 8, D + r * NB + 2 * q, true);
+            }
+        }
+        cp_async_commit();
+        const int ocol = col0 + (tid >> 3);                    // (tid < 128) the column this thread helps to sum
+        const double vc = tid < NB && ocol < wc ? ld_cg(v + c0 + ocol) : 0.0;
+        const int nB = (f.b + NB - 1) / NB, n_groups = nB + (f.nd - 1 - hi);
+        double acc[4] = {0.0, 0.0, 0.0, 0.0};
+        int seen = 0;
+        for (int g0 = 0; g0 < n_groups; g0 += F64_AHEAD) {
+            double2 l[F64_AHEAD][2][2];
+            int row[F64_AHEAD], rend[F64_AHEAD], need[F64_AHEAD];
+#pragma unroll
+            for (int a = 0; a < F64_AHEAD; ++a) {
+                const int g = g0 + a;
+                int r, e;
+                if (g < nB) { r = f.s + (nB - 1 - g) * NB; e = min(r + NB, f.N); need[a] = 0; }
+                else { const int rb = f.nd - 1 - (g - nB); r = rb * NB; e = min(r + NB, f.s); need[a] = F64_CL * (f.nd - rb); }
+                row[a] = r + (int)rank * F64_R + 2 * warp;
+                rend[a] = g < n_groups ? e : INT_MIN;              // (no row past the last group)
+#pragma unroll
+                for (int u = 0; u < 2; ++u)
+#pragma unroll
+                    for (int ps = 0; ps < 2; ++ps) {
+                        const int c = ps * 64 + lane * 2;
+                        l[a][u][ps] = (row[a] + u < rend[a] && c < wc)
+                                          ? __ldg((const double2*)(P + (int64_t)(row[a] + u) * f.ldp + c0 + c)) : make_double2(0.0, 0.0);
+                    }
+            }
+#pragma unroll
+            for (int a = 0; a < F64_AHEAD; ++a) {
+                if (g0 + a >= n_groups) break;
+                if (seen < need[a]) seen = wait_flag(&f.flag[1], need[a], err, &s_flag, &turn, wait);
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const double x = row[a] + u < rend[a] ? ld_cg(v + row[a] + u) : 0.0;
+#pragma unroll
+                    for (int ps = 0; ps < 2; ++ps) {
+                        acc[2 * ps] = fma(l[a][u][ps].x, x, acc[2 * ps]);
+                        acc[2 * ps + 1] = fma(l[a][u][ps].y, x, acc[2 * ps + 1]);
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int ps = 0; ps < 2; ++ps) *reinterpret_cast<double2*>(&s_red[warp][ps * 64 + lane * 2]) = make_double2(acc[2 * ps], acc[2 * ps + 1]);
+        __syncthreads();
+        if (tid < NB) {
+            double sum = 0.0;
+#pragma unroll
+            for (int q = 0; q < AW; ++q) sum += s_red[q][tid];
+            s_part[tid] = sum;
+        }
+        cl_sync();                                     // every CTA's sums are in place
+        if (tid < NB) {                                // thread (column tid / 8, CTA tid % 8)
+            double sum = cl_ld_f64(cl_map(&s_part[ocol], (uint32_t)(tid & 7)));
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+            cl_st_remote64(cl_map(&s_t[ocol], (uint32_t)(tid & 7)), ocol < wc ? vc - sum : 0.0);
+        }
+        cp_async_wait();
+        cl_sync();                                     // t is complete in every CTA
+        // x_c = sum_r Dinv[r][c] t_r: lane = (column, half of the rows' pairs), eight rows a thread
+        const int cc = lane & 15, rg = 2 * warp + (lane >> 4);
+        double x = 0.0;
+#pragma unroll
+        for (int q = 0; q < NB / 16; ++q) x = fma(s_D[(rg + 16 * q) * F64_R + cc], s_t[rg + 16 * q], x);
+        x += __shfl_xor_sync(0xffffffffu, x, 16);
+        if (lane < 16) s_red[0][warp * F64_R + cc] = x;
+        __syncthreads();
+        const bool mine = tid < NB && (tid & 7) == 0 && ocol < wc;
+        if (tid < NB) {
+            double sum = s_red[0][(tid & 7) * F64_R + (tid >> 3)];
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+            if (mine) {
+                __stcg(v + c0 + ocol, sum);
+                z[f.I[c0 + ocol]] = sum;
+            }
+        }
+        f64_publish(&f.flag[1], mine);
+    }
+}
 
 // Dynamic shared memory of the sweep kernels: GD inverted diagonal blocks plus, for
 // GD = 2, one factor block (FP16 when read from the copy).
@@ -1093,8 +1339,31 @@ int cl_grid(int n_items, int* out) {
     return RSD_OK;
 }
 
-// Upward / downward sweep kernel of a level: the cluster kernels on a cl_sweep level,
-// else the per-CTA kernels with the level's group size.
+// Clusters of the FP64 cluster sweeps resident at once on the current device.
+int f64_cl_grid(int n_items, int* out) {
+    static int max_cl[64] = {};
+    int dev = 0;
+    RSD_CUDA_TRY(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= 64) return RSD_ERR_ARG;
+    if (!max_cl[dev]) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(F64_CL * 64);
+        cfg.blockDim = dim3(AT);
+        int n1 = 0, n2 = 0;
+        RSD_CUDA_TRY(cudaOccupancyMaxActiveClusters(&n1, (void*)k_fwd_sweep_f64, &cfg));
+        RSD_CUDA_TRY(cudaOccupancyMaxActiveClusters(&n2, (void*)k_bwd_sweep_f64, &cfg));
+        max_cl[dev] = std::max(1, std::min(n1, n2));
+    }
+    *out = std::max(1, std::min(n_items, max_cl[dev]));
+    return RSD_OK;
+}
+
+// FP64 levels of few fronts are bound by their chains of blocks and run on clusters;
+// many fronts fill the chip with one CTA a block.
+inline bool f64_cluster_level(const Level& L) { return is_fp64(L.prec) && (int)L.fronts.size() <= F64_CL_FRONTS; }
+
+// Upward / downward sweep kernel of a level: the cluster kernels on a cl_sweep level or an
+// FP64 level of few fronts, else the per-CTA kernels with the level's group size.
 template <typename T, typename A>
 int launch_fwd_level(const Level& L, int grid, cudaStream_t st, const FrontDesc* fr, const int* items, int n, int* tk,
                      int* err, long long wait) {
@@ -1105,6 +1374,11 @@ int launch_fwd_level(const Level& L, int grid, cudaStream_t st, const FrontDesc*
             k_fwd_sweep_cl<<<ncl * SWEEP_CL, AT, CL_SMEM, st>>>(fr, items, n, tk, err, wait);
             return RSD_OK;
         }
+    } else if (f64_cluster_level(L)) {
+        int ncl = 0;
+        RSD_TRY(f64_cl_grid(n, &ncl));
+        k_fwd_sweep_f64<<<ncl * F64_CL, AT, 0, st>>>(fr, items, n, tk, err, wait);
+        return RSD_OK;
     }
     launch_fwd<T, A>(sweep_group(L), L.h16, grid, st, fr, items, n, tk, err, wait);
     return RSD_OK;
@@ -1120,6 +1394,11 @@ int launch_bwd_level(const Level& L, int grid, cudaStream_t st, const FrontDesc*
             k_bwd_sweep_cl<<<ncl * SWEEP_CL, AT, CL_SMEM, st>>>(fr, items, n, tk, err, z, wait);
             return RSD_OK;
         }
+    } else if (f64_cluster_level(L)) {
+        int ncl = 0;
+        RSD_TRY(f64_cl_grid(n, &ncl));
+        k_bwd_sweep_f64<<<ncl * F64_CL, AT, 0, st>>>(fr, items, n, tk, err, z, wait);
+        return RSD_OK;
     }
     launch_bwd<T, A>(sweep_group(L), L.h16, grid, st, fr, items, n, tk, err, z, wait);
     return RSD_OK;
