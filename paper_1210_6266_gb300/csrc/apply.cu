@@ -99,6 +99,31 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
+// Sums of a[0..16) over the warp, merged as they go (16 exchanges and additions instead of
+// 80): lane l gets the sum of a[l >> 1].
+template <typename A>
+__device__ __forceinline__ A warp_sum16(const A (&a)[16], int lane) {
+    A b[8], c[4], d[2];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const A give = lane & 16 ? a[i] : a[i + 8];
+        b[i] = (lane & 16 ? a[i + 8] : a[i]) + __shfl_xor_sync(0xffffffffu, give, 16);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const A give = lane & 8 ? b[i] : b[i + 4];
+        c[i] = (lane & 8 ? b[i + 4] : b[i]) + __shfl_xor_sync(0xffffffffu, give, 8);
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const A give = lane & 4 ? c[i] : c[i + 2];
+        d[i] = (lane & 4 ? c[i + 2] : c[i]) + __shfl_xor_sync(0xffffffffu, give, 4);
+    }
+    const A give = lane & 2 ? d[0] : d[1];
+    const A e = (lane & 2 ? d[1] : d[0]) + __shfl_xor_sync(0xffffffffu, give, 2);
+    return e + __shfl_xor_sync(0xffffffffu, e, 1);
+}
+
 // Wait until *flag >= target; returns the last value seen.  Thread 0 polls, the block syncs.
 // After `limit` clock cycles (the handle's wait bound) the wait gives up, raises
 // ERR_TIMEOUT and returns as if the target had been reached; once the flag is raised,
@@ -298,25 +323,21 @@ __global__ void __launch_bounds__(AT, GD == 1 ? 2 : 1) k_fwd_sweep(const FrontDe
             }
         }
         }
+        static_assert(RPW == 16, "warp_sum16");
+        A sum[GD];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-            for (int g = 0; g < GD; ++g)
-#pragma unroll
-                for (int u = 0; u < RPW; ++u) acc[g][u] += __shfl_xor_sync(0xffffffffu, acc[g][u], o);
+        for (int g = 0; g < GD; ++g) sum[g] = warp_sum16(acc[g], lane);
         __syncthreads();                             // s_t holds v on the item's rows
-        if (lane == 0) {
+        if ((lane & 1) == 0) {
 #pragma unroll
-            for (int g = 0; g < GD; ++g)
-#pragma unroll
-                for (int u = 0; u < RPW; ++u) {
-                    const int q = g * NB + warp + AW * u;
-                    if constexpr (H) {
-                        if (r0 + q < r1) s_t[q] -= acc[g][u] * s_ri[q];
-                    } else {
-                        if (r0 + q < r1) s_t[q] -= acc[g][u];
-                    }
+            for (int g = 0; g < GD; ++g) {
+                const int q = g * NB + warp + AW * (lane >> 1);
+                if constexpr (H) {
+                    if (r0 + q < r1) s_t[q] -= sum[g] * s_ri[q];
+                } else {
+                    if (r0 + q < r1) s_t[q] -= sum[g];
                 }
+            }
         }
         __syncthreads();
         if (!diag) {
@@ -346,19 +367,13 @@ __global__ void __launch_bounds__(AT, GD == 1 ? 2 : 1) k_fwd_sweep(const FrontDe
                         for (int e = 0; e < VW; ++e) part[u] += (A)vget(d, e) * yv[e];
                     }
                 }
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-                    for (int u = 0; u < RPW; ++u) part[u] += __shfl_xor_sync(0xffffffffu, part[u], o);
-                if (lane == 0) {
-#pragma unroll
-                    for (int u = 0; u < RPW; ++u) {
-                        const int rr = warp + AW * u;
-                        if constexpr (H) {
-                            if (rr < w) s_t[g * NB + rr] -= part[u] * s_ri[g * NB + rr];
-                        } else {
-                            if (rr < w) s_t[g * NB + rr] -= part[u];
-                        }
+                const A psum = warp_sum16(part, lane);
+                if ((lane & 1) == 0) {
+                    const int rr = warp + AW * (lane >> 1);
+                    if constexpr (H) {
+                        if (rr < w) s_t[g * NB + rr] -= psum * s_ri[g * NB + rr];
+                    } else {
+                        if (rr < w) s_t[g * NB + rr] -= psum;
                     }
                 }
                 __syncthreads();
@@ -380,23 +395,17 @@ __global__ void __launch_bounds__(AT, GD == 1 ? 2 : 1) k_fwd_sweep(const FrontDe
                     for (int e = 0; e < VW; ++e) part[u] += (A)vget(d, e) * t[e];
                 }
             }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-                for (int u = 0; u < RPW; ++u) part[u] += __shfl_xor_sync(0xffffffffu, part[u], o);
-            if (lane == 0) {
-#pragma unroll
-                for (int u = 0; u < RPW; ++u) {
-                    const int rr = warp + AW * u;
-                    if (rr < w) {
-                        __stcg(v + r0 + g * NB + rr, part[u]);
-                        s_y[rr] = part[u];
-                    }
+            const A y = warp_sum16(part, lane);
+            if ((lane & 1) == 0) {
+                const int rr = warp + AW * (lane >> 1);
+                if (rr < w) {
+                    __stcg(v + r0 + g * NB + rr, y);
+                    s_y[rr] = y;
                 }
             }
             // each block is published as soon as it is done, so the next item can take
             // this block's column while the second block of the pair is solved
-            publish_flag(&f.flag[0], blk + g + 1, lane == 0);
+            publish_flag(&f.flag[0], blk + g + 1, (lane & 1) == 0);
         }
         __syncthreads();
     }
@@ -857,17 +866,11 @@ k_fwd_sweep_cl(const FrontDesc* __restrict__ fronts, const int* __restrict__ ite
             }
         }
         asm volatile("cp.async.wait_group 0;" ::: "memory");
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-            for (int u = 0; u < 16; ++u) acc[u] += __shfl_xor_sync(0xffffffffu, acc[u], o);
+        const float mine = warp_sum16(acc, lane);     // row 16 warp + lane / 2
         __syncthreads();                              // s_v and s_ri (written at the item's start) are in place
         {
-            float mine = acc[0];                      // lane u < 16 takes row 16 warp + u
-#pragma unroll
-            for (int u = 1; u < 16; ++u) mine = lane == u ? acc[u] : mine;
-            const int rr = warp * 16 + lane;
-            if (lane < 16) s_t[rr] = rr < w ? s_v[rr] - mine * s_ri[rr] : 0.f;
+            const int rr = warp * 16 + (lane >> 1);
+            if ((lane & 1) == 0) s_t[rr] = rr < w ? s_v[rr] - mine * s_ri[rr] : 0.f;
         }
         __syncthreads();
         float yq[4] = {0.f, 0.f, 0.f, 0.f};
