@@ -53,18 +53,22 @@ namespace {
 
 constexpr int ND = 8;                        // digits per entry
 constexpr int TN = 64;                       // tile columns (and rows per digit block)
+constexpr int TN_FEW = 16;                   // tile columns of a launch with few tiles
 constexpr int KB = 64;                       // K columns per digit block
 constexpr int WP = 512;                      // panel width: the longest K with exact sums
 constexpr int BLK = 64 * 128;                // bytes of a digit block (64 rows x 64 FP16)
 constexpr int GROUP = ND * BLK;              // a row tile's eight digits for one K block
-constexpr int A_ST = 5;                      // ring stages of A (two digit blocks each)
 constexpr int A_BYTES = 2 * BLK;
 constexpr int UPD_DB = 7, UPD_FB = 59;       // digits of the updates
 constexpr float UPD_NORM2 = 7.9f;            // a row's largest sum of (x 2^-e)^2
 constexpr int SLV_DB = 8, SLV_FB = 62;       // digits of the panel solve
 constexpr int EPI_WARPS = 16;                // four per TMEM lane quadrant, 16 columns each
 constexpr int F64_THREADS = 64 + 32 * EPI_WARPS;
-constexpr int F64_SMEM = 2 * GROUP + A_ST * A_BYTES + 1024 + 256;
+template <int W> struct F64Smem {            // W: tile columns
+    static constexpr int B_BYTES = ND * W * 128;                 // a K block of B, all digits
+    static constexpr int A_ST = W == TN ? 5 : 10;                // ring stages of A (two digit blocks each)
+    static constexpr int TOTAL = 2 * B_BYTES + A_ST * A_BYTES + 1024 + 384;
+};
 
 // One front's operands and target of one launch.  Row tiles are 64 rows counted from the
 // front's row 0; A's and B's buffers hold [K block][row tile][digit][64 x 128 B].
@@ -76,8 +80,8 @@ struct F64Task {
     int a_nrt, b_nrt;                        // row tiles per K block
     int ldp, ldu, s;
     int r_lo, r_hi, c_lo, c_hi;              // rows and columns of C to write
-    int tm0, tn0, ntm, ntn;                  // 128-row and 64-column tiles
-    int b_rt0;                               // B's row tile for column tile tn is tn - b_rt0
+    int tm0, tn0, ntm, ntn;                  // 128-row and W-column tiles
+    int b_c0;                                // B's row for column c is c - b_c0 (a multiple of 64)
     int nkb, lower;
     int tile_begin;
 };
@@ -242,15 +246,14 @@ __device__ __forceinline__ int store_digits(const double (&x)[8], const int (&e)
 // block) and Dinv_cj 2^s_j, s_j the exponent of L_jj (a row's entries then compare across
 // columns of different scale).  blockIdx.x < na: SA_ROWS rows of A, else of Dinv.
 // Nonsymmetric fronts, blockIdx.z = 0: P against (U_kk^T)^-1, s_j of U_jj; 1: PU against L_kk^-1.
-constexpr int SA_ROWS = 64;
 __global__ void __launch_bounds__(256) k_split_a(const FrontDesc* __restrict__ fronts, const F64Front* __restrict__ wk, int k,
-                                                int na, int* __restrict__ err, int* __restrict__ bad_front) {
+                                                int na, int nr, int* __restrict__ err, int* __restrict__ bad_front) {
     __shared__ int sj[NB];
     const FrontDesc f = fronts[blockIdx.y];
     if (f.s <= k) return;
     const int w = min(NB, f.s - k), ch = threadIdx.x & 15, j0 = ch * 8;
     const bool isA = (int)blockIdx.x < na;
-    const int r0 = isA ? k + w + (int)blockIdx.x * SA_ROWS : ((int)blockIdx.x - na) * SA_ROWS;
+    const int r0 = isA ? k + w + (int)blockIdx.x * nr : ((int)blockIdx.x - na) * nr;
     if (isA && r0 >= f.N) return;
     const F64Front wf = wk[gridDim.z * blockIdx.y + blockIdx.z];
     const bool lu = gridDim.z == 2, upper = blockIdx.z == 1;
@@ -261,7 +264,7 @@ __global__ void __launch_bounds__(256) k_split_a(const FrontDesc* __restrict__ f
     if (threadIdx.x < NB) sj[threadIdx.x] = (int)threadIdx.x < w ? exp_above(diag[(int64_t)(k + threadIdx.x) * f.ldp + k + threadIdx.x], &ok) : 0;
     __syncthreads();
 #pragma unroll 1
-    for (int r = r0 + (threadIdx.x >> 4); r < r0 + SA_ROWS; r += 16) {
+    for (int r = r0 + (threadIdx.x >> 4); r < r0 + nr; r += 16) {
         const bool in = isA ? r < f.N : r < w;
         const double* src = (isA ? P + (int64_t)r * f.ldp + k : Dk + r * NB) + j0;
         int top = E_NONE, e[8];
@@ -341,9 +344,11 @@ __global__ void __launch_bounds__(256) k_split_x(const FrontDesc* __restrict__ f
 
 // ---- the GEMM ------------------------------------------------------------------------------
 
-// tile `g` of a launch: its task, 128-row tile and 64-column tile.  Lower tasks (C's lower
-// triangle) have min(ntn, c0 + 2q) tiles in row tile q, c0 = 2 tm0 + 2 - tn0.
+// tile `g` of a launch: its task, 128-row tile and W-column tile.  Lower tasks (C's lower
+// triangle) have min(ntn, c0 + m q) tiles in row tile q, m = 128 / W, c0 = m (tm0 + 1) - tn0.
+template <int W>
 __device__ __forceinline__ int f64_tile(const F64Task* __restrict__ tasks, int ntask, int g, int* tm, int* tn) {
+    constexpr int m = BM / W;
     int lo = 0, hi = ntask - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
@@ -353,18 +358,19 @@ __device__ __forceinline__ int f64_tile(const F64Task* __restrict__ tasks, int n
     const int l = g - t.tile_begin;
     int q, c;
     if (t.lower) {
-        const int c0 = 2 * t.tm0 + 2 - t.tn0;
-        const int qs = max(0, (t.ntn - c0 + 1) / 2), before = c0 * qs + qs * (qs - 1);
-        if (l < before) {
-            const float b = (float)(c0 - 1);
-            q = (int)((sqrtf(b * b + 4.0f * (float)l) - b) * 0.5f);
+        const int c0 = m * (t.tm0 + 1) - t.tn0;
+        auto before = [&](int r) { return c0 * r + m / 2 * r * (r - 1); };    // tiles of row tiles 0 .. r - 1
+        const int qs = max(0, (t.ntn - c0 + m - 1) / m);                       // the first with all ntn
+        if (l < before(qs)) {
+            const float b = (float)c0 - 0.5f * m;
+            q = (int)((sqrtf(b * b + 2.0f * m * (float)l) - b) / m);
             q = max(0, min(q, qs - 1));
-            while (q > 0 && c0 * q + q * (q - 1) > l) --q;
-            while (q + 1 < qs && c0 * (q + 1) + (q + 1) * q <= l) ++q;
-            c = l - (c0 * q + q * (q - 1));
+            while (q > 0 && before(q) > l) --q;
+            while (q + 1 < qs && before(q + 1) <= l) ++q;
+            c = l - before(q);
         } else {
-            q = qs + (l - before) / t.ntn;
-            c = (l - before) % t.ntn;
+            q = qs + (l - before(qs)) / t.ntn;
+            c = (l - before(qs)) % t.ntn;
         }
     } else {
         q = l / t.ntn;
@@ -375,20 +381,26 @@ __device__ __forceinline__ int f64_tile(const F64Task* __restrict__ tasks, int n
     return lo;
 }
 
-__device__ __forceinline__ void tmem_ld8(uint32_t a, uint32_t (&r)[8]) {
+__device__ __forceinline__ void tmem_ld(uint32_t a, uint32_t (&r)[4]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a));
+}
+
+__device__ __forceinline__ void tmem_ld(uint32_t a, uint32_t (&r)[8]) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
                  : "r"(a));
 }
 
-// SOLVE = false: C -= A B^T.  SOLVE = true: C = A B^T.
-template <bool SOLVE>
+// SOLVE = false: C -= A B^T.  SOLVE = true: C = A B^T.  W: tile columns.
+template <bool SOLVE, int W>
 __global__ void __launch_bounds__(F64_THREADS, 1)
 k_gemm_f64_tc(const F64Task* __restrict__ tasks, int ntask, int n_tiles, int* __restrict__ err) {
     extern __shared__ unsigned char smem_raw[];
+    constexpr int B_BYTES = F64Smem<W>::B_BYTES, A_ST = F64Smem<W>::A_ST;
     const uint32_t raw = smem_u32(smem_raw);
-    const uint32_t base = (raw + 1023) & ~1023u;                // B: 2 x 64 KB, A: A_ST x 16 KB, barriers
-    const uint32_t sA = base + 2 * GROUP, bars = sA + A_ST * A_BYTES;
+    const uint32_t base = (raw + 1023) & ~1023u;                // two K blocks of B, A_ST x 16 KB of A, barriers
+    const uint32_t sA = base + 2 * B_BYTES, bars = sA + A_ST * A_BYTES;
     const uint32_t b_full = bars, b_empty = bars + 16, a_full = bars + 32, a_empty = a_full + 8 * A_ST;
     const uint32_t acc_full = a_empty + 8 * A_ST, acc_empty = acc_full + 8;
     uint32_t* tmem_slot = (uint32_t*)(smem_raw + (acc_empty + 8 - raw));
@@ -401,7 +413,7 @@ k_gemm_f64_tc(const F64Task* __restrict__ tasks, int ntask, int n_tiles, int* __
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(512) : "memory");
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(ND * W) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -415,16 +427,23 @@ k_gemm_f64_tc(const F64Task* __restrict__ tasks, int ntask, int n_tiles, int* __
             bool ok = true;
             for (int g = blockIdx.x; g < n_tiles && ok; g += gridDim.x) {
                 int tm, tn;
-                const F64Task& t = tasks[f64_tile(tasks, ntask, g, &tm, &tn)];
+                const F64Task& t = tasks[f64_tile<W>(tasks, ntask, g, &tm, &tn)];
                 const char* A = t.A + (int64_t)(2 * tm) * GROUP;
-                const char* B = t.B + (int64_t)(tn - t.b_rt0) * GROUP;
+                const int br = tn * W - t.b_c0;                  // B's first row
+                const char* B = t.B + (int64_t)(br / TN) * GROUP + (br % TN) * 128;
                 const int64_t sa = (int64_t)t.a_nrt * GROUP, sb = (int64_t)t.b_nrt * GROUP;
                 const int nkb = t.nkb;
                 for (int kb = 0; kb < nkb && ok; ++kb, ++ib) {
                     const uint32_t q = ib & 1;
                     if (!mbar_wait(b_empty + 8 * q, ((ib >> 1) & 1) ^ 1, err)) { ok = false; break; }
-                    mbar_expect_tx(b_full + 8 * q, GROUP);
-                    bulk_load(base + q * GROUP, B + kb * sb, GROUP, b_full + 8 * q);
+                    mbar_expect_tx(b_full + 8 * q, B_BYTES);
+                    if constexpr (W == TN) {
+                        bulk_load(base + q * B_BYTES, B + kb * sb, B_BYTES, b_full + 8 * q);
+                    } else {
+#pragma unroll
+                        for (int d = 0; d < ND; ++d)
+                            bulk_load(base + q * B_BYTES + d * W * 128, B + kb * sb + d * BLK, W * 128, b_full + 8 * q);
+                    }
                     for (int i = 0; i < ND; ++i, ++ia) {
                         const uint32_t s = ia % A_ST;
                         if (!mbar_wait(a_empty + 8 * s, ((ia / A_ST) & 1) ^ 1, err)) { ok = false; break; }
@@ -446,7 +465,7 @@ k_gemm_f64_tc(const F64Task* __restrict__ tasks, int ntask, int n_tiles, int* __
             bool ok = true;
             for (int g = blockIdx.x; g < n_tiles && ok; g += gridDim.x, ++it) {
                 int tm, tn;
-                const int nkb = tasks[f64_tile(tasks, ntask, g, &tm, &tn)].nkb;
+                const int nkb = tasks[f64_tile<W>(tasks, ntask, g, &tm, &tn)].nkb;
                 if (!mbar_wait(acc_empty, (it & 1) ^ 1, err)) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 for (int kb = 0; kb < nkb && ok; ++kb, ++ib) {
@@ -457,12 +476,13 @@ k_gemm_f64_tc(const F64Task* __restrict__ tasks, int ntask, int n_tiles, int* __
                         if (!mbar_wait(a_full + 8 * s, (ia / A_ST) & 1, err)) { ok = false; break; }
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                         // digit i of A times digits j of B, j < 8 - i, into the sums d = i + j
-                        for (int j = 0; j < ND - i; j += 4) {
-                            const uint32_t idesc = idesc_of(0u, 64 * min(4, ND - i - j));
+                        constexpr int JN = 256 / W;              // digits of B per MMA, at most
+                        for (int j = 0; j < ND - i; j += JN) {
+                            const uint32_t idesc = idesc_of(0u, W * min(JN, ND - i - j));
 #pragma unroll
                             for (int kk = 0; kk < 4; ++kk)
-                                mma_f16(tmem + (i + j) * TN, smem_desc(sA + s * A_BYTES + kk * 32),
-                                        smem_desc(base + q * GROUP + j * BLK + kk * 32), idesc, (kb | i | kk) != 0);
+                                mma_f16(tmem + (i + j) * W, smem_desc(sA + s * A_BYTES + kk * 32),
+                                        smem_desc(base + q * B_BYTES + j * W * 128 + kk * 32), idesc, (kb | i | kk) != 0);
                         }
                         mma_commit(a_empty + 8 * s);
                     }
@@ -472,20 +492,20 @@ k_gemm_f64_tc(const F64Task* __restrict__ tasks, int ntask, int n_tiles, int* __
             }
         }
     } else {
-        constexpr int CW = TN / (EPI_WARPS / 4);             // columns per thread
+        constexpr int CW = W / (EPI_WARPS / 4), GW = CW < 8 ? CW : 8;   // columns per thread, per load
         constexpr int DB = SOLVE ? SLV_DB : UPD_DB, S = 4 * DB;
         constexpr int E0 = 14 * DB - 7 * DB - 2 * (SOLVE ? SLV_FB : UPD_FB);   // exponent of the sum d = 7
         const int quarter = warp & 3, part = (warp - 2) >> 2, row = quarter * 32 + lane;
         uint32_t it = 0;
         for (int g = blockIdx.x; g < n_tiles; g += gridDim.x, ++it) {
             int tm, tn;
-            const F64Task& t = tasks[f64_tile(tasks, ntask, g, &tm, &tn)];
-            const int gr = tm * BM + row, c_base = tn * TN + part * CW;
+            const F64Task& t = tasks[f64_tile<W>(tasks, ntask, g, &tm, &tn)];
+            const int gr = tm * BM + row, c_base = tn * W + part * CW;
             const int r_lo = t.r_lo, r_hi = t.r_hi, c_lo = t.c_lo, s = t.s;
             const int c_hi = t.lower ? min(t.c_hi, gr + 1) : t.c_hi;
             const bool in = gr >= r_lo && gr < r_hi && c_base < c_hi && c_base + CW > c_lo;
             const int ea = in ? t.ea[gr] : 0;
-            const int* eb = t.eb + (c_base - t.b_rt0 * TN);
+            const int* eb = t.eb + (c_base - t.b_c0);
             double* P = t.P + (int64_t)gr * t.ldp;
             double* U = t.U + (int64_t)(gr - s) * t.ldu - s;
             if (!SOLVE && in && c_base >= c_lo) asm volatile("prefetch.global.L2 [%0];" ::"l"(c_base < s ? P + c_base : U + c_base));
@@ -494,25 +514,25 @@ k_gemm_f64_tc(const F64Task* __restrict__ tasks, int ntask, int n_tiles, int* __
             long long a1[CW];
             uint32_t a0[CW];
 #pragma unroll
-            for (int q = 0; q < CW / 8; ++q)
+            for (int q = 0; q < CW / GW; ++q)
 #pragma unroll
                 for (int lowhalf = 0; lowhalf < 2; ++lowhalf) {
-                    uint32_t v[4][8];
+                    uint32_t v[4][GW];
 #pragma unroll
                     for (int d = 0; d < 4; ++d)
-                        tmem_ld8(tmem + ((uint32_t)(quarter * 32) << 16) + (4 * lowhalf + d) * TN + part * CW + q * 8, v[d]);
+                        tmem_ld(tmem + ((uint32_t)(quarter * 32) << 16) + (4 * lowhalf + d) * W + part * CW + q * GW, v[d]);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-                    for (int c = 0; c < 8; ++c) {
+                    for (int c = 0; c < GW; ++c) {
                         int n[4];
 #pragma unroll
                         for (int d = 0; d < 4; ++d) n[d] = __float2int_rn(__uint_as_float(v[d][c]));
                         const long long sum = (long long)n[0] * (1 << 3 * DB) + (long long)n[1] * (1 << 2 * DB) + (long long)n[2] * (1 << DB) + n[3];
                         if (!lowhalf) {
-                            a1[8 * q + c] = sum;
+                            a1[GW * q + c] = sum;
                         } else {
-                            a1[8 * q + c] += sum >> S;
-                            a0[8 * q + c] = (uint32_t)(sum & ((1ll << S) - 1));
+                            a1[GW * q + c] += sum >> S;
+                            a0[GW * q + c] = (uint32_t)(sum & ((1ll << S) - 1));
                         }
                     }
                 }
@@ -530,28 +550,29 @@ k_gemm_f64_tc(const F64Task* __restrict__ tasks, int ntask, int n_tiles, int* __
                     }
             }
 #pragma unroll
-            for (int q = 0; q < CW / 8; ++q) {
-                const int c0 = c_base + 8 * q;
-                if (c0 >= c_hi || c0 + 8 <= c_lo) continue;
+            for (int q = 0; q < CW / GW; ++q) {
+                const int c0 = c_base + GW * q;
+                if (c0 >= c_hi || c0 + GW <= c_lo) continue;
                 double* C = c0 >= s ? U : P;
-                if (c0 >= c_lo && c0 + 8 <= c_hi && (c0 + 8 <= s || (c0 >= s && !(s & 1)))) {
+                if (c0 >= c_lo && c0 + GW <= c_hi && (c0 + GW <= s || (c0 >= s && !(s & 1)))) {
                     double2* C2 = reinterpret_cast<double2*>(C + c0);
-                    double2 v[4];
+                    double2 v[GW / 2];
                     if constexpr (!SOLVE)
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) v[c] = C2[c];
+                        for (int c = 0; c < GW / 2; ++c) v[c] = C2[c];
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        const double x = from_fixed<S>(a1[8 * q + 2 * c], a0[8 * q + 2 * c], ea + __ldg(eb + 8 * q + 2 * c) + E0);
-                        const double y = from_fixed<S>(a1[8 * q + 2 * c + 1], a0[8 * q + 2 * c + 1], ea + __ldg(eb + 8 * q + 2 * c + 1) + E0);
+                    for (int c = 0; c < GW / 2; ++c) {
+                        const int k = GW * q + 2 * c;
+                        const double x = from_fixed<S>(a1[k], a0[k], ea + __ldg(eb + k) + E0);
+                        const double y = from_fixed<S>(a1[k + 1], a0[k + 1], ea + __ldg(eb + k + 1) + E0);
                         C2[c] = SOLVE ? make_double2(x, y) : make_double2(v[c].x - x, v[c].y - y);
                     }
                 } else {
 #pragma unroll
-                    for (int c = 0; c < 8; ++c) {
+                    for (int c = 0; c < GW; ++c) {
                         const int cc = c0 + c;
                         if (cc < c_lo || cc >= c_hi) continue;
-                        const double x = from_fixed<S>(a1[8 * q + c], a0[8 * q + c], ea + __ldg(eb + 8 * q + c) + E0);
+                        const double x = from_fixed<S>(a1[GW * q + c], a0[GW * q + c], ea + __ldg(eb + GW * q + c) + E0);
                         double* p = (cc >= s ? U : P) + cc;
                         *p = SOLVE ? x : *p - x;
                     }
@@ -563,7 +584,7 @@ k_gemm_f64_tc(const F64Task* __restrict__ tasks, int ntask, int n_tiles, int* __
     __syncthreads();
     if (warp == 1) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ND * W) : "memory");
     }
 }
 
@@ -575,10 +596,13 @@ size_t front_bytes(int N) {
     return (WP / KB + 2) * g + 4 * (size_t)GROUP + 4 * al(sizeof(int) * (size_t)N) + al(sizeof(int) * NB);
 }
 
-int64_t tiles_of(const F64Task& t) {
+// tiles of W columns covering the task's rows and columns
+int64_t set_tiles(F64Task& t, int W) {
+    t.tm0 = t.r_lo / BM; t.ntm = (t.r_hi + BM - 1) / BM - t.tm0;
+    t.tn0 = t.c_lo / W; t.ntn = (t.c_hi + W - 1) / W - t.tn0;
     if (!t.lower) return (int64_t)t.ntm * t.ntn;
     int64_t n = 0;
-    for (int q = 0; q < t.ntm; ++q) n += std::min(t.ntn, 2 * (t.tm0 + q) + 2 - t.tn0);
+    for (int q = 0; q < t.ntm; ++q) n += std::min(t.ntn, BM / W * (t.tm0 + q + 1) - t.tn0);
     return n;
 }
 
@@ -604,7 +628,7 @@ int factor_level_f64_tc(Handle& h, int li) {
     Level& L = h.levels[li];
     cudaStream_t st = h.stream;
     const int nf_all = (int)L.fronts.size(), sides = h.lu ? 2 : 1;
-    struct Launch { size_t off; int n, tiles, solve; double flops, bytes; };
+    struct Launch { size_t off; int n, tiles, solve, few; double flops, bytes; };
     struct Group { int f0, nf, max_s; };
     std::vector<Group> groups;
     std::vector<F64Front> wk((size_t)nf_all * sides);
@@ -639,11 +663,30 @@ int factor_level_f64_tc(Handle& h, int li) {
     // every launch's task list, uploaded once
     std::vector<F64Task> tasks;
     std::vector<Launch> launches;
-    auto begin = [&](int solve) { launches.push_back({tasks.size(), 0, 0, solve, 0, 0}); };
+    // Launches of few 128 x 64 tiles take 16-column tiles: a tile is a serial chain (the loads
+    // and MMAs of its K, then an epilogue of 16 columns a thread), about 28 us at K = 128 with
+    // most SMs idle; with four columns a thread and a quarter of the MMAs 14 us.  With more than
+    // half a wave of wide tiles the narrow ones, which load A four times as often, gain nothing.
+    auto finish = [&]() {
+        if (launches.empty()) return;
+        Launch& l = launches.back();
+        if (l.tiles * 2 > h.num_sms) return;
+        l.few = 1;
+        l.tiles = 0;
+        for (int i = 0; i < l.n; ++i) {
+            F64Task& t = tasks[l.off + i];
+            t.tile_begin = l.tiles;
+            l.tiles += (int)set_tiles(t, TN_FEW);
+        }
+    };
+    auto begin = [&](int solve) {
+        finish();
+        launches.push_back({tasks.size(), 0, 0, solve, 0, 0, 0});
+    };
     auto add = [&](F64Task t) {
         Launch& l = launches.back();
         t.tile_begin = l.tiles;
-        l.tiles += (int)tiles_of(t);
+        l.tiles += (int)set_tiles(t, TN);
         ++l.n;
         const double m = t.r_hi - t.r_lo, n = t.c_hi - t.c_lo;
         const double c = t.lower ? m * n - 0.5 * n * (n - 1) : m * n;
@@ -667,8 +710,6 @@ int factor_level_f64_tc(Handle& h, int li) {
                 t.P = (double*)(sd ? f.PU : f.P); t.U = (double*)f.U;
                 t.ldp = f.ldp; t.ldu = f.ldu; t.s = f.s;
                 t.r_lo = r0; t.r_hi = f.N; t.c_lo = c0; t.c_hi = c1;
-                t.tm0 = r0 / BM; t.ntm = (f.N + BM - 1) / BM - t.tm0;
-                t.tn0 = c0 / TN; t.ntn = (c1 + TN - 1) / TN - t.tn0;
                 t.nkb = nkb;
                 t.lower = lower;
                 add(t);
@@ -695,9 +736,7 @@ int factor_level_f64_tc(Handle& h, int li) {
                     t.P = (double*)(sd ? f.PU : f.P); t.U = (double*)f.U;
                     t.ldp = f.ldp; t.ldu = f.ldu; t.s = f.s;
                     t.r_lo = k + wd; t.r_hi = f.N; t.c_lo = k; t.c_hi = k + wd;
-                    t.tm0 = t.r_lo / BM; t.ntm = (f.N + BM - 1) / BM - t.tm0;
-                    t.tn0 = k / TN; t.ntn = (wd + TN - 1) / TN;
-                    t.b_rt0 = k / TN;
+                    t.b_c0 = k;
                     t.nkb = (wd + KB - 1) / KB;
                     add(t);
                 }
@@ -718,6 +757,7 @@ int factor_level_f64_tc(Handle& h, int li) {
             }
         }
     }
+    finish();
     const size_t o_tasks = al(sizeof(F64Front) * wk.size()), total = o_tasks + sizeof(F64Task) * tasks.size();
     char* meta = nullptr;
     RSD_CUDA_TRY(cudaMallocAsync((void**)&meta, total, st));
@@ -728,16 +768,20 @@ int factor_level_f64_tc(Handle& h, int li) {
                                      sizeof(F64Task) * tasks.size(), cudaMemcpyHostToDevice, st));
     const F64Front* d_wk = (const F64Front*)meta;
     const F64Task* d_tasks = (const F64Task*)(meta + o_tasks);
-    RSD_CUDA_TRY(cudaFuncSetAttribute(k_gemm_f64_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, F64_SMEM));
-    RSD_CUDA_TRY(cudaFuncSetAttribute(k_gemm_f64_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, F64_SMEM));
+    using Kernel = void (*)(const F64Task*, int, int, int*);
+    static constexpr Kernel kern[2][2] = {{k_gemm_f64_tc<false, TN>, k_gemm_f64_tc<true, TN>},
+                                          {k_gemm_f64_tc<false, TN_FEW>, k_gemm_f64_tc<true, TN_FEW>}};
+    static constexpr int smem[2] = {F64Smem<TN>::TOTAL, F64Smem<TN_FEW>::TOTAL};
+    for (int few = 0; few < 2; ++few)
+        for (int sv = 0; sv < 2; ++sv)
+            RSD_CUDA_TRY(cudaFuncSetAttribute(kern[few][sv], cudaFuncAttributeMaxDynamicSharedMemorySize, smem[few]));
     size_t li_ = 0;
     auto run = [&]() -> int {
         const Launch& l = launches[li_++];
         if (!l.tiles) return RSD_OK;
         const int pi = prof_begin(h, K_GEMM_TC16, st);
         const unsigned grid = (unsigned)std::min(l.tiles, h.num_sms);
-        if (l.solve) k_gemm_f64_tc<true><<<grid, F64_THREADS, F64_SMEM, st>>>(d_tasks + l.off, l.n, l.tiles, h.d_err);
-        else k_gemm_f64_tc<false><<<grid, F64_THREADS, F64_SMEM, st>>>(d_tasks + l.off, l.n, l.tiles, h.d_err);
+        kern[l.few][l.solve]<<<grid, F64_THREADS, smem[l.few], st>>>(d_tasks + l.off, l.n, l.tiles, h.d_err);
         count_launch();
         prof_end(h, pi, l.flops, l.bytes, st);
         RSD_CUDA_TRY(cudaGetLastError());
@@ -763,8 +807,12 @@ int factor_level_f64_tc(Handle& h, int li) {
                 if (!rows) return RSD_OK;
                 const int pi = prof_begin(h, K_COPY16, st);
                 if (x) k_split_x<<<dim3((unsigned)((rows + 15) / 16), (unsigned)g.nf, (unsigned)sides), 256, 0, st>>>(d_fr, d_wk + (size_t)g.f0 * sides, k, K0, h.d_err, h.d_front_bad);
-                else k_split_a<<<dim3((unsigned)((rows + SA_ROWS - 1) / SA_ROWS + NB / SA_ROWS), (unsigned)g.nf, (unsigned)sides), 256, 0, st>>>(
-                         d_fr, d_wk + (size_t)g.f0 * sides, k, (rows + SA_ROWS - 1) / SA_ROWS, h.d_err, h.d_front_bad);
+                else {
+                    // 64 rows a CTA share the load of s_j; with few CTAs 16, for the shorter chain
+                    const int nr = (rows + 63) / 64 * g.nf * sides > h.num_sms ? 64 : 16, na = (rows + nr - 1) / nr;
+                    k_split_a<<<dim3((unsigned)(na + NB / nr), (unsigned)g.nf, (unsigned)sides), 256, 0, st>>>(
+                        d_fr, d_wk + (size_t)g.f0 * sides, k, na, nr, h.d_err, h.d_front_bad);
+                }
                 count_launch();
                 prof_end(h, pi, 0.0, bytes, st);
                 RSD_CUDA_TRY(cudaGetLastError());
