@@ -3,7 +3,7 @@
 //
 // The FP64 pipe bounds it: an SM retires 1.65 FP64 FMAs per clock and a warp's FMA takes
 // 65 clocks, so the block's 0.7M FMAs are over 200 us on one SM whatever the schedule, and
-// a level near the root has few fronts.  A cluster of CL CTAs therefore takes one front:
+// a level near the root has few fronts.  A cluster of CL (up to 16) CTAs therefore takes one front:
 //   - the 32 x 32 diagonal sub-block is factored and inverted by every CTA (redundantly:
 //     cheaper than handing it on), one column per step, lane = row, the columns spread
 //     over the eight warps;
@@ -13,9 +13,10 @@
 //     every CTA the same way;
 //   - the inverse is spread by columns (four adjacent ones to a CTA), which needs no
 //     exchange: X_JK = -X_JJ sum_M L_JM X_MK.
-// Measured: one 128-block per launch 0.57 ms before (one CTA, the block in registers, two
+// Measured: one 128-block per launch 0.57 ms at first (one CTA, the block in registers, two
 // barriers and a reciprocal square root per column for the factor and again for the
-// inverse), 0.14 ms on 8 CTAs; 64 fronts on 2 CTAs each 0.19 ms.
+// inverse), 0.16 on 8 CTAs scaling column by column, 0.13 on 16 with the unscaled chain of
+// chol_inv32 (four times 22 us of it in the 32 x 32 blocks); 64 fronts on 2 CTAs each 0.25 ms.
 // L fills the lower triangle of a 128 x 129 array, X (transposed, one column further
 // right) its upper triangle.
 #include <algorithm>
@@ -30,15 +31,14 @@ constexpr int DT = 256, DW = DT / 32;    // threads, warps
 constexpr int SBK = 32;                  // sub-block
 constexpr int LD = NB + 1;               // row stride of L / X (odd: lanes over rows hit distinct banks)
 constexpr int SLD = SBK + 1;
-constexpr size_t DIAG_SMEM = sizeof(double) * ((size_t)NB * LD + 2 * SBK * SLD + 2 * SBK + 2);
+constexpr size_t DIAG_SMEM = sizeof(double) * ((size_t)NB * LD + 2 * SBK * SLD + 5 * SBK);
 
 __device__ __forceinline__ void cl_st_f64(uint32_t a, double v) {
     asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
 }
 
 // 1 / sqrt(d) for d > 0: an FP32 estimate y of the reduced argument (2^-21) and one
-// third-order Householder step, y + y e (1/2 + 3/8 e) with e = 1 - d y^2: four FMAs deep on the
-// chain from pivot to pivot (about 320 clocks; rsqrt() takes 358, 1 / sqrt(d) 960).
+// third-order Householder step, y + y e (1/2 + 3/8 e) with e = 1 - d y^2.
 __device__ __forceinline__ double rsqrt_chain(double d) {
     const long long b = __double_as_longlong(d);
     const int ex = (int)(b >> 52) - 1023;
@@ -51,11 +51,33 @@ __device__ __forceinline__ double rsqrt_chain(double d) {
     return fma(y * e, fma(0.375, e, 0.5), y);
 }
 
+// 1 / d for finite d != 0: an FP32 estimate y (2^-22) and y + y (e + e^2), e = 1 - d y: three
+// FMAs deep on the chain from pivot to pivot (about 260 clocks; 1.0 / d takes 360).
+__device__ __forceinline__ double rcp_chain(double d) {
+    const long long b = __double_as_longlong(d);
+    const int ex = (int)((b >> 52) & 0x7ff) - 1023;
+    if (ex < -1000 || ex > 1000) return 1.0 / d;
+    const float f = __int_as_float((127 << 23) | (int)((b >> 29) & 0x7fffff));      // |d| = f 2^ex, f in [1, 2)
+    float yf;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(yf) : "f"(f));
+    const int yb = __float_as_int(yf);
+    const double y = __longlong_as_double((b & 0x8000000000000000ll) | ((long long)((yb >> 23) - 127 + 1023 - ex) << 52) |
+                                          ((long long)(yb & 0x7fffff) << 29));
+    const double e = fma(-d, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+
 // Cholesky of the 32 x 32 block in D (lower part) and its inverse, all eight warps: thread
 // (lane, warp) holds row `lane` of columns warp + 8 q of both.  On return D holds L and Y
 // the inverse (both with zeros above the diagonal).  Returns 1 on a pivot that is not
 // positive or not finite (replaced by 1; 1 / inf would hide an infinite pivot behind zeros).
-__device__ int chol_inv32(double* __restrict__ D, double* __restrict__ Y, double* __restrict__ col, double* __restrict__ dinv,
+// The columns are eliminated unscaled, D = L' diag(d) L'^T with L' unit lower: the chain
+// from pivot to pivot is one FMA, a reciprocal and a product, every other entry takes one FMA a
+// step (of D right of the pivot, of L'^-1 left of it), and the square roots come at the end, all 32
+// at once.  The warp that owns column j + 1 updates it first and publishes it while the
+// others are still at step j: 22 us a block where scaling by 1 / sqrt(d) step by step took 27
+// (its own FMAs wait for those of the other warp of its scheduler).
+__device__ int chol_inv32(double* __restrict__ D, double* __restrict__ Y, double* __restrict__ buf, double* __restrict__ piv,
                           int lane, int warp) {
     double a[4], y[4];
 #pragma unroll
@@ -65,43 +87,53 @@ __device__ int chol_inv32(double* __restrict__ D, double* __restrict__ Y, double
         y[q] = c == lane ? 1.0 : 0.0;
     }
     int bad = 0;
+    // column j (updated by all before it): pivot, then the column and L'_j to buffer j & 1
+    auto publish = [&](double& aj, int j) {
+        double d = __shfl_sync(0xffffffffu, aj, j);
+        if (!(d > 0.0 && d <= 1.7976931348623157e308)) { bad = 1; d = 1.0; }
+        double* b = buf + (j & 1) * 2 * SBK;
+        b[lane] = aj;
+        b[SBK + lane] = lane > j ? aj * rcp_chain(d) : 0.0;
+        if (lane == j) { aj = d; piv[j] = d; }
+    };
+    if (warp == 0) publish(a[0], 0);
 #pragma unroll
     for (int jb = 0; jb < 4; ++jb) {
 #pragma unroll 1
         for (int jj = 0; jj < DW; ++jj) {
             const int j = DW * jb + jj;
-            double* cj = col + (j & 1) * SBK;
-            if (warp == jj) {
-                double d = __shfl_sync(0xffffffffu, a[jb], j);
-                if (!(d > 0.0 && d <= 1.7976931348623157e308)) { bad = 1; d = 1.0; }
-                const double inv = rsqrt_chain(d);
-                const double l = lane > j ? a[jb] * inv : (lane == j ? d * inv : 0.0);
-                a[jb] = l;
-                cj[lane] = l;
-                if (lane == 0) dinv[j & 1] = inv;
-            }
             __syncthreads();
-            const double li = cj[lane];
-            // the next pivot's column first, then the rest right of column j
+            const double* cj = buf + (j & 1) * 2 * SBK;
+            const double li = cj[SBK + lane];
+            // the next pivot's column first
+            const bool wrap = jj == DW - 1;
+            if (!wrap && warp == jj + 1) {
+                a[jb] -= li * cj[j + 1];
+                publish(a[jb], j + 1);
+            }
+            if (jb < 3 && wrap && warp == 0) {
+                a[jb < 3 ? jb + 1 : 3] -= li * cj[j + 1];
+                publish(a[jb < 3 ? jb + 1 : 3], j + 1);
+            }
 #pragma unroll
             for (int q = jb; q < 4; ++q)
-                if (warp + DW * q > j) a[q] -= li * cj[warp + DW * q];
-            // row j of the inverse, then the rows below it
-            const double inv = dinv[j & 1];
+                if (warp + DW * q > j + 1) a[q] -= li * cj[warp + DW * q];
 #pragma unroll
             for (int q = 0; q <= jb; ++q) {
                 if (warp + DW * q > j) continue;
-                const double xj = __shfl_sync(0xffffffffu, y[q], j) * inv;
-                y[q] = lane == j ? xj : (lane > j ? y[q] - li * xj : y[q]);
+                y[q] -= li * __shfl_sync(0xffffffffu, y[q], j);          // (li = 0 on rows <= j)
             }
         }
     }
     __syncthreads();
+    const double inv = rsqrt_chain(piv[lane]);
+    if (warp == 0) buf[lane] = inv;
+    __syncthreads();
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
         const int c = warp + DW * q;
-        D[lane * SLD + c] = c <= lane ? a[q] : 0.0;
-        Y[lane * SLD + c] = c <= lane ? y[q] : 0.0;
+        D[lane * SLD + c] = c <= lane ? a[q] * buf[c] : 0.0;
+        Y[lane * SLD + c] = c <= lane ? y[q] * inv : 0.0;
     }
     __syncthreads();
     return bad;
@@ -119,8 +151,8 @@ __global__ void __launch_bounds__(DT, 1) k_chol_diag_f64(const FrontDesc* __rest
     double* Lf = (double*)diag_smem;             // NB x LD
     double* D = Lf + NB * LD;                    // 32 x SLD: the diagonal sub-block
     double* Y = D + SBK * SLD;                   // 32 x SLD: its inverse
-    double* col = Y + SBK * SLD;                 // two columns
-    double* dinv = col + 2 * SBK;                // two reciprocal pivots
+    double* buf = Y + SBK * SLD;                 // two columns, raw and scaled
+    double* piv = buf + 4 * SBK;
     const FrontDesc f = fronts[blockIdx.x / CL];
     if (f.s <= k) return;                        // the whole cluster
     const int w = min(NB, f.s - k), nJ = (w + SBK - 1) / SBK;
@@ -140,7 +172,7 @@ __global__ void __launch_bounds__(DT, 1) k_chol_diag_f64(const FrontDesc* __rest
     for (int J = 0; J < nJ; ++J) {
         const int o = SBK * J, below = SBK * (J + 1), rows = nJ * SBK;
         if (J > 0) cluster_or_cta_sync<CL>();          // the sub-block's rows are in D
-        bad |= chol_inv32(D, Y, col, dinv, lane, warp);
+        bad |= chol_inv32(D, Y, buf, piv, lane, warp);
         // L_JJ out (one CTA), X_JJ into the columns this CTA owns
         if (rank == J % CL)
             for (int e = tid; e < SBK * SBK; e += DT) {
@@ -251,8 +283,10 @@ __global__ void __launch_bounds__(DT, 1) k_chol_diag_f64(const FrontDesc* __rest
 // LU and the inverses of L and U^T of the 32 x 32 block at A (row stride LD), all eight warps,
 // thread (lane, warp) holding row `lane` of columns warp + 8 q; A keeps L and U, YL = L^-1, YW =
 // (U^T)^-1 (lower, zeros above).  Returns 1 on a pivot that is zero or not finite (replaced by 1).
-__device__ int lu_inv32(double* __restrict__ A, double* __restrict__ YL, double* __restrict__ YW, double* __restrict__ col,
-                        double* __restrict__ rowu, double* __restrict__ dinv, int lane, int warp) {
+// As in chol_inv32 the next pivot's column goes ahead, and (U^T)^-1 is formed unscaled
+// (with U'_ji = u_ji / u_jj) and its rows divided by the pivots at the end.
+__device__ int lu_inv32(double* __restrict__ A, double* __restrict__ YL, double* __restrict__ YW, double* __restrict__ buf,
+                        double* __restrict__ rcp, int lane, int warp) {
     double a[4], yl[4], yw[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -261,42 +295,57 @@ __device__ int lu_inv32(double* __restrict__ A, double* __restrict__ YL, double*
         yl[q] = yw[q] = c == lane ? 1.0 : 0.0;
     }
     int bad = 0;
+    // column j (updated by all before it): pivot, then L_j to buffer j & 1
+    auto publish = [&](double& aj, int j) {
+        double d = __shfl_sync(0xffffffffu, aj, j);
+        if (!(d != 0.0) || !(fabs(d) <= 1.7976931348623157e308)) {
+            bad = 1;
+            d = 1.0;
+            if (lane == j) aj = 1.0;
+        }
+        const double r = rcp_chain(d);
+        if (lane > j) aj *= r;
+        buf[(j & 1) * 2 * SBK + lane] = lane > j ? aj : 0.0;
+        if (lane == j) rcp[j] = r;
+    };
+    if (warp == 0) publish(a[0], 0);
+    if (lane == 0) {                                  // row 0 of U
+#pragma unroll
+        for (int q = 0; q < 4; ++q) buf[SBK + warp + DW * q] = a[q];
+    }
 #pragma unroll
     for (int jb = 0; jb < 4; ++jb) {
 #pragma unroll 1
         for (int jj = 0; jj < DW; ++jj) {
             const int j = DW * jb + jj;
-            double* cj = col + (j & 1) * SBK;
-            double* rj = rowu + (j & 1) * SBK;
-            if (warp == jj) {
-                double d = __shfl_sync(0xffffffffu, a[jb], j);
-                if (!(d != 0.0) || !(fabs(d) <= 1.7976931348623157e308)) {
-                    bad = 1;
-                    d = 1.0;
-                    if (lane == j) a[jb] = 1.0;
-                }
-                const double inv = 1.0 / d;
-                if (lane > j) a[jb] *= inv;
-                cj[lane] = lane > j ? a[jb] : 0.0;
-                if (lane == 0) dinv[j & 1] = inv;
-            }
-            if (lane == j) {
-#pragma unroll
-                for (int q = jb; q < 4; ++q) rj[warp + DW * q] = a[q];
-            }
             __syncthreads();
+            const double* cj = buf + (j & 1) * 2 * SBK;      // L_j, row j of U
+            const double* rj = cj + SBK;
             const double li = cj[lane];
+            const bool wrap = jj == DW - 1;
+            if (!wrap && warp == jj + 1) {
+                a[jb] -= li * rj[j + 1];
+                publish(a[jb], j + 1);
+            }
+            if (jb < 3 && wrap && warp == 0) {
+                a[jb < 3 ? jb + 1 : 3] -= li * rj[j + 1];
+                publish(a[jb < 3 ? jb + 1 : 3], j + 1);
+            }
 #pragma unroll
             for (int q = jb; q < 4; ++q)
-                if (warp + DW * q > j) a[q] -= li * rj[warp + DW * q];
-            const double inv = dinv[j & 1], ui = lane > j ? rj[lane] : 0.0;
+                if (warp + DW * q > j + 1) a[q] -= li * rj[warp + DW * q];
+            if (lane == j + 1) {                             // row j + 1 of U is final
+                double* rn = buf + ((j + 1) & 1) * 2 * SBK + SBK;
+#pragma unroll
+                for (int q = jb; q < 4; ++q) rn[warp + DW * q] = a[q];
+            }
+            const double ui = lane > j ? rj[lane] * rcp[j] : 0.0;
 #pragma unroll
             for (int q = 0; q <= jb; ++q) {
                 if (warp + DW * q > j) continue;
-                const double xl = __shfl_sync(0xffffffffu, yl[q], j);
-                const double xw = __shfl_sync(0xffffffffu, yw[q], j) * inv;
-                yl[q] = lane > j ? yl[q] - li * xl : yl[q];
-                yw[q] = lane == j ? xw : (lane > j ? yw[q] - ui * xw : yw[q]);
+                const double xl = __shfl_sync(0xffffffffu, yl[q], j), xw = __shfl_sync(0xffffffffu, yw[q], j);
+                yl[q] -= li * xl;
+                yw[q] -= ui * xw;
             }
         }
     }
@@ -306,13 +355,13 @@ __device__ int lu_inv32(double* __restrict__ A, double* __restrict__ YL, double*
         const int c = warp + DW * q;
         A[lane * LD + c] = a[q];
         YL[lane * SLD + c] = c <= lane ? yl[q] : 0.0;
-        YW[lane * SLD + c] = c <= lane ? yw[q] : 0.0;
+        YW[lane * SLD + c] = c <= lane ? yw[q] * rcp[lane] : 0.0;
     }
     __syncthreads();
     return bad;
 }
 
-constexpr size_t LU_SMEM = sizeof(double) * ((size_t)NB * LD + 2 * SBK * SLD + 4 * SBK + 2);
+constexpr size_t LU_SMEM = sizeof(double) * ((size_t)NB * LD + 2 * SBK * SLD + 5 * SBK);
 
 template <int CL>
 __global__ void __launch_bounds__(DT, 1) k_lu_diag_f64(const FrontDesc* __restrict__ fronts, int k, int* __restrict__ err,
@@ -321,9 +370,8 @@ __global__ void __launch_bounds__(DT, 1) k_lu_diag_f64(const FrontDesc* __restri
     double* A = (double*)diag_smem;              // NB x LD: L below the diagonal, U on and above it
     double* YL = A + NB * LD;                    // 32 x SLD: L_JJ^-1
     double* YW = YL + SBK * SLD;                 // 32 x SLD: (U_JJ^T)^-1
-    double* col = YW + SBK * SLD;
-    double* rowu = col + 2 * SBK;
-    double* dinv = rowu + 2 * SBK;
+    double* buf = YW + SBK * SLD;                // two columns of L and rows of U
+    double* rcp = buf + 4 * SBK;                 // reciprocal pivots
     const FrontDesc f = fronts[blockIdx.x / CL];
     if (f.s <= k) return;                        // the whole cluster
     const int w = min(NB, f.s - k), nJ = (w + SBK - 1) / SBK, rows = nJ * SBK;
@@ -344,7 +392,7 @@ __global__ void __launch_bounds__(DT, 1) k_lu_diag_f64(const FrontDesc* __restri
     for (int J = 0; J < nJ; ++J) {
         const int o = SBK * J, below = SBK * (J + 1);
         if (J > 0) cluster_or_cta_sync<CL>();          // the block row is here
-        bad |= lu_inv32(A + o * LD + o, YL, YW, col, rowu, dinv, lane, warp);
+        bad |= lu_inv32(A + o * LD + o, YL, YW, buf, rcp, lane, warp);
         for (int e = tid; e < SBK * SBK; e += DT) {
             const int c = e % SBK, r = e / SBK;
             if (((o + c) >> 2) % CL == rank) {
@@ -449,6 +497,7 @@ using DiagKernel = void (*)(const FrontDesc*, int, int*, int*);
 
 int launch_cl(DiagKernel kern, int CL, size_t smem, const FrontDesc* d_fronts, int nf, int k, int* err, int* bad_front, cudaStream_t st) {
     RSD_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (CL > 8) RSD_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(nf * CL));
     cfg.blockDim = dim3(DT);
@@ -467,6 +516,36 @@ int launch_cl(DiagKernel kern, int CL, size_t smem, const FrontDesc* d_fronts, i
 
 }  // namespace
 
+// How many clusters of 16 (more than the portable 8) the current device holds at once; 0
+// where it takes none.
+static int wide_clusters(DiagKernel kern, size_t smem) {
+    static int known[64][2] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) { cudaGetLastError(); return 0; }
+    int& n = known[dev][smem == LU_SMEM];
+    if (!n) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(16 * 16);
+        cfg.blockDim = dim3(DT);
+        cfg.dynamicSmemBytes = smem;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = 16;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int m = 0;
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+            cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&m, (void*)kern, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            m = 0;
+        }
+        n = m + 1;
+    }
+    return n - 1;
+}
+
 // The largest cluster that still gives every front with rows past k SMs of its own: the
 // FP64 pipes it adds are worth more than anything else to a lone block (see above), and
 // past one wave a larger cluster only queues.
@@ -484,10 +563,13 @@ int launch_diag_f64(Handle& h, int li, int f0, int nf, int k, cudaStream_t st) {
     if (!alive) return RSD_OK;
     const FrontDesc* fr = L.d_fronts + f0;
     const int pi = prof_begin(h, K_POTRF, st);
-    static constexpr DiagKernel chol[4] = {k_chol_diag_f64<1>, k_chol_diag_f64<2>, k_chol_diag_f64<4>, k_chol_diag_f64<8>};
-    static constexpr DiagKernel lu[4] = {k_lu_diag_f64<1>, k_lu_diag_f64<2>, k_lu_diag_f64<4>, k_lu_diag_f64<8>};
-    const int lg = alive * 8 <= h.num_sms ? 3 : alive * 4 <= h.num_sms ? 2 : alive * 2 <= h.num_sms ? 1 : 0;
-    const int rc = launch_cl((h.lu ? lu : chol)[lg], 1 << lg, h.lu ? LU_SMEM : DIAG_SMEM, fr, nf, k, h.d_err, h.d_front_bad, st);
+    static constexpr DiagKernel kern[2][5] = {
+        {k_chol_diag_f64<1>, k_chol_diag_f64<2>, k_chol_diag_f64<4>, k_chol_diag_f64<8>, k_chol_diag_f64<16>},
+        {k_lu_diag_f64<1>, k_lu_diag_f64<2>, k_lu_diag_f64<4>, k_lu_diag_f64<8>, k_lu_diag_f64<16>}};
+    const size_t smem = h.lu ? LU_SMEM : DIAG_SMEM;
+    int lg = alive * 8 <= h.num_sms ? 3 : alive * 4 <= h.num_sms ? 2 : alive * 2 <= h.num_sms ? 1 : 0;
+    if (lg == 3 && alive <= wide_clusters(kern[h.lu][4], smem)) lg = 4;
+    const int rc = launch_cl(kern[h.lu][lg], 1 << lg, smem, fr, nf, k, h.d_err, h.d_front_bad, st);
     prof_end(h, pi, flops, bytes, st);
     return rc;
 }
