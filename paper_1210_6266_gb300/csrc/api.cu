@@ -1019,6 +1019,7 @@ static int build_handle(Handle& h, Analysis& a, const int64_t* rowptr, const int
         acc(sizeof(double) * gm_maxS);
         acc(sizeof(double) * gm_maxS * (h.gamma + 1));
         acc(sizeof(double) * gm_maxIf * (h.gamma + 1) * h.gamma);
+        acc(sizeof(double) * gm_maxIf * h.gamma * h.gamma);
         acc(sizeof(double) * gm_maxIf);
         acc(sizeof(int) * gm_maxIf);
         acc(sizeof(double) * gm_maxK);
@@ -1028,7 +1029,8 @@ static int build_handle(Handle& h, Analysis& a, const int64_t* rowptr, const int
     const bool fg = h.krylov == RSD_KRYLOV_FGMRES;
     const int m = h.restart;
     if (fg && m > 64) { set_last_error("FGMRES restart > 64"); return RSD_ERR_ARG; }
-    const size_t o_fg = fg ? take(sizeof(double) * ((size_t)(2 * m + 1) * a.n + (size_t)(m + 1) * m + m + 64)) : 0;
+    const size_t o_fg = fg ? take(sizeof(double) * ((size_t)(2 * m + 1) * a.n + (size_t)(m + 1) * m + m + 64 +
+                                                   (size_t)(m + 1) * (m + 1) + (size_t)2 * (m + 1) * FG_BLOCKS)) : 0;
     const size_t o_child = take(sizeof(int) * a.n_nodes);
     const size_t o_vecs = take(sizeof(double) * 4 * (size_t)a.n + 4096);
     const size_t o_partial = take(sizeof(double) * 2048);
@@ -1311,6 +1313,7 @@ static int build_handle(Handle& h, Analysis& a, const int64_t* rowptr, const int
         h.d_gm_w = dput(gm_maxS);
         h.d_gm_V = dput(gm_maxS * (h.gamma + 1));
         h.d_gm_H = dput(gm_maxIf * (h.gamma + 1) * h.gamma);
+        h.d_gm_G = dput(gm_maxIf * h.gamma * h.gamma);
         h.d_gm_beta = dput(gm_maxIf);
         h.d_gm_kused = (int*)cur;
         cur += align_up(sizeof(int) * std::max<size_t>(gm_maxIf, 1), 256);
@@ -1322,6 +1325,8 @@ static int build_handle(Handle& h, Analysis& a, const int64_t* rowptr, const int
         h.d_fg_Z = h.d_fg_V + (size_t)(m + 1) * a.n;
         h.d_fg_H = h.d_fg_Z + (size_t)m * a.n;
         h.d_fg_y = h.d_fg_H + (size_t)(m + 1) * m;
+        h.d_fg_G = h.d_fg_y + m + 64;
+        h.d_fg_part = h.d_fg_G + (size_t)(m + 1) * (m + 1);
         if (!h.h_fg && cudaMallocHost((void**)&h.h_fg, sizeof(double) * 256) != cudaSuccess) {
             cudaGetLastError();
             return RSD_ERR_NOMEM;

@@ -103,20 +103,93 @@ __global__ void k_residual(int n, const int64_t* __restrict__ rowptr, const int*
     if (row < n && sub == 0) r[row] = f[row] - s;
 }
 
-// One modified Gram-Schmidt step of FGMRES, fused with the next inner product:
-// w -= h v (h read from the device, skipped when v is null), then per-block partial sums
-// of w . next (next = w gives ||w||^2 after the update).
-__global__ void k_mgs_step(int64_t n, const double* __restrict__ hval, const double* __restrict__ v,
-                           double* __restrict__ w, const double* __restrict__ next, double* __restrict__ partial) {
-    const double hv = v ? *hval : 0.0;
+// Modified Gram-Schmidt of FGMRES step j with two sums in place of j + 2: h_q = <w -
+// sum_{i<q} h_i v_i, v_q> = r_q - sum_{i<q} G_qi h_i with r_q = <w, v_q> and the Gram entries
+// G_qi = <v_q, v_i> (as in the inner GMRES, paper_gamma.cu).  This kernel: per-block partial
+// sums of r_q (q <= j, to partial[q FG_BLOCKS + block]) and G_jq (q < j, to slot
+// stride + q), eight of each per pass over the block's entries.
+constexpr int FG_QB = 8;
+__global__ void __launch_bounds__(RT) k_fg_dots(int64_t n, int j, const double* __restrict__ V, const double* __restrict__ w,
+                                                double* __restrict__ partial, int stride) {
+    __shared__ double s_red[RT / 32][2 * FG_QB];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const double* vj = V + (int64_t)j * n;
+    for (int q0 = 0; q0 <= j; q0 += FG_QB) {
+        const int nq = min(FG_QB, j + 1 - q0);
+        double a[FG_QB], b[FG_QB];
+#pragma unroll
+        for (int q = 0; q < FG_QB; ++q) a[q] = b[q] = 0;
+        for (int64_t i = blockIdx.x * (int64_t)RT + threadIdx.x; i < n; i += (int64_t)gridDim.x * RT) {
+            const double wi = w[i], vi = vj[i];
+#pragma unroll
+            for (int q = 0; q < FG_QB; ++q)
+                if (q < nq) {
+                    const double v = V[(int64_t)(q0 + q) * n + i];
+                    a[q] += wi * v;
+                    b[q] += vi * v;
+                }
+        }
+#pragma unroll
+        for (int q = 0; q < FG_QB; ++q) {
+            a[q] = warp_sum(a[q]);
+            b[q] = warp_sum(b[q]);
+            if (lane == 0) { s_red[warp][q] = a[q]; s_red[warp][FG_QB + q] = b[q]; }
+        }
+        __syncthreads();
+        if (threadIdx.x < 2 * FG_QB) {
+            const int q = threadIdx.x % FG_QB;
+            double t = 0;
+#pragma unroll
+            for (int k = 0; k < RT / 32; ++k) t += s_red[k][threadIdx.x];
+            if (q < nq) partial[(int64_t)((threadIdx.x / FG_QB) * stride + q0 + q) * gridDim.x + blockIdx.x] = t;
+        }
+        __syncthreads();
+    }
+}
+
+// The sums of k_fg_dots (a warp each) and the forward substitution: h_q to hc[q], row j of
+// the Gram entries to G (row stride `stride`).  One CTA.
+__global__ void __launch_bounds__(1024) k_fg_solve(int j, const double* __restrict__ partial, int nblocks, int stride,
+                                                   double* __restrict__ G, double* __restrict__ hc) {
+    __shared__ double s_r[64], s_g[64], s_G[64][65];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int e = threadIdx.x; e < j * j; e += blockDim.x) s_G[e / j][e % j] = G[(e / j) * stride + e % j];
+    for (int v = warp; v <= 2 * j; v += blockDim.x >> 5) {      // r_0 .. r_j, then G_j0 .. G_j,j-1
+        const int slot = v <= j ? v : stride + v - j - 1;
+        double t = 0;
+        for (int k = lane; k < nblocks; k += 32) t += partial[(int64_t)slot * nblocks + k];
+        t = warp_sum(t);
+        if (lane == 0) {
+            if (v <= j) s_r[v] = t;
+            else { s_g[v - j - 1] = t; G[j * stride + v - j - 1] = t; }
+        }
+    }
+    __syncthreads();
+    if (warp) return;
+    double r0 = lane <= j ? s_r[lane] : 0.0, r1 = lane + 32 <= j ? s_r[lane + 32] : 0.0;
+    for (int i = 0; i < j; ++i) {
+        const double hi = __shfl_sync(0xffffffffu, i < 32 ? r0 : r1, i & 31);
+        const int q0 = lane, q1 = lane + 32;
+        if (q0 > i && q0 <= j) r0 -= (q0 < j ? s_G[q0][i] : s_g[i]) * hi;
+        if (q1 > i && q1 <= j) r1 -= (q1 < j ? s_G[q1][i] : s_g[i]) * hi;
+    }
+    if (lane <= j) hc[lane] = r0;
+    if (lane + 32 <= j) hc[lane + 32] = r1;
+}
+
+// w -= sum_q h_q v_q, q <= j, and per-block partial sums of ||w||^2.
+__global__ void __launch_bounds__(RT) k_fg_orth(int64_t n, int j, const double* __restrict__ hc, const double* __restrict__ V,
+                                                double* __restrict__ w, double* __restrict__ partial) {
+    __shared__ double s_h[64];
+    if (threadIdx.x <= j) s_h[threadIdx.x] = hc[threadIdx.x];
+    __syncthreads();
     double s = 0;
     for (int64_t i = blockIdx.x * (int64_t)RT + threadIdx.x; i < n; i += (int64_t)gridDim.x * RT) {
         double wi = w[i];
-        if (v) {
-            wi -= hv * v[i];
-            w[i] = wi;
-        }
-        s += wi * (next == w ? wi : next[i]);
+#pragma unroll 4
+        for (int q = 0; q <= j; ++q) wi -= s_h[q] * V[(int64_t)q * n + i];
+        w[i] = wi;
+        s += wi * wi;
     }
     s = block_sum(s);
     if (threadIdx.x == 0) partial[blockIdx.x] = s;
@@ -265,17 +338,14 @@ int fgmres(Handle& h, const double* f, double* x, double tol, rsd_stats* st) {
             RSD_TRY(spmv(h, zj, w));
             double* hc = Hd + (int64_t)j * (m + 1);
             const int pk = prof_begin(h, K_KRYLOV);
-            for (int i = 0; i <= j + 1; ++i) {
-                // step i: subtract h_{i-1,j} v_{i-1} (i > 0), then w . v_i (or ||w||^2 at i = j + 1)
-                const double* vprev = i > 0 ? V + (int64_t)(i - 1) * n : nullptr;
-                const double* nxt = i <= j ? V + (int64_t)i * n : w;
-                k_mgs_step<<<RED_BLOCKS, RT, 0, h.stream>>>(n, i > 0 ? hc + i - 1 : nullptr, vprev, w, nxt, h.d_partial);
-                k_reduce_final<<<1, RT, 0, h.stream>>>(h.d_partial, RED_BLOCKS, i <= j ? hc + i : h.d_scal + 7);
-                count_launch(2);
-            }
+            k_fg_dots<<<FG_BLOCKS, RT, 0, h.stream>>>(n, j, V, w, h.d_fg_part, m + 1);
+            k_fg_solve<<<1, 1024, 0, h.stream>>>(j, h.d_fg_part, FG_BLOCKS, m + 1, h.d_fg_G, hc);
+            k_fg_orth<<<RED_BLOCKS, RT, 0, h.stream>>>(n, j, hc, V, w, h.d_partial);
+            k_reduce_final<<<1, RT, 0, h.stream>>>(h.d_partial, RED_BLOCKS, h.d_scal + 7);
+            count_launch(4);
             k_scale_by_norm<<<RED_BLOCKS, RT, 0, h.stream>>>(n, h.d_scal + 7, w, V + (int64_t)(j + 1) * n, hc + j + 1);
             count_launch();
-            prof_end(h, pk, (4.0 * (j + 2)) * n, (24.0 * (j + 2) + 16.0) * n);
+            prof_end(h, pk, (6.0 * (j + 1) + 2.0) * n, (16.0 * (j + 1) + 40.0) * n);
             RSD_CUDA_TRY(cudaGetLastError());
             RSD_CUDA_TRY(cudaMemcpyAsync(h.h_fg, hc, sizeof(double) * (j + 2), cudaMemcpyDeviceToHost, h.stream));
             RSD_CUDA_TRY(cudaStreamSynchronize(h.stream));

@@ -83,6 +83,24 @@ __device__ __forceinline__ void smv_load(const void* p, int64_t off, T (&o)[SmvE
     }
 }
 
+// the same from a 16-byte load already made
+template <typename T, bool H16>
+__device__ __forceinline__ void smv_unpack(const uint4& u, T (&o)[SmvElems<T, H16>::W]) {
+    if constexpr (H16) {
+        const __half2* h = reinterpret_cast<const __half2*>(&u);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const float2 f = __half22float2(h[k]);
+            o[2 * k] = f.x;
+            o[2 * k + 1] = f.y;
+        }
+    } else {
+        const T* e = reinterpret_cast<const T*>(&u);
+#pragma unroll
+        for (int k = 0; k < SmvElems<T, H16>::W; ++k) o[k] = e[k];
+    }
+}
+
 // t_l = X_l[R_l]^T x for every leaf with rows coupled to the level; one CTA per (leaf, 32 x W
 // columns), W columns per lane read with one 16-byte load per row.  The rows' offsets and x
 // values are staged in shared memory 256 at a time; the eight warps take every eighth row
@@ -263,15 +281,132 @@ __global__ void __launch_bounds__(256) k_smv_iface(int S, const int* __restrict_
     }
 }
 
+// Both products of a leaf in one CTA (small leaves): t_l = X_l[R]^T x in shared memory, then
+// yl_k = X_l[row_k] . t_l.  A thread takes one 16-byte chunk of columns and every
+// `groups`-th row for t_l, the groups' partial sums being added in order; a warp takes four rows at a time
+// for yl.  The leaf's rows come from L2 once and, mostly, from L1 the second time.
+template <typename T, bool H16>
+__global__ void __launch_bounds__(256) k_smv_both(const FrontDesc* __restrict__ ty, const FrontDesc* __restrict__ tx,
+                                                  const int* __restrict__ cl_ptr, const int* __restrict__ cl_row,
+                                                  const int* __restrict__ cl_pos, int max_s, const double* __restrict__ x,
+                                                  double* __restrict__ yl) {
+    constexpr int W = SmvElems<T, H16>::W, R = 4;
+    __shared__ int s_row[256];
+    __shared__ T s_x[256];
+    extern __shared__ __align__(16) unsigned char smv_smem[];
+    T* s_t = (T*)smv_smem;                             // max_s rounded up to W
+    T* s_red = s_t + (max_s + W - 1) / W * W;          // groups x (nch W)
+    const int l = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int k0 = cl_ptr[l], k1 = cl_ptr[l + 1];
+    if (k0 == k1) return;
+    const int s = ty[l].s, ldp = ty[l].ldp;
+    const void* Y = H16 ? (const void*)((const __half*)ty[l].P16 + (int64_t)s * ldp) : (const void*)((const T*)ty[l].P + (int64_t)s * ldp);
+    const void* X = H16 ? (const void*)((const __half*)tx[l].P16 + (int64_t)s * ldp) : (const void*)((const T*)tx[l].P + (int64_t)s * ldp);
+    const float* ri = H16 ? ty[l].ri + s : nullptr;
+    const int nch = (s + W - 1) / W, groups = 256 / nch;          // (nch <= 256)
+    const int ch = tid % nch, g = tid / nch;
+    T acc[W];
+#pragma unroll
+    for (int e = 0; e < W; ++e) acc[e] = 0;
+    for (int kb = k0; kb < k1; kb += 256) {
+        const int nb = min(256, k1 - kb);
+        __syncthreads();
+        if (tid < nb) {
+            const int row = cl_row[kb + tid];
+            s_row[tid] = row;
+            const T xv = (T)x[cl_pos[kb + tid]];
+            s_x[tid] = H16 ? xv * (T)ri[row] : xv;
+        }
+        __syncthreads();
+        if (g < groups) {
+            constexpr int U = 8;                       // rows in flight per thread
+            const char* Yc = (const char*)Y + (int64_t)ch * 16;
+            for (int q = g; q < nb; q += U * groups) {
+                uint4 v[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (q + u * groups < nb) v[u] = __ldg((const uint4*)(Yc + (int64_t)s_row[q + u * groups] * ldp * (16 / W)));
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (q + u * groups < nb) {
+                        T e[W];
+                        smv_unpack<T, H16>(v[u], e);
+                        const T xv = s_x[q + u * groups];
+#pragma unroll
+                        for (int w = 0; w < W; ++w) acc[w] += e[w] * xv;
+                    }
+            }
+        }
+    }
+    if (g < groups) {
+#pragma unroll
+        for (int e = 0; e < W; ++e) s_red[(g * nch + ch) * W + e] = acc[e];
+    }
+    __syncthreads();
+    for (int e = tid; e < nch * W; e += 256) {
+        T v = 0;
+        for (int q = 0; q < groups; ++q) v += s_red[q * nch * W + e];
+        s_t[e] = e < s ? v : (T)0;                     // (columns past s: the rows' padding is not read as data)
+    }
+    __syncthreads();
+    for (int k = k0 + warp * R; k < k1; k += 8 * R) {
+        const int nr = min(R, k1 - k);
+        int64_t off[R];
+        T d[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            off[r] = (int64_t)cl_row[k + min(r, nr - 1)] * ldp;
+            d[r] = 0;
+        }
+        for (int c0 = lane; c0 < nch; c0 += 64) {      // two chunks of each row in flight
+            uint4 v[2][R];
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+                    if (c0 + 32 * h < nch) v[h][r] = __ldg((const uint4*)((const char*)X + (off[r] + (int64_t)(c0 + 32 * h) * W) * (16 / W)));
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int c = c0 + 32 * h;
+                if (c >= nch) break;
+                T tv[W];
+#pragma unroll
+                for (int q = 0; q < W; ++q) tv[q] = s_t[c * W + q];
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    T e[W];
+                    smv_unpack<T, H16>(v[h][r], e);
+#pragma unroll
+                    for (int q = 0; q < W; ++q) d[r] += (c * W + q < s ? e[q] : (T)0) * tv[q];
+                }
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) d[r] += __shfl_xor_sync(0xffffffffu, d[r], o);
+            if (lane == 0 && r < nr) yl[k + r] = H16 ? (double)(d[r] * (T)ri[cl_row[k + r]]) : (double)d[r];
+        }
+    }
+}
+
 // The GMRES vector kernels give each interface a cluster of GC CTAs, CTA r of the cluster
 // holding the r-th contiguous chunk of the interface's entries, so a long interface (the
-// root's) is spread over GC SMs instead of one.
-constexpr int GC = 8;
+// root's) is spread over GC SMs instead of one; a level of many short ones takes smaller
+// clusters, so that its CTAs still run at once (65^3, 64 interfaces of 631 entries: 37 us
+// a step in clusters of 8, 22 in clusters of 4).
+constexpr int GC_MAX = 8;
+inline int gm_cluster(int n_if, int num_sms) {
+    int gc = GC_MAX;
+    while (gc > 1 && n_if * gc > 2 * num_sms) gc /= 2;
+    return gc;
+}
 
 struct GmChunk {
     int i, o, s, lo, hi;        // interface, its offset and size; this CTA's entries [lo, hi)
 };
 
+template <int GC>
 __device__ __forceinline__ GmChunk gm_chunk(const int* __restrict__ if_off, int i, int r) {
     GmChunk c;
     c.i = i;
@@ -287,6 +422,7 @@ __device__ __forceinline__ GmChunk gm_chunk(const int* __restrict__ if_off, int 
 // partials added in rank order by every CTA, so every thread of the cluster gets the same
 // bits.  part[] alternates between calls: a CTA rewrites part[p] only after the barrier of
 // the call in between, which every CTA passes after its reads of part[p].
+template <int GC>
 __device__ double cluster_sum_all(double v, double* red, double* part, double* tot, int& p) {
     const double b = block_sum_all(v, red);
     if (threadIdx.x == 0) part[p] = b;
@@ -302,72 +438,133 @@ __device__ double cluster_sum_all(double v, double* red, double* part, double* t
 }
 
 // v_0 = g / beta on every interface of the level (g indexed by global DOF).
+template <int GC>
 __global__ void __cluster_dims__(GC, 1, 1) __launch_bounds__(GT)
     k_gm_init(const int* __restrict__ if_off, const int* __restrict__ if_dofs, const double* __restrict__ g,
               double* __restrict__ V, double* __restrict__ beta, int* __restrict__ kused) {
     __shared__ double red[33], part[2], tot;
     const int r = (int)cl_rank();
-    const GmChunk c = gm_chunk(if_off, blockIdx.x / GC, r);
+    const GmChunk c = gm_chunk<GC>(if_off, blockIdx.x / GC, r);
     int p = 0;
     double a = 0;
     for (int e = c.lo + threadIdx.x; e < c.hi; e += blockDim.x) { const double v = g[if_dofs[c.o + e]]; a += v * v; }
-    const double b = sqrt(cluster_sum_all(a, red, part, &tot, p));
+    const double b = sqrt(cluster_sum_all<GC>(a, red, part, &tot, p));
     if (r == 0 && threadIdx.x == 0) { beta[c.i] = b; kused[c.i] = b > 0.0 ? 0 : -1; }
     const double inv = b > 0.0 ? 1.0 / b : 0.0;
     for (int e = c.lo + threadIdx.x; e < c.hi; e += blockDim.x) V[c.o + e] = g[if_dofs[c.o + e]] * inv;
     cl_sync();                                  // no CTA leaves while a peer reads its partials
 }
 
-// Arnoldi step j with modified Gram-Schmidt on w = S~ v_j, per interface: h_qj = <w, v_q>,
-// w -= h_qj v_q for q = 0..j in turn, h_{j+1,j} = ||w||, v_{j+1} = w / h_{j+1,j}.  One pass
-// over the chunk per q: the update by v_q and the product with v_{q+1} (or w's norm after
-// the last) of the updated entries.  An interface whose h_{j+1,j} falls to 1e-14 beta
-// (exact breakdown) stops with j + 1 columns; one that completes min(gamma, s) steps stops
-// with that many.
+// Sums of a[0..16) over the warp, merged as they go: lane l gets the sum of a[l >> 1].
+__device__ __forceinline__ double warp_sum16_f64(const double (&a)[16], int lane) {
+    double b[8], c[4], d[2];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) b[i] = (lane & 16 ? a[i + 8] : a[i]) + __shfl_xor_sync(0xffffffffu, lane & 16 ? a[i] : a[i + 8], 16);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) c[i] = (lane & 8 ? b[i + 4] : b[i]) + __shfl_xor_sync(0xffffffffu, lane & 8 ? b[i] : b[i + 4], 8);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) d[i] = (lane & 4 ? c[i + 2] : c[i]) + __shfl_xor_sync(0xffffffffu, lane & 4 ? c[i] : c[i + 2], 4);
+    const double e = (lane & 2 ? d[1] : d[0]) + __shfl_xor_sync(0xffffffffu, lane & 2 ? d[0] : d[1], 2);
+    return e + __shfl_xor_sync(0xffffffffu, e, 1);
+}
+
+// Arnoldi step j with modified Gram-Schmidt on w = S~ v_j, per interface (a cluster, CTA r
+// its r-th chunk): h_qj = <w - sum_{i<q} h_ij v_i, v_q>.  With the products r_q = <w, v_q>
+// and the Gram entries G_qi = <v_q, v_i> that is h_q = r_q - sum_{i<q} G_qi h_i, so one pass
+// and one cluster sum give every r_q and the new row G_j, and a forward substitution the h's,
+// where one sum per q made a step a chain of j + 2 cluster sums (Swirydowicz, Langou,
+// Ananthan, Yang, Thomas, "Low synchronization Gram-Schmidt and GMRES algorithms", 2021).
+// Then w -= sum h_q v_q, h_{j+1,j} = ||w||, v_{j+1} = w / h_{j+1,j}.
+// An interface whose h_{j+1,j} falls to 1e-14 beta (exact breakdown) stops with j + 1
+// columns; one that completes min(gamma, s) steps stops with that many.
+// (w itself stays a launch of its own: its gathers want more CTAs than the clusters have.)
+template <int GC>
 __global__ void __cluster_dims__(GC, 1, 1) __launch_bounds__(GT)
-    k_gm_mgs(int j, int gamma, int S, const int* __restrict__ if_off, double* __restrict__ w, double* __restrict__ V,
-             double* __restrict__ H, const double* __restrict__ beta, int* __restrict__ kused) {
+    k_gm_step(int j, int gamma, int S, const int* __restrict__ if_off, double* __restrict__ w, double* __restrict__ V,
+              double* __restrict__ H, double* __restrict__ G, const double* __restrict__ beta, int* __restrict__ kused) {
+    constexpr int QB = 8;                              // products of each kind per pass
     __shared__ double red[33], part[2], tot;
-    const int r = (int)cl_rank();
-    const GmChunk c = gm_chunk(if_off, blockIdx.x / GC, r);
+    __shared__ double s_red[GT / 32][2 * QB], s_part[2][2 * QB], s_rg[2][GAMMA_MAX];
+    __shared__ double s_G[GAMMA_MAX][GAMMA_MAX + 1], s_h[GAMMA_MAX];
+    const int r = (int)cl_rank(), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const GmChunk c = gm_chunk<GC>(if_off, blockIdx.x / GC, r);
     const int m = min(gamma, c.s);
     if (kused[c.i] != 0 || j >= m) return;     // the whole cluster
-    const bool lead = r == 0 && threadIdx.x == 0;
+    const bool lead = r == 0 && tid == 0;
     double* Hi = H + (int64_t)c.i * (gamma + 1) * gamma;
+    double* Gi = G + (int64_t)c.i * gamma * gamma;
     double* wi = w + c.o;
-    int p = 0;
-    double a = 0;
-    for (int e = c.lo + threadIdx.x; e < c.hi; e += blockDim.x) a += wi[e] * V[c.o + e];
-    double hq = cluster_sum_all(a, red, part, &tot, p);
-    for (int q = 0; q <= j; ++q) {
-        if (lead) Hi[q * gamma + j] = hq;
-        const double* vq = V + (int64_t)q * S + c.o;
-        a = 0;
-        if (q < j) {
-            const double* vn = vq + S;
-#pragma unroll 4
-            for (int e = c.lo + threadIdx.x; e < c.hi; e += blockDim.x) {
-                const double x = wi[e] - hq * vq[e];
-                wi[e] = x;
-                a += x * vn[e];
-            }
-        } else {
-#pragma unroll 4
-            for (int e = c.lo + threadIdx.x; e < c.hi; e += blockDim.x) {
-                const double x = wi[e] - hq * vq[e];
-                wi[e] = x;
-                a += x * x;
+    const double* vj = V + (int64_t)j * S + c.o;
+    for (int e = tid; e < j * j; e += GT) s_G[e / j][e % j] = Gi[(e / j) * gamma + e % j];     // rows 0 .. j - 1
+    // r_q and G_jq, q <= j, QB of each per pass
+    int pp = 0;
+    for (int q0 = 0; q0 <= j; q0 += QB, pp ^= 1) {
+        const int nq = min(QB, j + 1 - q0);
+        double a[2 * QB];
+#pragma unroll
+        for (int q = 0; q < 2 * QB; ++q) a[q] = 0;
+        for (int e = c.lo + tid; e < c.hi; e += GT) {
+            const double we = wi[e], ve = vj[e];
+#pragma unroll
+            for (int q = 0; q < QB; ++q)
+                if (q < nq) {
+                    const double vq = V[(int64_t)(q0 + q) * S + c.o + e];
+                    a[q] += we * vq;
+                    if (q0 + q < j) a[QB + q] += ve * vq;
+                }
+        }
+        const double ws = warp_sum16_f64(a, lane);
+        if ((lane & 1) == 0) s_red[warp][lane >> 1] = ws;
+        __syncthreads();
+        if (tid < 256) {                               // value tid / 16, warp tid % 16
+            double v = s_red[tid & 15][tid >> 4];
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if ((tid & 15) == 0) s_part[pp][tid >> 4] = v;
+        }
+        cl_sync();                                     // (s_part alternates: see cluster_sum_all)
+        if (tid < 16 * GC) {                           // value tid / GC, CTA tid % GC
+            double v = cl_ld_f64(cl_map(&s_part[pp][tid / GC], (uint32_t)(tid % GC)));
+#pragma unroll
+            for (int o = GC / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            const int q = tid / GC;
+            if (tid % GC == 0 && q % QB < nq) s_rg[q / QB][q0 + q % QB] = v;
+        }
+        __syncthreads();
+    }
+    if (warp == 0) {                                   // forward substitution, lane = q
+        double rq = lane <= j ? s_rg[0][lane] : 0.0;
+        for (int i = 0; i < j; ++i) {
+            const double hi = __shfl_sync(0xffffffffu, rq, i);
+            const double g = lane > i && lane <= j ? (lane < j ? s_G[lane][i] : s_rg[1][i]) : 0.0;
+            rq -= g * hi;
+        }
+        if (lane <= j) {
+            s_h[lane] = rq;
+            if (r == 0) {
+                Hi[lane * gamma + j] = rq;
+                if (lane < j) Gi[j * gamma + lane] = s_rg[1][lane];
             }
         }
-        hq = cluster_sum_all(a, red, part, &tot, p);
     }
-    const double nrm = sqrt(hq);
+    __syncthreads();
+    double a = 0;
+    for (int e = c.lo + tid; e < c.hi; e += GT) {
+        double we = wi[e];
+#pragma unroll 4
+        for (int q = 0; q <= j; ++q) we -= s_h[q] * V[(int64_t)q * S + c.o + e];
+        wi[e] = we;
+        a += we * we;
+    }
+    int p = 0;
+    const double nrm = sqrt(cluster_sum_all<GC>(a, red, part, &tot, p));
     if (lead) Hi[(j + 1) * gamma + j] = nrm;
     if (nrm <= 1e-14 * beta[c.i]) {
         if (lead) kused[c.i] = j + 1;
     } else {
         double* vn = V + (int64_t)(j + 1) * S + c.o;
-        for (int e = c.lo + threadIdx.x; e < c.hi; e += blockDim.x) vn[e] = wi[e] / nrm;
+        const double inv = 1.0 / nrm;
+        for (int e = c.lo + tid; e < c.hi; e += GT) vn[e] = wi[e] * inv;
         if (j + 1 == m && lead) kused[c.i] = m;
     }
     cl_sync();                                  // no CTA leaves while a peer reads its partials
@@ -376,51 +573,69 @@ __global__ void __cluster_dims__(GC, 1, 1) __launch_bounds__(GT)
 // u_t = V_k y with y the least-squares solution of min || beta e1 - H_k y || (H_k the
 // (k+1) x k Hessenberg matrix; Givens rotations), written to z on the interface DOFs.
 // Every CTA of an interface solves the small problem itself (the same bits) and writes
-// its chunk.
-__global__ void __launch_bounds__(GT) k_gm_finish(int gamma, int S, const int* __restrict__ if_off,
+// its chunk.  The small problem takes one warp, lane = column (then row): a rotation's
+// norm on entries scaled by a power of two, the rest of the rotation one step for all
+// columns; one thread alone took 30 us (an FP64 operation's latency is 65 clocks).
+__global__ void __launch_bounds__(GT) k_gm_finish(int GC, int gamma, int S, const int* __restrict__ if_off,
                                                   const int* __restrict__ if_dofs, const double* __restrict__ V,
                                                   const double* __restrict__ H, const double* __restrict__ beta,
                                                   const int* __restrict__ kused, double* __restrict__ z) {
     __shared__ double y[GAMMA_MAX];
-    __shared__ double R[GAMMA_MAX + 1][GAMMA_MAX];      // rotated Hessenberg
-    __shared__ double gv[GAMMA_MAX + 1];
-    const GmChunk c = gm_chunk(if_off, blockIdx.x / GC, blockIdx.x % GC);
-    const int ku = kused[c.i];
-    const int k = ku < 0 ? 0 : (ku == 0 ? min(gamma, c.s) : ku);
-    if (threadIdx.x == 0 && k > 0) {
-        const double* Hi = H + (int64_t)c.i * (gamma + 1) * gamma;
-        for (int r = 0; r <= k; ++r)
-            for (int cc = 0; cc < k; ++cc) R[r][cc] = (r <= cc + 1) ? Hi[r * gamma + cc] : 0.0;
-        for (int r = 0; r <= k; ++r) gv[r] = 0.0;
-        gv[0] = beta[c.i];
-        for (int cc = 0; cc < k; ++cc) {
-            const double a = R[cc][cc], b = R[cc + 1][cc];
-            const double den = hypot(a, b);
-            const double cs = den > 0 ? a / den : 1.0, sn = den > 0 ? b / den : 0.0;
-            for (int c2 = cc; c2 < k; ++c2) {
-                const double t0 = R[cc][c2], t1 = R[cc + 1][c2];
-                R[cc][c2] = cs * t0 + sn * t1;
-                R[cc + 1][c2] = -sn * t0 + cs * t1;
+    __shared__ double R[GAMMA_MAX + 1][GAMMA_MAX + 1];  // rotated Hessenberg
+    const int i = blockIdx.x / GC, o = if_off[i], s = if_off[i + 1] - o, per = (s + GC - 1) / GC;
+    const int lo = min(s, (int)(blockIdx.x % GC) * per), hi = min(s, lo + per);
+    const int ku = kused[i], tid = threadIdx.x, lane = tid & 31;
+    const int k = ku < 0 ? 0 : (ku == 0 ? min(gamma, s) : ku);
+    const double* Hi = H + (int64_t)i * (gamma + 1) * gamma;
+    for (int e = tid; e < (k + 1) * k; e += GT) R[e / k][e % k] = e / k <= e % k + 1 ? Hi[(e / k) * gamma + e % k] : 0.0;
+    __syncthreads();
+    if (tid < 32 && k > 0) {
+        double g0 = beta[i], t = 0.0;                  // the entry of the right-hand side being rotated; row `lane`'s
+        for (int c = 0; c < k; ++c) {
+            const double a = R[c][c], b = R[c + 1][c];
+            const double mx = fmax(fabs(a), fabs(b));
+            double cs = 1.0, sn = 0.0, den = mx;
+            if (mx > 0.0 && mx <= 1.7976931348623157e308) {
+                const int ex = (int)((__double_as_longlong(mx) >> 52) & 0x7ff);
+                const int sc = max(-1000, min(1000, 1023 - ex));
+                const double as = ldexp(a, sc), bs = ldexp(b, sc);
+                const double d2 = as * as + bs * bs, inv = 1.0 / sqrt(d2);
+                cs = as * inv;
+                sn = bs * inv;
+                den = ldexp(d2 * inv, -sc);
+            } else if (mx != 0.0) {                    // not finite
+                cs = sn = den = a + b;
             }
-            const double g0 = gv[cc], g1 = gv[cc + 1];
-            gv[cc] = cs * g0 + sn * g1;
-            gv[cc + 1] = -sn * g0 + cs * g1;
+            double r0 = 0.0, r1 = 0.0;
+            if (lane > c && lane < k) { r0 = R[c][lane]; r1 = R[c + 1][lane]; }
+            __syncwarp();
+            if (lane > c && lane < k) {
+                R[c][lane] = cs * r0 + sn * r1;
+                R[c + 1][lane] = -sn * r0 + cs * r1;
+            }
+            if (lane == c) { R[c][c] = den; t = cs * g0; }
+            g0 = -sn * g0;
+            __syncwarp();
         }
+        const double d = lane < k ? R[lane][lane] : 1.0;
+        const double rd = d != 0.0 ? 1.0 / d : 0.0;
         for (int r = k - 1; r >= 0; --r) {
-            double t = gv[r];
-            for (int c2 = r + 1; c2 < k; ++c2) t -= R[r][c2] * y[c2];
-            y[r] = R[r][r] != 0.0 ? t / R[r][r] : 0.0;
+            const double yr = __shfl_sync(0xffffffffu, t * rd, r);
+            if (lane < r) t -= R[lane][r] * yr;
+            if (lane == r) y[r] = yr;
         }
     }
     __syncthreads();
-    for (int e = c.lo + threadIdx.x; e < c.hi; e += blockDim.x) {
+    for (int e = lo + tid; e < hi; e += GT) {
         double u = 0;
-        for (int q = 0; q < k; ++q) u += y[q] * V[(int64_t)q * S + c.o + e];
-        z[if_dofs[c.o + e]] = u;
+        for (int q = 0; q < k; ++q) u += y[q] * V[(int64_t)q * S + o + e];
+        z[if_dofs[o + e]] = u;
     }
 }
 
 }  // namespace
+
+static int round_up_int(int v, int a) { return (v + a - 1) / a * a; }
 
 // Apply-time launches of one level's inner GMRES: reads g (global DOF order, h.d_pg) on
 // the level's interface DOFs and writes u_t = GMRES_gamma(S~_t, g_t) into z there.
@@ -438,17 +653,32 @@ int gamma_interface_solve(Handle& h, int li, double* z) {
     const bool c16 = smv_reads_fp16(Ll);
     const int gam = h.gamma;
     int pi = prof_begin(h, K_GAMMA);
-    k_gm_init<<<G.n_if * GC, GT, 0, h.stream>>>(G.d_if_off, G.d_if_dofs, h.d_pg, h.d_gm_V, h.d_gm_beta, h.d_gm_kused);
+    const int gc = gm_cluster(G.n_if, h.num_sms), lg = gc == 8 ? 3 : gc == 4 ? 2 : gc == 2 ? 1 : 0;
+    using Init = void (*)(const int*, const int*, const double*, double*, double*, int*);
+    using Step = void (*)(int, int, int, const int*, double*, double*, double*, double*, const double*, int*);
+    static constexpr Init init[4] = {k_gm_init<1>, k_gm_init<2>, k_gm_init<4>, k_gm_init<8>};
+    static constexpr Step step[4] = {k_gm_step<1>, k_gm_step<2>, k_gm_step<4>, k_gm_step<8>};
+    init[lg]<<<G.n_if * gc, GT, 0, h.stream>>>(G.d_if_off, G.d_if_dofs, h.d_pg, h.d_gm_V, h.d_gm_beta, h.d_gm_kused);
     count_launch();
     prof_end(h, pi, 0.0, 0.0);
     const int wcol = f64 ? 2 : (c16 ? 8 : 4);     // columns per lane of k_smv_leaf
     const dim3 gl((unsigned)nleaf, (unsigned)std::max(1, (Ll.max_s + 32 * wcol - 1) / (32 * wcol)));
     const unsigned gi = (unsigned)std::max(1, std::min(h.num_sms * 8, (G.S + 31) / 32));   // 32 positions per CTA
+    // One CTA a leaf does both products where the leaves fill the chip and a leaf's rows
+    // of the level fit L1 beside those of the CTAs it shares it with (the second reading hits
+    // there); larger leaves keep the two kernels, which spread a leaf over many CTAs.
+    const int W = 16 / (f64 ? 8 : c16 ? 2 : 4);
+    const bool both = nleaf >= h.num_sms && (Ll.max_s + W - 1) / W <= 256 && G.xbytes / 2 <= 192.0 * 1024 * nleaf;
+    const size_t both_smem = ((size_t)round_up_int(Ll.max_s, W) + 256 * W) * (f64 ? 8 : 4);
     for (int j = 0; j < gam; ++j) {
         const double* vj = h.d_gm_V + (int64_t)j * G.S;
         const unsigned gr = (unsigned)std::max(1, std::min(h.num_sms * 4, (G.nk + 31) / 32));   // 8 warps of 4 rows
         pi = prof_begin(h, K_GAMMA_SMV);
-        if (f64) {
+        if (both) {
+            if (f64) k_smv_both<double, false><<<nleaf, 256, both_smem, h.stream>>>(ty, Ll.d_fronts, G.d_cl_ptr, G.d_cl_row, G.d_cl_pos, Ll.max_s, vj, h.d_gm_yl);
+            else if (c16) k_smv_both<float, true><<<nleaf, 256, both_smem, h.stream>>>(Ll.d_fronts, Ll.d_fronts, G.d_cl_ptr, G.d_cl_row, G.d_cl_pos, Ll.max_s, vj, h.d_gm_yl);
+            else k_smv_both<float, false><<<nleaf, 256, both_smem, h.stream>>>(ty, Ll.d_fronts, G.d_cl_ptr, G.d_cl_row, G.d_cl_pos, Ll.max_s, vj, h.d_gm_yl);
+        } else if (f64) {
             k_smv_leaf<double, false><<<gl, 256, 0, h.stream>>>(ty, G.d_cl_ptr, G.d_cl_row, G.d_cl_pos, h.d_tl_off, vj,
                                                                 h.d_tl);
             k_smv_rows<double, false><<<gr, 256, 0, h.stream>>>(G.nk, G.d_cl_leaf, G.d_cl_row, Ll.d_fronts, h.d_tl_off,
@@ -472,12 +702,13 @@ int gamma_interface_solve(Handle& h, int li, double* z) {
                                               G.d_ci_ptr, G.d_ci_k, h.d_gm_yl, vj, h.d_gm_w);
         prof_end(h, pi, 0.0, 0.0);
         pi = prof_begin(h, K_GAMMA);
-        k_gm_mgs<<<G.n_if * GC, GT, 0, h.stream>>>(j, gam, G.S, G.d_if_off, h.d_gm_w, h.d_gm_V, h.d_gm_H, h.d_gm_beta, h.d_gm_kused);
+        step[lg]<<<G.n_if * gc, GT, 0, h.stream>>>(j, gam, G.S, G.d_if_off, h.d_gm_w, h.d_gm_V, h.d_gm_H, h.d_gm_G, h.d_gm_beta,
+                                                   h.d_gm_kused);
         prof_end(h, pi, 0.0, 0.0);
-        count_launch(4);
+        count_launch(both ? 3 : 4);
     }
     pi = prof_begin(h, K_GAMMA);
-    k_gm_finish<<<G.n_if * GC, GT, 0, h.stream>>>(gam, G.S, G.d_if_off, G.d_if_dofs, h.d_gm_V, h.d_gm_H, h.d_gm_beta,
+    k_gm_finish<<<G.n_if * gc, GT, 0, h.stream>>>(gc, gam, G.S, G.d_if_off, G.d_if_dofs, h.d_gm_V, h.d_gm_H, h.d_gm_beta,
                                              h.d_gm_kused, z);
     count_launch();
     prof_end(h, pi, 0.0, 0.0);

@@ -196,6 +196,8 @@ inline bool smv_reads_fp16(const Level& Ll) {
     return (Ll.op16 == TC_OP_F16 || Ll.h16) && !Ll.d_fronts_bwd && !is_fp64(Ll.prec);
 }
 
+// blocks of FGMRES's inner-product kernel (fixed: the sums' order)
+constexpr int FG_BLOCKS = 304;
 // CTAs per cluster of the cluster sweeps (diagonal blocks per work item of a cl_sweep level)
 constexpr int SWEEP_CL = 8;
 inline int sweep_item_blocks(const Level& L) { return L.cl_sweep ? SWEEP_CL : sweep_group(L); }
@@ -285,11 +287,13 @@ struct Handle {
     int* d_tl_off = nullptr;             // leaf slot -> offset of its t_l in d_tl
     double* d_tl = nullptr;              // X_l^T x per leaf
     double *d_gm_w = nullptr, *d_gm_V = nullptr, *d_gm_H = nullptr, *d_gm_beta = nullptr;
+    double* d_gm_G = nullptr;            // Gram entries <v_q, v_i>, i < q, per interface
     double* d_gm_yl = nullptr;           // per coupling: X_l[row] . t_l
     int* d_gm_kused = nullptr;
     // outer Krylov method (RSD_KRYLOV_PCG or RSD_KRYLOV_FGMRES) and FGMRES storage
     int krylov = RSD_KRYLOV_PCG, restart = 30;
     double *d_fg_V = nullptr, *d_fg_Z = nullptr, *d_fg_H = nullptr, *d_fg_y = nullptr;
+    double *d_fg_G = nullptr, *d_fg_part = nullptr;   // Gram entries of the basis, partial sums
     double* h_fg = nullptr;              // pinned host mirror of H columns and y
     // bounded waits of the substitution sweeps: clock cycles before a wait gives up
     long long wait_cycles = 4000000000LL;
