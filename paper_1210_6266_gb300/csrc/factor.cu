@@ -518,10 +518,26 @@ __device__ __forceinline__ void potrf_store_panel(const float* __restrict__ A, f
     }
 }
 
+// Scratch of a front slot of a tensor-core level: Mt, Tt and two Linv (see factor_level_tc).
+constexpr int64_t SCR_MT = 512 * 512, SCR_TT = 512 * 128, SCR_LINV = 512 * 512;
+constexpr int64_t SCR_FRONT = SCR_MT + SCR_TT + 2 * SCR_LINV;    // floats per front slot (two Linv)
+static_assert(WOUT == 512, "scratch blocks are sized for 512-wide outer panels");
+
+struct PotrfOut {
+    float* P;
+    int64_t ldp;
+    float* D;
+    int k, w;
+    bool rnd;
+    float* Li;          // 512-wide copy of D (row stride 512) and of D^T, or null
+    float* Mt;
+};
+
 // Row block K of the inverse (rows 32K..32K+31, all 128 columns, zero above the diagonal
-// and in rows past the front) to D
-__device__ __forceinline__ void potrf_store_inverse(const float* __restrict__ X, float* __restrict__ D, int w, int K,
-                                                    bool rnd, int t0, int nt) {
+// and in rows past the front) to D, and to its places in Linv and Mt
+__device__ __forceinline__ void potrf_store_inverse(const float* __restrict__ X, const PotrfOut& out, int K, int t0, int nt) {
+    const int w = out.w;
+    const bool rnd = out.rnd;
     for (int e = t0; e < DB * (NB / 4); e += nt) {
         const int i = DB * K + e / (NB / 4), c = 4 * (e % (NB / 4));
         float4 dv = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
@@ -532,17 +548,19 @@ __device__ __forceinline__ void potrf_store_inverse(const float* __restrict__ X,
             dv.z = c + 2 <= i ? tf32_store(x.z, rnd) : 0.0f;
             dv.w = c + 3 <= i ? tf32_store(x.w, rnd) : 0.0f;
         }
-        *reinterpret_cast<float4*>(D + i * NB + c) = dv;
+        *reinterpret_cast<float4*>(out.D + i * NB + c) = dv;
+        if (out.Li) *reinterpret_cast<float4*>(out.Li + i * 512 + c) = dv;
+    }
+    if (!out.Mt) return;
+    // columns 32K .. 32K+31 of D^T on and above the diagonal (below it stays zero)
+    for (int e = t0; e < DB * (K + 1) * (DB / 4); e += nt) {
+        const int c = e / (DB / 4), i = DB * K + 4 * (e % (DB / 4));
+        float v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[q] = (i + q < w && c <= i + q) ? tf32_store(X[(i + q) * XLD + c], rnd) : 0.0f;
+        *reinterpret_cast<float4*>(out.Mt + (int64_t)c * 512 + i) = make_float4(v[0], v[1], v[2], v[3]);
     }
 }
-
-struct PotrfOut {
-    float* P;
-    int64_t ldp;
-    float* D;
-    int k, w;
-    bool rnd;
-};
 
 // panel K's work off the critical chain, by nw warps (index wi).  Part 1: trailing tiles
 // and the finalised X row block K (warps left over store panel K of L); a named barrier
@@ -579,7 +597,7 @@ __device__ __forceinline__ void potrf_background(float* __restrict__ A, float* _
         const int I = K + 1 + it / (K + 1), J = it % (K + 1);
         tile32_atb<true>(LT + DB * I, XLD, X + DB * K * XLD + DB * J, XLD, A + DB * J * XLD + DB * I, XLD, 1.0f, lane);
     }
-    if (wi >= n2) potrf_store_inverse(X, out.D, out.w, K, out.rnd, 32 * (wi - n2) + lane, 32 * (nw - n2));
+    if (wi >= n2) potrf_store_inverse(X, out, K, 32 * (wi - n2) + lane, 32 * (nw - n2));
 }
 
 // rows [r_lo, r_hi) of the block into A (lower part; zero above the diagonal; identity
@@ -618,7 +636,8 @@ __device__ __forceinline__ void potrf_load_rows(float* __restrict__ A, const flo
 }
 
 __global__ void __launch_bounds__(256, 1) k_potrf_diag_blk(const FrontDesc* __restrict__ fronts, int k,
-                                                       int* __restrict__ err, int round_tf32, int* __restrict__ bad_front) {
+                                                       int* __restrict__ err, int round_tf32, int* __restrict__ bad_front,
+                                                       float* __restrict__ scr, int K0, int which) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float* A = (float*)smem_raw;                  // 128 x XLD
     float* X = A + NB * XLD;                      // 128 x XLD
@@ -629,9 +648,15 @@ __global__ void __launch_bounds__(256, 1) k_potrf_diag_blk(const FrontDesc* __re
     __shared__ float s_ri[NB];                    // 1 / l_jj
     __shared__ int s_bad;
     const FrontDesc f = fronts[blockIdx.x];
+    grid_dep_wait();
     if (f.s <= k) return;
-    const int w = min(NB, f.s - k);
-    const PotrfOut out{(float*)f.P, (int64_t)f.ldp, (float*)f.Dinv + (int64_t)(k / NB) * NB * NB, k, w, round_tf32 != 0};
+    const int w = min(NB, f.s - k), j0 = k - K0;
+    PotrfOut out{(float*)f.P, (int64_t)f.ldp, (float*)f.Dinv + (int64_t)(k / NB) * NB * NB, k, w, round_tf32 != 0, nullptr, nullptr};
+    if (scr) {                                    // the block's places in Linv and Mt
+        float* sf = scr + (int64_t)blockIdx.x * SCR_FRONT;
+        out.Li = sf + SCR_MT + SCR_TT + which * SCR_LINV + (int64_t)j0 * 512 + j0;
+        if (j0 + NB < WOUT) out.Mt = sf + (int64_t)j0 * 512 + j0;
+    }
     const float* P = (const float*)f.P;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) s_bad = 0;
@@ -640,6 +665,7 @@ __global__ void __launch_bounds__(256, 1) k_potrf_diag_blk(const FrontDesc* __re
     for (int J = 0; J < NB / DB; ++J) {
         const int o = J * DB;
         const int nb_below = NB / DB - 1 - J;
+        if (J == NB / DB - 1) grid_dep_launch();   // the next launch's blocks set up during the last quarter
         if (warp == 0) {
             if (potrf_chol32(A, LJ, s_rs, s_ri, o, lane) && lane == 0) s_bad = 1;
         } else if (J == 0) {
@@ -679,7 +705,7 @@ __global__ void __launch_bounds__(256, 1) k_potrf_diag_blk(const FrontDesc* __re
     potrf_background(A, X, LT, XT, out, NB / DB - 1, warp, 8, 0, lane);
     if (warp >= NB / DB - 1) potrf_store_panel(A, out.P, out.ldp, k, w, NB / DB - 1, out.rnd, 32 * (warp - (NB / DB - 1)) + lane, 32 * (8 - (NB / DB - 1)));
     __syncthreads();
-    potrf_store_inverse(X, out.D, w, NB / DB - 1, out.rnd, tid, 256);
+    potrf_store_inverse(X, out, NB / DB - 1, tid, 256);
     if (tid == 0 && s_bad) {
         atomicExch(&err[ERR_NOT_SPD], 1);
         atomicMin(&err[ERR_NOT_SPD_NODE], f.node);
@@ -1059,15 +1085,24 @@ int launch_extend_add(Handle& h, int li) {
 //   (a0) the outer update of the whole panel, as above;
 //   (a)-(c) restricted to the W x W diagonal block of the panel (its 128-blocks factored
 //        one after another: small GEMMs and the diagonal factor+inverse);
-//   (e)  Mt = L_pp^-T for the W x W block L_pp, from its inverted diagonal blocks:
-//        Mt_jj = Dinv_j^T and, block column i after block column i, for the rows j < i
-//        Mt[j, i] = -(sum_{k<i} Mt[j, k] L_ik^T) Dinv_i^T    (from Mt L_pp^T = I);
-//        then Linv = Mt^T;
+//   (e)  Linv = L_pp^-1 and Mt = Linv^T for the W x W block L_pp, block row j after block
+//        row j: their diagonal blocks Dinv_j and Dinv_j^T come from the diagonal kernel,
+//        Tt = Mt[0:j, 0:j] L_{j,<j}^T, Linv[j, 0:j] = -Dinv_j Tt^T, Mt[0:j, j] = -Tt Dinv_j^T.
+//        Tt reads what the update (a) of block column j reads, and the two products
+//        read what the solve (c) of block column j reads, so they are further tasks of
+//        those launches and only the last block row adds one;
 //   (f)  the rows below the block in one step, X = A L_pp^-T = A Linv^T, in place: the
 //        column tile [256, W) first (it reads A[:, 0:W]), then [0, 256) (it reads only
 //        A[:, 0:256], which the first launch left untouched).
 // (e)-(f) replace the per-128-column updates and solves of the rows below the block
 // (many thin, memory-bound GEMMs) by two K = W GEMMs.
+//
+// (a)-(e) are a serial chain of short launches, each 10-30 us of which most is latency, and
+// at the root (one front) this chain is the setup time.  Its kernels are launched to set up
+// (lists, barriers, TMEM, tensor maps) while the one before still runs.  49^3 elasticity
+// (root of 18,000 columns): setup + solve 45.8 -> 42.1 ms; 65^3 gradient 39.7 -> 36.8 ms;
+// 24 grids of 17 to 65 nodes a side in one call 153.0 -> 147.3 ms (block inverse in launches of its own, no early
+// launch -> this).
 //
 // Levels with few fronts (the root and the level below it) also look ahead: the
 // diagonal-block work runs on a high-priority stream (the "chain") beside the bulk
@@ -1079,44 +1114,6 @@ int launch_extend_add(Handle& h, int li) {
 // receives the same products in either order; only the outer update's K range is
 // summed in two parts, and the rows below a diagonal block are solved in two groups.
 constexpr int LOOKAHEAD_FRONTS = 16;
-constexpr int64_t SCR_MT = 512 * 512, SCR_TT = 512 * 128, SCR_LINV = 512 * 512;
-constexpr int64_t SCR_FRONT = SCR_MT + SCR_TT + 2 * SCR_LINV;    // floats per front slot (two Linv)
-static_assert(WOUT == 512, "scratch blocks are sized for 512-wide outer panels");
-
-// Mt's diagonal blocks: Mt[j, j] = Dinv_j^T (upper triangular), j < ceil(W / NB).
-__global__ void k_mt_diag(const FrontDesc* __restrict__ fronts, int K0, float* __restrict__ scr) {
-    const FrontDesc f = fronts[blockIdx.z];
-    if (f.s <= K0) return;
-    const int W = min(WOUT, f.s - K0);
-    const int j = blockIdx.y;
-    if (j * NB >= W) return;
-    float* Mt = scr + (int64_t)blockIdx.z * SCR_FRONT;
-    const float* D = (const float*)f.Dinv + (int64_t)(K0 / NB + j) * NB * NB;
-    __shared__ float t[32][33];
-    const int bx = blockIdx.x & 3, by = blockIdx.x >> 2;     // 4 x 4 tiles of 32 x 32
-    for (int r = threadIdx.y; r < 32; r += blockDim.y) t[r][threadIdx.x] = D[(by * 32 + r) * NB + bx * 32 + threadIdx.x];
-    __syncthreads();
-    for (int r = threadIdx.y; r < 32; r += blockDim.y)
-        Mt[(int64_t)(j * NB + bx * 32 + r) * 512 + j * NB + by * 32 + threadIdx.x] = t[threadIdx.x][r];
-}
-
-// Linv = Mt^T on the W x W block, zero elsewhere in the 512 x 512 slot.
-__global__ void k_linv_transpose(const FrontDesc* __restrict__ fronts, int K0, float* __restrict__ scr, int which) {
-    const FrontDesc f = fronts[blockIdx.z];
-    if (f.s <= K0) return;
-    const int W = min(WOUT, f.s - K0);
-    const float* Mt = scr + (int64_t)blockIdx.z * SCR_FRONT;
-    float* Li = scr + (int64_t)blockIdx.z * SCR_FRONT + SCR_MT + SCR_TT + which * SCR_LINV;
-    __shared__ float t[32][33];
-    const int bx = blockIdx.x, by = blockIdx.y;               // 16 x 16 tiles of 32 x 32
-    for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-        const int row = by * 32 + r, col = bx * 32 + threadIdx.x;
-        t[r][threadIdx.x] = (row < W && col < W) ? Mt[(int64_t)row * 512 + col] : 0.f;
-    }
-    __syncthreads();
-    for (int r = threadIdx.y; r < 32; r += blockDim.y)
-        Li[(int64_t)(bx * 32 + r) * 512 + by * 32 + threadIdx.x] = t[threadIdx.x][r];
-}
 
 static int ensure_chain(Handle& h) {
     if (h.chain) return RSD_OK;
@@ -1160,30 +1157,6 @@ static int factor_level_tc(Handle& h, int li, bool lookahead) {
     std::vector<GemmTask> tasks;
     auto wend = [](const FrontDesc& f, int K0) { return std::min(K0 + WOUT, f.s); };
     auto P = [&](const FrontDesc& f, int r, int c) { return (char*)f.P + ((int64_t)r * f.ldp + c) * es; };
-    // (a) rows [r0, r1) of column block k from the finished columns [K0, k)
-    auto add_update = [&](const FrontDesc& f, int k, int K0, int r0, int r1) {
-        if (f.s <= k || k <= K0 || r1 <= r0) return;
-        GemmTask t{};
-        t.A = P(f, r0, K0); t.B = P(f, k, K0); t.C = P(f, r0, k);
-        t.lda = t.ldb = t.ldc = f.ldp;
-        t.M = r1 - r0; t.N = std::min(NB, f.s - k); t.K = k - K0;
-        t.lower = 0; t.beta = 1;
-        t.map_a = t.map_b = f.node;
-        t.a_r0 = r0; t.a_c0 = K0; t.b_r0 = k; t.b_c0 = K0;
-        tasks.push_back(t);
-    };
-    // (c) rows [r0, r1) of column block k times the inverted diagonal block
-    auto add_solve = [&](const FrontDesc& f, int k, int r0, int r1) {
-        if (f.s <= k || r1 <= r0) return;
-        GemmTask t{};
-        t.A = P(f, r0, k); t.B = (const char*)f.Dinv + (int64_t)(k / NB) * NB * NB * es; t.C = P(f, r0, k);
-        t.lda = t.ldc = f.ldp; t.ldb = NB;
-        t.M = r1 - r0; t.N = std::min(NB, f.s - k); t.K = t.N;
-        t.lower = 0; t.beta = 0;
-        t.map_a = t.map_b = f.node;
-        t.a_r0 = r0; t.a_c0 = k; t.b_r0 = (k / NB) * NB; t.b_c0 = 0;
-        tasks.push_back(t);
-    };
     // (a0) rows [r0, r1) of the panel at K0 from the columns [kb, ke)
     auto add_outer = [&](const FrontDesc& f, int K0, int kb, int ke, int r0, int r1) {
         if (f.s <= K0 || ke <= kb || r1 <= r0) return;
@@ -1199,74 +1172,62 @@ static int factor_level_tc(Handle& h, int li, bool lookahead) {
         tasks.push_back(t);
     };
     auto general = [&](int ma, int a_r0, int a_c0, int mb, int b_r0, int b_c0, void* C, int ldc,
-                       int M, int N, int K, float alpha) {
+                       int M, int N, int K, float alpha, int beta = 0, int round = 1) {
         GemmTask t{};
         t.C = C; t.ldc = ldc; t.M = M; t.N = N; t.K = K;
-        t.lower = 0; t.beta = 0; t.alpha = alpha; t.round = 1;
+        t.lower = 0; t.beta = beta; t.alpha = alpha; t.round = round;
         t.map_a = ma; t.map_b = mb;
         t.a_r0 = a_r0; t.a_c0 = a_c0; t.b_r0 = b_r0; t.b_c0 = b_c0;
         tasks.push_back(t);
     };
 
-    // (a)-(c) and (e) for the diagonal block of every front at K0, on stream cs; the
-    // block inverse goes to Linv buffer `which`
     // The level is issued twice: a dry pass in which the GEMM launcher only records each
     // launch's task and tile lists (and nothing else is launched), then, after one upload
     // of everything recorded, the real pass.  Per-launch uploads would stall the issuing
     // thread behind the streams' queues and serialise copies between the chain's kernels.
     bool dry = false;
+    // (a)-(c) and (e) for the diagonal block of every front at K0, on stream cs; the
+    // block inverse goes to Linv buffer `which`
     auto factor_block = [&](int K0, int which, cudaStream_t cs, int slot) -> int {
         for (int j = 0; j < WOUT / NB; ++j) {
             const int k = K0 + j * NB;
             if (k >= L.max_s) break;
-            tasks.clear();
-            for (auto& f : L.fronts) add_update(f, k, K0, k, wend(f, K0));
-            RSD_TRY(gemm_tc_launch(h, li, tasks, 0, cs, slot));
+            if (j > 0) {
+                tasks.clear();
+                for (int q = 0; q < nf; ++q) {
+                    const FrontDesc& f = L.fronts[q];
+                    if (f.s <= k) continue;
+                    const int w = std::min(NB, f.s - k);
+                    // (a) block column j from the block's finished columns
+                    general(tc_map_panel(f.node), k, K0, tc_map_panel(f.node), k, K0, P(f, k, k), f.ldp, wend(f, K0) - k, w, j * NB, -1.0f, 1, 0);
+                    // (e) Tt = Mt[0:j, 0:j] L_{j,<j}^T
+                    general(map_mt(q), 0, 0, tc_map_panel(f.node), k, K0, tt[q], 128, j * NB, w, j * NB, 1.0f);
+                }
+                RSD_TRY(gemm_tc_launch(h, li, tasks, TC_CHAIN, cs, slot));
+            }
             double pf = 0, pb = 0;
             for (auto& f : L.fronts)
                 if (f.s > k) { const double w = std::min(NB, f.s - k); pf += 2.0 * w * w * w / 3.0; pb += (2.0 * w * w + NB * NB) * es; }
             if (!dry) {
                 const int ppi = prof_begin(h, K_POTRF, cs);
-                k_potrf_diag_blk<<<(unsigned)nf, 256, potrf_smem, cs>>>(L.d_fronts, k, h.d_err, 1, h.d_front_bad);
+                RSD_CUDA_TRY(launch_dependent(k_potrf_diag_blk, dim3((unsigned)nf), dim3(256), potrf_smem, cs, (const FrontDesc*)L.d_fronts, k,
+                                              h.d_err, 1, h.d_front_bad, scr, K0, which));
                 count_launch();
                 prof_end(h, ppi, pf, pb, cs);
-                RSD_CUDA_TRY(cudaGetLastError());
             }
             tasks.clear();
-            for (auto& f : L.fronts) add_solve(f, k, k + std::min(NB, std::max(0, f.s - k)), wend(f, K0));
-            RSD_TRY(gemm_tc_launch(h, li, tasks, 1, cs, slot));
-        }
-        // (e) Mt = L_pp^-T, then Linv = Mt^T
-        if (!dry) {
-            k_mt_diag<<<dim3(16, WOUT / NB, (unsigned)nf), dim3(32, 8), 0, cs>>>(L.d_fronts, K0, scr);
-            count_launch();
-            RSD_CUDA_TRY(cudaGetLastError());
-        }
-        for (int i = 1; i < WOUT / NB; ++i) {
-            const int k = K0 + i * NB;
-            if (k >= L.max_s) break;
-            tasks.clear();                              // Tt = Mt[0:i NB, 0:i NB] L_{i,<i}^T
             for (int q = 0; q < nf; ++q) {
                 const FrontDesc& f = L.fronts[q];
                 if (f.s <= k) continue;
-                general(map_mt(q), 0, 0, tc_map_panel(f.node), k, K0, tt[q], 128,
-                        i * NB, std::min(NB, f.s - k), i * NB, 1.0f);
+                const int w = std::min(NB, f.s - k), r0 = k + w, r1 = wend(f, K0);
+                // (c) the block's rows below times the inverted diagonal block
+                if (r1 > r0) general(tc_map_panel(f.node), r0, k, tc_map_dinv(f.node), k, 0, P(f, r0, k), f.ldp, r1 - r0, w, w, 1.0f);
+                if (j == 0) continue;
+                // (e) Linv[j, 0:j] = -Dinv_j Tt^T and, where a later block reads it, Mt[0:j, j] = -Tt Dinv_j^T
+                general(tc_map_dinv(f.node), k, 0, map_tt(q), 0, 0, (which ? lv1 : lv0)[q] + (int64_t)j * NB * 512, 512, w, j * NB, w, -1.0f);
+                if (r1 > r0) general(map_tt(q), 0, 0, tc_map_dinv(f.node), k, 0, mt[q] + j * NB, 512, j * NB, w, w, -1.0f);
             }
-            RSD_TRY(gemm_tc_launch(h, li, tasks, TC_GENERAL, cs, slot));
-            tasks.clear();                              // Mt[0:i NB, i] = -Tt Dinv_i^T
-            for (int q = 0; q < nf; ++q) {
-                const FrontDesc& f = L.fronts[q];
-                if (f.s <= k) continue;
-                const int w = std::min(NB, f.s - k);
-                general(map_tt(q), 0, 0, tc_map_dinv(f.node), k, 0, mt[q] + i * NB, 512,
-                        i * NB, w, w, -1.0f);
-            }
-            RSD_TRY(gemm_tc_launch(h, li, tasks, TC_GENERAL, cs, slot));
-        }
-        if (!dry) {
-            k_linv_transpose<<<dim3(16, 16, (unsigned)nf), dim3(32, 8), 0, cs>>>(L.d_fronts, K0, scr, which);
-            count_launch();
-            RSD_CUDA_TRY(cudaGetLastError());
+            RSD_TRY(gemm_tc_launch(h, li, tasks, TC_CHAIN, cs, slot));
         }
         return RSD_OK;
     };
@@ -1328,8 +1289,11 @@ static int factor_level_tc(Handle& h, int li, bool lookahead) {
                 if (!dry) RSD_CUDA_TRY(cudaStreamWaitEvent(Cs, h.ev_ready, 0));
                 if (p >= 1) {
                     tasks.clear();
-                    for (auto& f : L.fronts) add_outer(f, K0, K0 - WOUT, K0, K0, wend(f, K0));
-                    RSD_TRY(gemm_tc_launch(h, li, tasks, 3, Cs, cslot));
+                    for (auto& f : L.fronts)
+                        if (f.s > K0)
+                            general(tc_map_panel(f.node), K0, K0 - WOUT, tc_map_panel(f.node), K0, K0 - WOUT, P(f, K0, K0), f.ldp,
+                                    wend(f, K0) - K0, wend(f, K0) - K0, WOUT, -1.0f, 1, 0);
+                    RSD_TRY(gemm_tc_launch(h, li, tasks, TC_CHAIN, Cs, cslot));
                 }
                 RSD_TRY(factor_block(K0, which, Cs, cslot));
                 if (!dry) RSD_CUDA_TRY(cudaEventRecord(ev_linv, Cs));
@@ -1401,9 +1365,8 @@ int run_factor_level(Handle& h, int li) {
     }
     std::vector<GemmTask> tasks;
     int rc = RSD_OK;
-    auto run_gemm = [&](int kind) -> int {
+    auto run_gemm = [&]() -> int {
         if (tasks.empty()) return RSD_OK;
-        if (tc) return gemm_tc_launch(h, li, tasks, kind, h.stream);
         finalize_tasks(tasks, SB, SB);
         return f64 ? launch_gemm_simt<double>(h, tasks, d_tasks, -1.0, h.stream)
                    : launch_gemm_simt<float>(h, tasks, d_tasks, -1.0f, h.stream);
@@ -1429,7 +1392,7 @@ int run_factor_level(Handle& h, int li) {
                 t.a_r0 = K0; t.a_c0 = 0; t.b_r0 = K0; t.b_c0 = 0;
                 tasks.push_back(t);
             }
-            rc = run_gemm(3);
+            rc = run_gemm();
             if (rc != RSD_OK) break;
         }
         // (a) inner update of the NB-wide panel from the finished columns K0..k of its
@@ -1450,7 +1413,7 @@ int run_factor_level(Handle& h, int li) {
                 t.a_r0 = k; t.a_c0 = K0; t.b_r0 = k; t.b_c0 = K0;
                 tasks.push_back(t);
             }
-            rc = run_gemm(0);
+            rc = run_gemm();
             if (rc != RSD_OK) break;
         }
         // (b) diagonal block factor + inverse
@@ -1462,44 +1425,23 @@ int run_factor_level(Handle& h, int li) {
             if (rc != RSD_OK) break;
         } else {
             const int ppi = prof_begin(h, K_POTRF);
-            k_potrf_diag_blk<<<(unsigned)L.fronts.size(), 256, POTRF_BLK_SMEM, h.stream>>>(L.d_fronts, k, h.d_err, tc ? 1 : 0, h.d_front_bad);
+            k_potrf_diag_blk<<<(unsigned)L.fronts.size(), 256, POTRF_BLK_SMEM, h.stream>>>(L.d_fronts, k, h.d_err, 0, h.d_front_bad, nullptr, k, 0);
             count_launch();
             prof_end(h, ppi, pf, pb);
         }
         if (cudaGetLastError() != cudaSuccess) { rc = RSD_ERR_CUDA; break; }
         // (c) panel solve below the diagonal block
-        if (tc) {
-            tasks.clear();
-            for (auto& f : L.fronts) {
-                if (f.s <= k) continue;
-                const int w = std::min(NB, f.s - k);
-                if (f.N - k - w <= 0) continue;
-                GemmTask t{};
-                t.A = (const char*)f.P + ((int64_t)(k + w) * f.ldp + k) * es;
-                t.B = (const char*)f.Dinv + (int64_t)(k / NB) * NB * NB * es;
-                t.C = (char*)t.A;
-                t.lda = t.ldc = f.ldp; t.ldb = NB;
-                t.M = f.N - k - w; t.N = w; t.K = w;
-                t.lower = 0; t.beta = 0;
-                t.map_a = f.node; t.map_b = f.node;
-                t.a_r0 = k + w; t.a_c0 = k; t.b_r0 = (k / NB) * NB; t.b_c0 = 0;
-                tasks.push_back(t);
-            }
-            rc = gemm_tc_launch(h, li, tasks, 1, h.stream);
-            if (rc != RSD_OK) break;
-        } else {
-            const int rows = L.max_N;   // upper bound on rows below the diagonal
-            dim3 grid((unsigned)std::max(1, (rows - k + TR_ROWS - 1) / TR_ROWS), (unsigned)L.fronts.size());
-            double tf = 0, tb = 0;
-            for (auto& f : L.fronts)
-                if (f.s > k) { const double w = std::min(NB, f.s - k), m = f.N - k - w; tf += m * w * w; tb += 2.0 * m * w * es; }
-            const int tpi = prof_begin(h, K_TRSM);
-            if (f64) k_trsm_simt<double><<<grid, 256, trsm_smem, h.stream>>>(L.d_fronts, k, 0);
-            else k_trsm_simt<float><<<grid, 256, trsm_smem, h.stream>>>(L.d_fronts, k, 0);
-            count_launch();
-            prof_end(h, tpi, tf, tb);
-            if (cudaGetLastError() != cudaSuccess) { rc = RSD_ERR_CUDA; break; }
-        }
+        const int rows = L.max_N;   // upper bound on rows below the diagonal
+        dim3 grid((unsigned)std::max(1, (rows - k + TR_ROWS - 1) / TR_ROWS), (unsigned)L.fronts.size());
+        double tf = 0, tb = 0;
+        for (auto& f : L.fronts)
+            if (f.s > k) { const double w = std::min(NB, f.s - k), m = f.N - k - w; tf += m * w * w; tb += 2.0 * m * w * es; }
+        const int tpi = prof_begin(h, K_TRSM);
+        if (f64) k_trsm_simt<double><<<grid, 256, trsm_smem, h.stream>>>(L.d_fronts, k, 0);
+        else k_trsm_simt<float><<<grid, 256, trsm_smem, h.stream>>>(L.d_fronts, k, 0);
+        count_launch();
+        prof_end(h, tpi, tf, tb);
+        if (cudaGetLastError() != cudaSuccess) { rc = RSD_ERR_CUDA; break; }
     }
     // (d) Schur contribution to the ancestors: U -= X X^T
     if (rc == RSD_OK) {

@@ -143,6 +143,8 @@ k_gemm_tc(const TcTask* __restrict__ tasks, const TcTile* __restrict__ tiles,
     const int kb0 = tl.kb0, nk = tl.kb1 - tl.kb0;
 
     if (threadIdx.x == 0) {
+        tma_prefetch_map(maps + tk.map_a);
+        tma_prefetch_map(maps + tk.map_b);
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(bar_full + 8 * s, 1);
             mbar_init(bar_empty + 8 * s, 1);
@@ -159,6 +161,10 @@ k_gemm_tc(const TcTask* __restrict__ tasks, const TcTile* __restrict__ tiles,
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tmem_slot;
+    // The lists and maps read above were uploaded before the launch before this one began;
+    // everything below reads and writes what that launch may still be working on.
+    grid_dep_wait();
+    grid_dep_launch();
 
     if (warp == 0) {
         if (lane == 0) {
@@ -811,9 +817,9 @@ int gemm_tc_peak(int n, int reps, double seconds, cudaStream_t stream, int num_s
     return RSD_OK;
 }
 
-// kind 0: inner panel update, 1: panel solve (B = inverted diagonal block),
-// 2: U -= X X^T (lower tiles), 3: outer panel update, TC_GENERAL: map indices, alpha and
-// rounding taken from the task (128- or 256-wide tiles by the widest N).
+// kind 2: U -= X X^T (lower tiles), 3: outer panel update, TC_GENERAL: map indices, alpha
+// and rounding taken from the task (128- or 256-wide tiles by the widest N), TC_CHAIN: the
+// same in 128-wide tiles, launched to set up while the kernel before it still runs.
 int gemm_tc_launch(Handle& h, int /*li*/, const std::vector<GemmTask>& tasks, int kind, cudaStream_t stream,
                    int buf_slot, int max_ctas, int op) {
     TcState* st = state_of(h);
@@ -825,10 +831,10 @@ int gemm_tc_launch(Handle& h, int /*li*/, const std::vector<GemmTask>& tasks, in
     for (auto& g : tasks) max_n = std::max(max_n, g.N);
     int bn = (kind == 2 || kind == 3 || (kind == TC_GENERAL && max_n > 128)) ? 256 : 128;
     if (op != TC_OP_TF32 && kind != 2 && kind != 3) return RSD_ERR_ARG;     // 16-bit: long-K updates only
-    // tuned configuration of the update kinds (0, 2, 3): the tile width (TF32 outer and
-    // Schur updates; 16-bit operands run the 128 x 256 kernel only) and the split-K count
+    // tuned configuration of the update kinds (2, 3): the tile width (16-bit operands run
+    // the 128 x 256 kernel only) and the split-K count
     int tuned_split = 0;
-    if ((kind == 0 || kind == 2 || kind == 3) && (st->force_bn || !st->tune.empty())) {
+    if ((kind == 2 || kind == 3) && (st->force_bn || !st->tune.empty())) {
         int t256 = 0, maxk = 0;
         for (auto& g : tasks) {
             const int tm = (g.M + BM - 1) / BM, tn = (g.N + 255) / 256;
@@ -838,7 +844,7 @@ int gemm_tc_launch(Handle& h, int /*li*/, const std::vector<GemmTask>& tasks, in
         int tbn = 0;
         if (st->force_bn) { tbn = st->force_bn; tuned_split = st->force_split; }
         else tune_lookup(st->tune, op == TC_OP_TF32 ? TC_OP_TF32 : TC_OP_F16, t256, maxk, &tbn, &tuned_split);
-        if (tbn && kind != 0 && op == TC_OP_TF32) bn = tbn;
+        if (tbn && op == TC_OP_TF32) bn = tbn;
     }
     std::vector<TcTask> tt(tasks.size());
     std::vector<std::array<int, 3>> out;            // (task, tm, tn) output tiles
@@ -848,15 +854,13 @@ int gemm_tc_launch(Handle& h, int /*li*/, const std::vector<GemmTask>& tasks, in
         t.C = (float*)g.C;
         t.ldc = g.ldc; t.M = g.M; t.N = g.N; t.K = g.K;
         t.lower = g.lower; t.beta = g.beta;
-        t.map_a = kind == TC_GENERAL ? g.map_a : (op != TC_OP_TF32 ? tc_map_panel16(g.map_a) : tc_map_panel(g.map_a));
-        t.map_b = kind == TC_GENERAL ? g.map_b : (kind == 1 ? tc_map_dinv(g.map_b)
-                                                            : op != TC_OP_TF32 ? tc_map_panel16(g.map_b) : tc_map_panel(g.map_b));
+        t.map_a = kind >= TC_GENERAL ? g.map_a : (op != TC_OP_TF32 ? tc_map_panel16(g.map_a) : tc_map_panel(g.map_a));
+        t.map_b = kind >= TC_GENERAL ? g.map_b : (op != TC_OP_TF32 ? tc_map_panel16(g.map_b) : tc_map_panel(g.map_b));
         t.sa = op != TC_OP_TF32 ? g.sa : nullptr;
         t.sb = op != TC_OP_TF32 ? g.sb : nullptr;
         t.a_r0 = g.a_r0; t.a_c0 = g.a_c0; t.b_r0 = g.b_r0; t.b_c0 = g.b_c0;
-        t.alpha = kind == TC_GENERAL ? g.alpha : (kind == 1 ? 1.0f : -1.0f);
-        // panel-solve results are final factor entries
-        t.round_tf32 = kind == TC_GENERAL ? g.round : (kind == 1);
+        t.alpha = kind >= TC_GENERAL ? g.alpha : -1.0f;
+        t.round_tf32 = kind >= TC_GENERAL ? g.round : 0;
         const int tm = (g.M + BM - 1) / BM, tn = (g.N + bn - 1) / bn;
         // The persistent kernel runs consecutive tiles at the same time.  Wide outputs
         // (U -= X X^T) are walked in bands of TILE_BAND row blocks, column block by
@@ -872,13 +876,13 @@ int gemm_tc_launch(Handle& h, int /*li*/, const std::vector<GemmTask>& tasks, in
                 }
     }
     if (out.empty()) return RSD_OK;
-    // split K when the output tiles cannot fill the GPU (never for the in-place panel solve)
+    // split K when the output tiles cannot fill the GPU (never for in-place solves)
     const int bke = op != TC_OP_TF32 ? 64 : BK;            // elements per K block
     int max_kb = 0;
     for (auto& g : tasks) max_kb = std::max(max_kb, (g.K + bke - 1) / bke);
     int nsplit = 1;
     if (tuned_split > 0) nsplit = std::max(1, std::min(tuned_split, max_kb / 4));
-    else if (kind != 1 && kind != TC_GENERAL && (int)out.size() < sms)
+    else if (kind < TC_GENERAL && (int)out.size() < sms)
         nsplit = std::max(1, std::min(sms / (int)out.size(), max_kb / SPLIT_MIN_KB));
     if ((int)out.size() * nsplit * (bn / 256 > 0 ? bn / 256 : 1) > st->ws_slots * (256 / bn)) nsplit = 1;
     std::vector<TcTile> tl;
@@ -966,7 +970,10 @@ int gemm_tc_launch(Handle& h, int /*li*/, const std::vector<GemmTask>& tasks, in
     const int pi = prof_begin(h, op != TC_OP_TF32 ? K_GEMM_TC16 : K_GEMM_TC, stream);
     // short K (inner panel update, panel solve): 3-stage ring, two CTAs per SM so one
     // tile's epilogue overlaps the other's main loop; long K: deeper rings, one CTA per SM
-    if (bn == 128 && max_kb <= 16)
+    if (kind == TC_CHAIN && max_kb <= 16)
+        RSD_CUDA_TRY(launch_dependent(k_gemm_tc<128, 3>, dim3((unsigned)tl.size()), dim3(TC_THREADS), Smem<128, 3>::TOTAL, stream,
+                                      (const TcTask*)d_tasks, (const TcTile*)d_tiles, (const CUtensorMap*)st->d_maps, bf.d_ws, h.d_err));
+    else if (bn == 128 && max_kb <= 16)
         k_gemm_tc<128, 3><<<(unsigned)tl.size(), TC_THREADS, Smem<128, 3>::TOTAL, stream>>>(d_tasks, d_tiles, st->d_maps, bf.d_ws, h.d_err);
     else if (bn == 128)
         k_gemm_tc<128, 6><<<(unsigned)tl.size(), TC_THREADS, Smem<128, 6>::TOTAL, stream>>>(d_tasks, d_tiles, st->d_maps, bf.d_ws, h.d_err);

@@ -319,12 +319,30 @@ void prof_end(Handle& h, int idx, double flops, double bytes, cudaStream_t strea
 inline int prof_begin(Handle& h, int cls) { return prof_begin(h, cls, h.stream); }
 inline void prof_end(Handle& h, int idx, double flops, double bytes) { prof_end(h, idx, flops, bytes, h.stream); }
 
-// Tensor-core GEMM launch (gemm_tc.cu).  kind 0: inner panel update, 1: panel solve with
-// an inverted diagonal block, 2: U -= X X^T (lower tiles), 3: outer panel update.
+// Launch on `st` with leave to start while the kernel before it on the stream still runs:
+// the kernel must call grid_dep_wait() in every block before it reads or writes anything
+// that kernel (or one before it) may touch.  grid_dep_launch() in the kernel before says
+// from where on its successor's blocks may come in; without it they come in at its end.
+__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <typename... P, typename... A>
+inline cudaError_t launch_dependent(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... a) {
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid; c.blockDim = block; c.dynamicSmemBytes = smem; c.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &at; c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, k, P(a)...);
+}
+
+// Tensor-core GEMM launch (gemm_tc.cu).  kind 2: U -= X X^T (lower tiles), 3: outer panel
+// update.
 // `slot` selects the launch buffers (one per stream that launches concurrently);
 // max_ctas > 0 caps the CTAs of the persistent kernel (leaving SMs to another stream).
 constexpr int TC_SLOTS = 2;
 constexpr int TC_GENERAL = 4;        // kind: explicit map indices, alpha and rounding
+constexpr int TC_CHAIN = 5;          // kind: the same, a link of the diagonal-block chain
 // Recorded launches: between record_begin and record_end, gemm_tc_launch only records
 // each launch's task and tile lists; record_end uploads them in one copy on `stream`,
 // and the next gemm_tc_launch calls, which must repeat the recorded sequence, launch
