@@ -112,6 +112,103 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+// Epilogue of one warp: columns [c_lo, c_hi) of 32 accumulator rows starting at row g0 of
+// the task (TMEM lanes of this warp), 32 columns at a time.  tcgen05.ld gives a thread one
+// row; read-modify-writing C in that layout touches 32 lines per load, 16 B of each, and
+// at short K these L1 wavefronts (16K cycles per 128 x 256 tile, against 4K cycles of MMA at
+// K = 512) set the pace.  So each 32 x 32 piece goes through 4 KB of the warp's own shared
+// memory (16-byte chunks exchanged by row, no bank conflicts) and C is read and written
+// a full 128-byte line per row, the next piece's C being fetched meanwhile: a fourth of the
+// wavefronts.  Setup + solve at 129^3 (FP16 form) 245.5 -> 230.3 ms, batched grids
+// 146.7 -> 140.1, 49^3 elasticity 41.9 -> 40.4, 65^3 gradient 37.4 -> 36.2.  `ws` non-null: the raw products of a split-K slice, row stride BN.
+template <int OP, int BN>
+struct TcEpilogue {
+    const TcTask& tk;
+    float* ws;                  // this warp's first row of the slot, or null
+    unsigned char* stage;       // 4 KB
+    int g0, n0, lane;
+
+    __device__ __forceinline__ bool live(int c0) const {
+        if (ws) return true;
+        return g0 < tk.M && n0 + c0 < tk.N && (!tk.lower || n0 + c0 <= g0 + 31);
+    }
+    __device__ __forceinline__ bool full(int c0) const {
+        return g0 + 32 <= tk.M && n0 + c0 + 32 <= tk.N && (!tk.lower || n0 + c0 + 31 <= g0);
+    }
+    __device__ __forceinline__ void fetch(int c0, float4 (&c)[8]) const {
+        if (ws || !tk.beta || !live(c0)) return;
+        const int gc = n0 + c0 + 4 * (lane & 7);
+        const bool fl = full(c0);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int gr = g0 + 4 * i + (lane >> 3);
+            const float* p = tk.C + (int64_t)gr * tk.ldc + gc;
+            if (fl) { c[i] = *(const float4*)p; continue; }
+            float v[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) v[q] = gr < tk.M && gc + q < tk.N && (!tk.lower || gc + q <= gr) ? p[q] : 0.f;
+            c[i] = make_float4(v[0], v[1], v[2], v[3]);
+        }
+    }
+    __device__ __forceinline__ void put(int c0, const uint32_t (&r)[32], const float4 (&c)[8]) const {
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            *(uint4*)(stage + lane * 128 + ((q ^ (lane & 7)) << 4)) = make_uint4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
+        __syncwarp();
+        const int q = lane & 7, gc = n0 + c0 + 4 * q;
+        const bool fl = full(c0);
+        float4 sb = make_float4(1.f, 1.f, 1.f, 1.f);
+        if constexpr (OP != TC_OP_TF32) {
+            if (!ws) {
+                sb.x = gc < tk.N ? __ldg(tk.sb + gc) : 0.f;
+                sb.y = gc + 1 < tk.N ? __ldg(tk.sb + gc + 1) : 0.f;
+                sb.z = gc + 2 < tk.N ? __ldg(tk.sb + gc + 2) : 0.f;
+                sb.w = gc + 3 < tk.N ? __ldg(tk.sb + gc + 3) : 0.f;
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int rr = 4 * i + (lane >> 3), gr = g0 + rr;
+            const float4 a = *(const float4*)(stage + rr * 128 + ((q ^ (rr & 7)) << 4));
+            if (ws) {
+                *(float4*)(ws + (int64_t)rr * BN + c0 + 4 * q) = a;
+                continue;
+            }
+            float4 o = tk.beta ? c[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+            if constexpr (OP != TC_OP_TF32) {
+                // undo the operands' row scales: entry (gr, gc) times sa[gr] sb[gc]
+                const float ar = gr < tk.M ? tk.alpha * __ldg(tk.sa + gr) : 0.f;
+                o.x += a.x * ar * sb.x; o.y += a.y * ar * sb.y; o.z += a.z * ar * sb.z; o.w += a.w * ar * sb.w;
+            } else {
+                o.x += tk.alpha * a.x; o.y += tk.alpha * a.y; o.z += tk.alpha * a.z; o.w += tk.alpha * a.w;
+            }
+            if (tk.round_tf32) { o.x = tf32_rn(o.x); o.y = tf32_rn(o.y); o.z = tf32_rn(o.z); o.w = tf32_rn(o.w); }
+            float* p = tk.C + (int64_t)gr * tk.ldc + gc;
+            if (fl) { *(float4*)p = o; continue; }
+            const float v[4] = {o.x, o.y, o.z, o.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (gr < tk.M && gc + u < tk.N && (!tk.lower || gc + u <= gr)) p[u] = v[u];
+        }
+    }
+    // columns [c_lo, c_hi) from TMEM address taddr (lane quadrant included); c0_regs holds the
+    // first piece's C
+    __device__ __forceinline__ void run(uint32_t taddr, int c_lo, int c_hi, float4 (&cur)[8], bool ok) const {
+#pragma unroll 1
+        for (int c0 = c_lo; c0 < c_hi; c0 += 32) {
+            if (!live(c0)) continue;
+            uint32_t r[32];
+            tmem_ld32(taddr + c0, r);
+            float4 nxt[8];
+            if (c0 + 32 < c_hi) fetch(c0 + 32, nxt);
+            if (ok) put(c0, r, cur);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) cur[i] = nxt[i];
+        }
+    }
+};
+
 template <int BN, int ST>
 struct Smem {
     static constexpr int STAGES = ST;
@@ -119,6 +216,8 @@ struct Smem {
     static constexpr int B_BYTES = BN * BK * 4;
     static constexpr int STAGE = A_BYTES + B_BYTES;
     static constexpr int TOTAL = STAGES * STAGE + 1024 /*align*/ + 256 /*barriers*/;
+    static constexpr int EPI = 256;                                // the persistent kernel's epilogue staging, past the barriers
+    static constexpr int TOTAL_PERSIST = TOTAL + (TCP_THREADS / 32 - 2) * 4096;
 };
 
 template <int BN, int ST>
@@ -211,49 +310,14 @@ k_gemm_tc(const TcTask* __restrict__ tasks, const TcTile* __restrict__ tiles,
         float* crow = tk.C + (int64_t)gr * tk.ldc;
         if (tk.beta && tl.ws_slot < 0 && gr < tk.M)
             prefetch_c_row(crow, n0, min(n0 + BN, tk.lower ? min(tk.N, gr + 1) : tk.N));
+        // the ring is free once the last MMA is done: the first 16 KB stage the epilogue
+        const TcEpilogue<TC_OP_TF32, BN> ep{tk, tl.ws_slot >= 0 ? ws + ((int64_t)tl.ws_slot * BM + quarter * 32) * BN : nullptr,
+                                            sbase + quarter * 4096, m0 + quarter * 32, n0, lane};
+        float4 cur[8];
+        ep.fetch(0, cur);
         const bool ok = mbar_wait(bar_done, 0, err);
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        float* wrow = tl.ws_slot >= 0 ? ws + ((int64_t)tl.ws_slot * BM + row) * BN : nullptr;
-#pragma unroll 1
-        for (int c0 = 0; c0 < BN; c0 += 32) {
-            uint32_t r[32];
-            tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + c0, r);
-            if (!ok) continue;
-            if (wrow) {                                   // split-K partial: raw product
-#pragma unroll
-                for (int q = 0; q < 8; ++q)
-                    *(float4*)(wrow + c0 + 4 * q) = make_float4(__uint_as_float(r[4 * q]), __uint_as_float(r[4 * q + 1]),
-                                                                __uint_as_float(r[4 * q + 2]), __uint_as_float(r[4 * q + 3]));
-                continue;
-            }
-            if (gr >= tk.M) continue;
-            const int gc0 = n0 + c0;
-            if (gc0 >= tk.N) continue;
-            if (tk.lower && gc0 > gr) continue;
-            if (gc0 + 32 <= tk.N && (!tk.lower || gc0 + 31 <= gr)) {
-#pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    float4* p = (float4*)(crow + gc0 + 4 * q);
-                    float4 o = tk.beta ? *p : make_float4(0.f, 0.f, 0.f, 0.f);
-                    o.x += tk.alpha * __uint_as_float(r[4 * q + 0]);
-                    o.y += tk.alpha * __uint_as_float(r[4 * q + 1]);
-                    o.z += tk.alpha * __uint_as_float(r[4 * q + 2]);
-                    o.w += tk.alpha * __uint_as_float(r[4 * q + 3]);
-                    if (tk.round_tf32) { o.x = tf32_rn(o.x); o.y = tf32_rn(o.y); o.z = tf32_rn(o.z); o.w = tf32_rn(o.w); }
-                    *p = o;
-                }
-            } else {
-#pragma unroll
-                for (int q = 0; q < 32; ++q) {
-                    const int gc = gc0 + q;
-                    if (gc < tk.N && (!tk.lower || gc <= gr)) {
-                        float* p = crow + gc;
-                        const float o = (tk.beta ? *p : 0.f) + tk.alpha * __uint_as_float(r[q]);
-                        *p = tk.round_tf32 ? tf32_rn(o) : o;
-                    }
-                }
-            }
-        }
+        ep.run(tmem + ((uint32_t)(quarter * 32) << 16), 0, BN, cur, ok);
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     }
     __syncthreads();
@@ -374,58 +438,13 @@ k_gemm_tc_persist(const TcTask* __restrict__ tasks, const TcTile* __restrict__ t
             float* crow = tk.C + (int64_t)gr * tk.ldc;
             if (tk.beta && tl.ws_slot < 0 && gr < tk.M)
                 prefetch_c_row(crow, n0 + cb, min(n0 + ce, tk.lower ? min(tk.N, gr + 1) : tk.N));
+            const TcEpilogue<OP, BN> ep{tk, tl.ws_slot >= 0 ? ws + ((int64_t)tl.ws_slot * BM + quarter * 32) * BN : nullptr,
+                                        sbase + STAGES * S::STAGE + S::EPI + (warp - 2) * 4096, m0 + quarter * 32, n0, lane};
+            float4 cur[8];
+            ep.fetch(cb, cur);
             const bool ok = mbar_wait(bar_accf + 8 * buf, use, err);
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            float* wrow = tl.ws_slot >= 0 ? ws + ((int64_t)tl.ws_slot * BM + row) * BN : nullptr;
-#pragma unroll 1
-            for (int c0 = cb; c0 < ce; c0 += 32) {
-                uint32_t r[32];
-                tmem_ld32(tmem + buf * BN + ((uint32_t)(quarter * 32) << 16) + c0, r);
-                if (!ok) continue;
-                if (wrow) {
-#pragma unroll
-                    for (int q = 0; q < 8; ++q)
-                        *(float4*)(wrow + c0 + 4 * q) = make_float4(__uint_as_float(r[4 * q]), __uint_as_float(r[4 * q + 1]),
-                                                                    __uint_as_float(r[4 * q + 2]), __uint_as_float(r[4 * q + 3]));
-                    continue;
-                }
-                if (gr >= tk.M) continue;
-                const int gc0 = n0 + c0;
-                if (gc0 >= tk.N) continue;
-                if (tk.lower && gc0 > gr) continue;
-                if constexpr (OP != TC_OP_TF32) {
-                    // undo the operands' row scales: entry (gr, gc) times sa[gr] sb[gc]
-                    const float ar = tk.alpha * tk.sa[gr];
-                    const int qe = min(32, tk.N - gc0);
-#pragma unroll
-                    for (int q = 0; q < 32; ++q)
-                        r[q] = __float_as_uint(q < qe ? __uint_as_float(r[q]) * ar * __ldg(tk.sb + gc0 + q) : 0.f);
-                }
-                const float al = OP != TC_OP_TF32 ? 1.0f : tk.alpha;
-                if (gc0 + 32 <= tk.N && (!tk.lower || gc0 + 31 <= gr)) {
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) {
-                        float4* p = (float4*)(crow + gc0 + 4 * q);
-                        float4 o = tk.beta ? *p : make_float4(0.f, 0.f, 0.f, 0.f);
-                        o.x += al * __uint_as_float(r[4 * q + 0]);
-                        o.y += al * __uint_as_float(r[4 * q + 1]);
-                        o.z += al * __uint_as_float(r[4 * q + 2]);
-                        o.w += al * __uint_as_float(r[4 * q + 3]);
-                        if (tk.round_tf32) { o.x = tf32_rn(o.x); o.y = tf32_rn(o.y); o.z = tf32_rn(o.z); o.w = tf32_rn(o.w); }
-                        *p = o;
-                    }
-                } else {
-#pragma unroll
-                    for (int q = 0; q < 32; ++q) {
-                        const int gc = gc0 + q;
-                        if (gc < tk.N && (!tk.lower || gc <= gr)) {
-                            float* p = crow + gc;
-                            const float o = (tk.beta ? *p : 0.f) + al * __uint_as_float(r[q]);
-                            *p = tk.round_tf32 ? tf32_rn(o) : o;
-                        }
-                    }
-                }
-            }
+            ep.run(tmem + buf * BN + ((uint32_t)(quarter * 32) << 16), cb, ce, cur, ok);
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar_acce + 8 * buf) : "memory");
         }
@@ -767,9 +786,9 @@ int gemm_tc_peak(int n, int reps, double seconds, cudaStream_t stream, int num_s
     RSD_CUDA_TRY(cudaMemcpyAsync(buf + o_maps, maps, sizeof(maps), cudaMemcpyHostToDevice, stream));
     RSD_CUDA_TRY(cudaMemcpyAsync(buf + o_task, &t, sizeof(t), cudaMemcpyHostToDevice, stream));
     RSD_CUDA_TRY(cudaMemcpyAsync(buf + o_tiles, tiles.data(), tiles.size() * sizeof(TcTile), cudaMemcpyHostToDevice, stream));
-    RSD_CUDA_TRY(cudaFuncSetAttribute(k_gemm_tc_persist<256, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<256, 4>::TOTAL));
-    RSD_CUDA_TRY(cudaFuncSetAttribute(k_gemm_tc_persist<256, 4, TC_OP_F16>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<256, 4>::TOTAL));
-    RSD_CUDA_TRY(cudaFuncSetAttribute(k_gemm_tc_persist<256, 4, TC_OP_BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<256, 4>::TOTAL));
+    RSD_CUDA_TRY(cudaFuncSetAttribute(k_gemm_tc_persist<256, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<256, 4>::TOTAL_PERSIST));
+    RSD_CUDA_TRY(cudaFuncSetAttribute(k_gemm_tc_persist<256, 4, TC_OP_F16>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<256, 4>::TOTAL_PERSIST));
+    RSD_CUDA_TRY(cudaFuncSetAttribute(k_gemm_tc_persist<256, 4, TC_OP_BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<256, 4>::TOTAL_PERSIST));
     int* err = (int*)(buf + o_err);
     const int ctas = std::min((int)tiles.size(), num_sms);
     auto launch = [&]() {
@@ -777,11 +796,11 @@ int gemm_tc_peak(int n, int reps, double seconds, cudaStream_t stream, int num_s
         const TcTile* tl = (const TcTile*)(buf + o_tiles);
         const CUtensorMap* mp = (const CUtensorMap*)(buf + o_maps);
         if (op == TC_OP_F16)
-            k_gemm_tc_persist<256, 4, TC_OP_F16><<<(unsigned)ctas, TCP_THREADS, Smem<256, 4>::TOTAL, stream>>>(tk, tl, (int)tiles.size(), mp, nullptr, err);
+            k_gemm_tc_persist<256, 4, TC_OP_F16><<<(unsigned)ctas, TCP_THREADS, Smem<256, 4>::TOTAL_PERSIST, stream>>>(tk, tl, (int)tiles.size(), mp, nullptr, err);
         else if (op == TC_OP_BF16)
-            k_gemm_tc_persist<256, 4, TC_OP_BF16><<<(unsigned)ctas, TCP_THREADS, Smem<256, 4>::TOTAL, stream>>>(tk, tl, (int)tiles.size(), mp, nullptr, err);
+            k_gemm_tc_persist<256, 4, TC_OP_BF16><<<(unsigned)ctas, TCP_THREADS, Smem<256, 4>::TOTAL_PERSIST, stream>>>(tk, tl, (int)tiles.size(), mp, nullptr, err);
         else
-            k_gemm_tc_persist<256, 4><<<(unsigned)ctas, TCP_THREADS, Smem<256, 4>::TOTAL, stream>>>(tk, tl, (int)tiles.size(), mp, nullptr, err);
+            k_gemm_tc_persist<256, 4><<<(unsigned)ctas, TCP_THREADS, Smem<256, 4>::TOTAL_PERSIST, stream>>>(tk, tl, (int)tiles.size(), mp, nullptr, err);
         count_launch();
     };
     cudaEvent_t e0, e1;
@@ -961,10 +980,9 @@ int gemm_tc_launch(Handle& h, int /*li*/, const std::vector<GemmTask>& tasks, in
     if (!st->attr_set) {
         RSD_CUDA_TRY(cudaFuncSetAttribute(k_gemm_tc<128, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<128, 3>::TOTAL));
         RSD_CUDA_TRY(cudaFuncSetAttribute(k_gemm_tc<128, 6>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<128, 6>::TOTAL));
-        RSD_CUDA_TRY(cudaFuncSetAttribute(k_gemm_tc<256, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<256, 4>::TOTAL));
-        RSD_CUDA_TRY(cudaFuncSetAttribute(k_gemm_tc_persist<256, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<256, 4>::TOTAL));
-        RSD_CUDA_TRY(cudaFuncSetAttribute(k_gemm_tc_persist<256, 4, TC_OP_F16>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<256, 4>::TOTAL));
-        RSD_CUDA_TRY(cudaFuncSetAttribute(k_gemm_tc_persist<256, 4, TC_OP_BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<256, 4>::TOTAL));
+        RSD_CUDA_TRY(cudaFuncSetAttribute(k_gemm_tc_persist<256, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<256, 4>::TOTAL_PERSIST));
+        RSD_CUDA_TRY(cudaFuncSetAttribute(k_gemm_tc_persist<256, 4, TC_OP_F16>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<256, 4>::TOTAL_PERSIST));
+        RSD_CUDA_TRY(cudaFuncSetAttribute(k_gemm_tc_persist<256, 4, TC_OP_BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<256, 4>::TOTAL_PERSIST));
         st->attr_set = true;
     }
     const int pi = prof_begin(h, op != TC_OP_TF32 ? K_GEMM_TC16 : K_GEMM_TC, stream);
@@ -980,13 +998,13 @@ int gemm_tc_launch(Handle& h, int /*li*/, const std::vector<GemmTask>& tasks, in
     else {
         const int ctas = std::min((int)tl.size(), sms);
         if (op == TC_OP_F16)
-            k_gemm_tc_persist<256, 4, TC_OP_F16><<<(unsigned)ctas, TCP_THREADS, Smem<256, 4>::TOTAL, stream>>>(
+            k_gemm_tc_persist<256, 4, TC_OP_F16><<<(unsigned)ctas, TCP_THREADS, Smem<256, 4>::TOTAL_PERSIST, stream>>>(
                 d_tasks, d_tiles, (int)tl.size(), st->d_maps, bf.d_ws, h.d_err);
         else if (op == TC_OP_BF16)
-            k_gemm_tc_persist<256, 4, TC_OP_BF16><<<(unsigned)ctas, TCP_THREADS, Smem<256, 4>::TOTAL, stream>>>(
+            k_gemm_tc_persist<256, 4, TC_OP_BF16><<<(unsigned)ctas, TCP_THREADS, Smem<256, 4>::TOTAL_PERSIST, stream>>>(
                 d_tasks, d_tiles, (int)tl.size(), st->d_maps, bf.d_ws, h.d_err);
         else
-            k_gemm_tc_persist<256, 4><<<(unsigned)ctas, TCP_THREADS, Smem<256, 4>::TOTAL, stream>>>(
+            k_gemm_tc_persist<256, 4><<<(unsigned)ctas, TCP_THREADS, Smem<256, 4>::TOTAL_PERSIST, stream>>>(
                 d_tasks, d_tiles, (int)tl.size(), st->d_maps, bf.d_ws, h.d_err);
     }
     count_launch();
