@@ -1038,26 +1038,31 @@ static int build_handle(Handle& h, Analysis& a, const int64_t* rowptr, const int
     const size_t o_err = take(sizeof(int) * ERR_SLOTS);
     const size_t o_bad = take(sizeof(int) * a.n_nodes);
     const size_t o_ticket = take(sizeof(int) * 2 * nl + 16);
-    // FP64 fronts factored on the tensor cores: the digits of one panel, last in the arena
-    // (levels are factored one after another and share it); without room for it the FP64
-    // levels run on the FP64 pipe as before
-    size_t f64_ws = 0;
+    // Workspaces of the factorisation, last in the arena (levels are factored one after
+    // another and share it): the digits of one panel of FP64 fronts factored on the tensor
+    // cores, the diagonal-block scratch of the TF32 and 16-bit levels (2.3 or 3.3 MB a front:
+    // allocating it stream-ordered on each setup stalled the host, 1.8 ms at 512 fronts;
+    // setup + solve of 24 grids of 17 to 65 nodes a side 140.1 -> 130.5 ms, of 49^3
+    // elasticity 40.1 -> 37.7 ms).  Without room for it the FP64 levels run on the FP64 pipe
+    // and the others allocate their scratch.
+    size_t f64_ws = 0, tc_ws = 0;
     for (int d = 0; d < nl; ++d) {
+        if (tc_level(h.levels[d]) && h.levels[d].factored) tc_ws = std::max(tc_ws, factor_tc_workspace((int)h.levels[d].nodes.size()));
         if (!is_fp64(h.levels[d].prec) || !h.levels[d].factored) continue;
         std::vector<int> rows;
         for (int t : h.levels[d].nodes) rows.push_back(a.I_off[t + 1] - a.I_off[t] + beff(t));
         f64_ws = std::max(f64_ws, f64_tc_workspace(rows, h.lu));
     }
-    const size_t o_f64 = off;
-    h.arena_bytes = off + f64_ws;
+    const size_t o_ws = off;
+    h.arena_bytes = off + std::max(f64_ws, tc_ws);
     {
         int dev = 0;
         cudaGetDevice(&dev);
         h.device = dev;
         size_t got = 0;
         h.arena = arena_take(h.arena_bytes, dev, &got);
-        if (!h.arena && f64_ws) {
-            f64_ws = 0;
+        if (!h.arena && (f64_ws || tc_ws)) {
+            f64_ws = tc_ws = 0;
             h.arena_bytes = off;
             h.arena = arena_take(h.arena_bytes, dev, &got);
         }
@@ -1069,8 +1074,12 @@ static int build_handle(Handle& h, Analysis& a, const int64_t* rowptr, const int
     }
     char* A = h.arena;
     if (f64_ws) {
-        h.f64_ws = A + o_f64;
+        h.f64_ws = A + o_ws;
         h.f64_ws_bytes = f64_ws;
+    }
+    if (tc_ws) {
+        h.tc_ws = A + o_ws;
+        h.tc_ws_bytes = tc_ws;
     }
     h.d_rowptr = (int64_t*)(A + o_rowptr);
     h.d_col = (int*)(A + o_col);

@@ -520,7 +520,8 @@ __device__ __forceinline__ void potrf_store_panel(const float* __restrict__ A, f
 
 // Scratch of a front slot of a tensor-core level: Mt, Tt and two Linv (see factor_level_tc).
 constexpr int64_t SCR_MT = 512 * 512, SCR_TT = 512 * 128, SCR_LINV = 512 * 512;
-constexpr int64_t SCR_FRONT = SCR_MT + SCR_TT + 2 * SCR_LINV;    // floats per front slot (two Linv)
+// floats per front slot; levels that look ahead alternate between two Linv
+constexpr int64_t scr_front(bool lookahead) { return SCR_MT + SCR_TT + (lookahead ? 2 : 1) * SCR_LINV; }
 static_assert(WOUT == 512, "scratch blocks are sized for 512-wide outer panels");
 
 struct PotrfOut {
@@ -637,7 +638,7 @@ __device__ __forceinline__ void potrf_load_rows(float* __restrict__ A, const flo
 
 __global__ void __launch_bounds__(256, 1) k_potrf_diag_blk(const FrontDesc* __restrict__ fronts, int k,
                                                        int* __restrict__ err, int round_tf32, int* __restrict__ bad_front,
-                                                       float* __restrict__ scr, int K0, int which) {
+                                                       float* __restrict__ scr, int64_t scr_stride, int K0, int which) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float* A = (float*)smem_raw;                  // 128 x XLD
     float* X = A + NB * XLD;                      // 128 x XLD
@@ -653,7 +654,7 @@ __global__ void __launch_bounds__(256, 1) k_potrf_diag_blk(const FrontDesc* __re
     const int w = min(NB, f.s - k), j0 = k - K0;
     PotrfOut out{(float*)f.P, (int64_t)f.ldp, (float*)f.Dinv + (int64_t)(k / NB) * NB * NB, k, w, round_tf32 != 0, nullptr, nullptr};
     if (scr) {                                    // the block's places in Linv and Mt
-        float* sf = scr + (int64_t)blockIdx.x * SCR_FRONT;
+        float* sf = scr + (int64_t)blockIdx.x * scr_stride;
         out.Li = sf + SCR_MT + SCR_TT + which * SCR_LINV + (int64_t)j0 * 512 + j0;
         if (j0 + NB < WOUT) out.Mt = sf + (int64_t)j0 * 512 + j0;
     }
@@ -1137,16 +1138,19 @@ static int factor_level_tc(Handle& h, int li, bool lookahead) {
     // the bulk persistent GEMM leaves SMs for the chain's diagonal blocks and its small
     // GEMMs (one wave of them)
     const int bulk_ctas = lookahead ? h.num_sms - std::min(h.num_sms / 4, std::max(8, 2 * nf)) : 0;
-    // per-front scratch: Mt, Tt, Linv (Mt's lower part stays zero)
-    float* scr = nullptr;
-    RSD_CUDA_TRY(cudaMallocAsync((void**)&scr, sizeof(float) * SCR_FRONT * nf, B));
-    RSD_CUDA_TRY(cudaMemsetAsync(scr, 0, sizeof(float) * SCR_FRONT * nf, B));
+    // per-front scratch: Mt, Tt, Linv (Mt's lower part and Linv's upper part stay zero)
+    const int64_t stride = scr_front(lookahead);
+    const size_t scr_bytes = sizeof(float) * stride * nf;
+    float* scr = (float*)h.tc_ws;
+    const bool own_scr = scr_bytes > h.tc_ws_bytes;
+    if (own_scr) RSD_CUDA_TRY(cudaMallocAsync((void**)&scr, scr_bytes, B));
+    RSD_CUDA_TRY(cudaMemsetAsync(scr, 0, scr_bytes, B));
     std::vector<float*> mt(nf), tt(nf), lv0(nf), lv1(nf);
     for (int i = 0; i < nf; ++i) {
-        mt[i] = scr + SCR_FRONT * i;
+        mt[i] = scr + stride * i;
         tt[i] = mt[i] + SCR_MT;
         lv0[i] = tt[i] + SCR_TT;
-        lv1[i] = lv0[i] + SCR_LINV;
+        lv1[i] = lookahead ? lv0[i] + SCR_LINV : lv0[i];
     }
     int mbase = 0;
     RSD_TRY(gemm_tc_scratch_maps(h, mt, tt, lv0, lv1, B, &mbase));
@@ -1211,7 +1215,7 @@ static int factor_level_tc(Handle& h, int li, bool lookahead) {
             if (!dry) {
                 const int ppi = prof_begin(h, K_POTRF, cs);
                 RSD_CUDA_TRY(launch_dependent(k_potrf_diag_blk, dim3((unsigned)nf), dim3(256), potrf_smem, cs, (const FrontDesc*)L.d_fronts, k,
-                                              h.d_err, 1, h.d_front_bad, scr, K0, which));
+                                              h.d_err, 1, h.d_front_bad, scr, stride, K0, which));
                 count_launch();
                 prof_end(h, ppi, pf, pb, cs);
             }
@@ -1341,9 +1345,11 @@ static int factor_level_tc(Handle& h, int li, bool lookahead) {
     const int rc_issue = issue();
     gemm_tc_replay_end(h, B);
     RSD_TRY(rc_issue);
-    cudaFreeAsync(scr, B);
+    if (own_scr) cudaFreeAsync(scr, B);
     return RSD_OK;
 }
+
+size_t factor_tc_workspace(int n_fronts) { return sizeof(float) * (size_t)scr_front(n_fronts <= LOOKAHEAD_FRONTS) * n_fronts; }
 
 // Partial Cholesky of every front of level li (steps (a)-(d) above).
 int run_factor_level(Handle& h, int li) {
@@ -1425,7 +1431,7 @@ int run_factor_level(Handle& h, int li) {
             if (rc != RSD_OK) break;
         } else {
             const int ppi = prof_begin(h, K_POTRF);
-            k_potrf_diag_blk<<<(unsigned)L.fronts.size(), 256, POTRF_BLK_SMEM, h.stream>>>(L.d_fronts, k, h.d_err, 0, h.d_front_bad, nullptr, k, 0);
+            k_potrf_diag_blk<<<(unsigned)L.fronts.size(), 256, POTRF_BLK_SMEM, h.stream>>>(L.d_fronts, k, h.d_err, 0, h.d_front_bad, nullptr, 0, k, 0);
             count_launch();
             prof_end(h, ppi, pf, pb);
         }

@@ -228,6 +228,8 @@ struct Handle {
     // the arena only fits without it (those fronts then run on the FP64 pipe)
     char* f64_ws = nullptr;
     size_t f64_ws_bytes = 0;
+    char* tc_ws = nullptr;               // scratch of a tensor-core level (factor_tc_workspace), or null
+    size_t tc_ws_bytes = 0;
     int* d_err = nullptr;
     int* d_front_bad = nullptr;          // per node: a pivot of its factorisation failed
     int promoted = 0;                    // fronts re-factored one precision up at setup
@@ -343,6 +345,7 @@ inline cudaError_t launch_dependent(void (*k)(P...), dim3 grid, dim3 block, size
 constexpr int TC_SLOTS = 2;
 constexpr int TC_GENERAL = 4;        // kind: explicit map indices, alpha and rounding
 constexpr int TC_CHAIN = 5;          // kind: the same, a link of the diagonal-block chain
+size_t factor_tc_workspace(int n_fronts);   // bytes of diagonal-block scratch of a tensor-core level
 // Recorded launches: between record_begin and record_end, gemm_tc_launch only records
 // each launch's task and tile lists; record_end uploads them in one copy on `stream`,
 // and the next gemm_tc_launch calls, which must repeat the recorded sequence, launch
