@@ -46,8 +46,7 @@ extern "C" {
 /* ---- precisions of the stored factors and the arithmetic on them ----------------- */
 #define RSD_PREC_FP64  0   /* FP64 storage and accuracy: the factorisation's products are split
                               into exact FP16 products on tcgen05 tensor cores and rounded to
-                              FP64 once; diagonal blocks and sweeps (and nonsymmetric fronts)
-                              in FP64 on CUDA cores                                      */
+                              FP64 once; diagonal blocks and sweeps in FP64 on CUDA cores */
 #define RSD_PREC_FP32  1   /* FP32 storage, FP32 arithmetic on CUDA cores                */
 #define RSD_PREC_TF32  2   /* FP32 storage; GEMM/TRSM updates on tcgen05 tensor cores in
                               TF32 with FP32 accumulation; diagonal blocks in FP32       */
@@ -137,7 +136,7 @@ typedef struct {
                             front is factored F_II = L U without pivoting (Eqs. 3.2-3.3 with
                             K_IL != K_LI^T, as the two-variable systems of Sec. 4, Eqs.
                             4.2-4.3, need), X = F_BI U^-1, Y = L^-1 F_IB, U_t = F_BB - X Y;
-                            FP64 or FP32 on CUDA cores; rsd_solve runs FGMRES; exact mode, or
+                            FP64 (as RSD_PREC_FP64) or FP32; rsd_solve runs FGMRES; exact mode, or
                             paper mode with gamma > 0.  A zero or non-finite pivot is
                             reported as RSD_ERR_NOT_SPD.                                    */
 } rsd_options;
