@@ -136,7 +136,10 @@ typedef struct {
                             front is factored F_II = L U without pivoting (Eqs. 3.2-3.3 with
                             K_IL != K_LI^T, as the two-variable systems of Sec. 4, Eqs.
                             4.2-4.3, need), X = F_BI U^-1, Y = L^-1 F_IB, U_t = F_BB - X Y;
-                            FP64 (as RSD_PREC_FP64) or FP32; rsd_solve runs FGMRES; exact mode, or
+                            FP64 (as RSD_PREC_FP64; on CUDA cores where equations and
+                            unknowns are scaled so differently, by powers of two or otherwise,
+                            that the split products would lose accuracy) or FP32; rsd_solve
+                            runs FGMRES; exact mode, or
                             paper mode with gamma > 0.  A zero or non-finite pivot is
                             reported as RSD_ERR_NOT_SPD.                                    */
 } rsd_options;

@@ -1038,6 +1038,7 @@ static int build_handle(Handle& h, Analysis& a, const int64_t* rowptr, const int
     const size_t o_err = take(sizeof(int) * ERR_SLOTS);
     const size_t o_bad = take(sizeof(int) * a.n_nodes);
     const size_t o_ticket = take(sizeof(int) * 2 * nl + 16);
+    const size_t o_lscale = h.lu ? take(sizeof(int) * ((size_t)a.n + LU_SCALE_EXTRA)) : 0;
     // Workspaces of the factorisation, last in the arena (levels are factored one after
     // another and share it): the digits of one panel of FP64 fronts factored on the tensor
     // cores, the diagonal-block scratch of the TF32 and 16-bit levels (2.3 or 3.3 MB a front:
@@ -1087,6 +1088,7 @@ static int build_handle(Handle& h, Analysis& a, const int64_t* rowptr, const int
     h.d_err = (int*)(A + o_err);
     h.d_front_bad = (int*)(A + o_bad);
     h.d_ticket = (int*)(A + o_ticket);
+    if (h.lu) h.d_lu_scale = (int*)(A + o_lscale);
     h.d_partial = (double*)(A + o_partial);
     h.d_scal = (double*)(A + o_scal);
     double* vecs = (double*)(A + o_vecs);
@@ -1346,41 +1348,57 @@ static int build_handle(Handle& h, Analysis& a, const int64_t* rowptr, const int
     RSD_TRY(gemm_tc_prepare(h));
     h.prof.host_part[5] = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t_plan).count();
     // ---- numeric setup, deepest level first ----
-    // Every level's fronts (disjoint arena regions) are zeroed and receive their K entries
-    // up front, leaves first: the device does this while the host plans the leaf level.
-    for (int d = nl - 1; d >= 0; --d) {
-        if (!h.levels[d].factored) continue;
-        RSD_TRY(launch_zero_fronts(h, d));
-        if (h.lu) RSD_TRY(launch_assemble_fronts_lu(h, d, h.d_rowptr, h.d_col, h.d_val, d_owner, d_rank, d_tin, d_tout));
-        else RSD_TRY(launch_assemble_fronts(h, d, h.d_rowptr, h.d_col, h.d_val, d_owner, d_rank, d_tin, d_tout));
-    }
-    if (!paper) {
-        const auto t_issue = std::chrono::steady_clock::now();
+    if (h.lu && h.f64_ws) RSD_TRY(launch_lu_scale(h));
+    auto factor_all = [&]() -> int {
+        // Every level's fronts (disjoint arena regions) are zeroed and receive their K entries
+        // up front, leaves first: the device does this while the host plans the leaf level.
         for (int d = nl - 1; d >= 0; --d) {
-            if (h.lu) {
-                RSD_TRY(launch_extend_add_lu(h, d));
-                RSD_TRY(run_factor_level_lu(h, d));
-                continue;
+            if (!h.levels[d].factored) continue;
+            RSD_TRY(launch_zero_fronts(h, d));
+            if (h.lu) RSD_TRY(launch_assemble_fronts_lu(h, d, h.d_rowptr, h.d_col, h.d_val, d_owner, d_rank, d_tin, d_tout));
+            else RSD_TRY(launch_assemble_fronts(h, d, h.d_rowptr, h.d_col, h.d_val, d_owner, d_rank, d_tin, d_tout));
+        }
+        if (!paper) {
+            const auto t_issue = std::chrono::steady_clock::now();
+            for (int d = nl - 1; d >= 0; --d) {
+                if (h.lu) {
+                    RSD_TRY(launch_extend_add_lu(h, d));
+                    RSD_TRY(run_factor_level_lu(h, d));
+                    continue;
+                }
+                RSD_TRY(launch_extend_add(h, d));
+                RSD_TRY(run_factor_level(h, d));
+                RSD_TRY(launch_factor_copy16(h, d));
             }
-            RSD_TRY(launch_extend_add(h, d));
-            RSD_TRY(run_factor_level(h, d));
-            RSD_TRY(launch_factor_copy16(h, d));
+            h.prof.host_issue_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t_issue).count();
+        } else {
+            // every interface front is K_II plus leaf updates: factor the leaves, scatter
+            // their updates into S~, then factor the interfaces
+            RSD_TRY(h.lu ? run_factor_level_lu(h, nl - 1) : run_factor_level(h, nl - 1));
+            if (!h.lu) RSD_TRY(launch_factor_copy16(h, nl - 1));   // TF32 leaves: the copy their solves read
+            if (!gmode) {
+                RSD_TRY(paper_extend_add(h));
+                for (int d = nl - 2; d >= 0; --d) RSD_TRY(run_factor_level(h, d));
+            }
         }
-        h.prof.host_issue_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t_issue).count();
-    } else {
-        // every interface front is K_II plus leaf updates: factor the leaves, scatter
-        // their updates into S~, then factor the interfaces
-        RSD_TRY(h.lu ? run_factor_level_lu(h, nl - 1) : run_factor_level(h, nl - 1));
-        if (!h.lu) RSD_TRY(launch_factor_copy16(h, nl - 1));   // TF32 leaves: the copy their solves read
-        if (!gmode) {
-            RSD_TRY(paper_extend_add(h));
-            for (int d = nl - 2; d >= 0; --d) RSD_TRY(run_factor_level(h, d));
-        }
-    }
-    RSD_CUDA_TRY(cudaStreamSynchronize(st));
-    stage_reset(h);                                   // every staged upload has completed
+        RSD_CUDA_TRY(cudaStreamSynchronize(st));
+        stage_reset(h);                               // every staged upload has completed
+        return RSD_OK;
+    };
+    RSD_TRY(factor_all());
     int err[ERR_SLOTS];
     RSD_CUDA_TRY(cudaMemcpy(err, h.d_err, sizeof(err), cudaMemcpyDeviceToHost));
+    if (err[ERR_SPREAD]) {
+        // nonsymmetric FP64 fronts whose scales the split products do not fit: everything
+        // again, FP64 levels on the FP64 pipe (what depends on their Schur contributions, a
+        // pivot that failed included, may have come from lost digits)
+        h.f64_ws = nullptr;
+        const int clear[ERR_SLOTS] = {0, 0, 0x7fffffff, 0};
+        RSD_CUDA_TRY(cudaMemcpyAsync(h.d_err, stage_host(h, clear, sizeof(clear)), sizeof(clear), cudaMemcpyHostToDevice, st));
+        RSD_CUDA_TRY(cudaMemsetAsync(h.d_front_bad, 0, sizeof(int) * a.n_nodes, st));
+        RSD_TRY(factor_all());
+        RSD_CUDA_TRY(cudaMemcpy(err, h.d_err, sizeof(err), cudaMemcpyDeviceToHost));
+    }
     if (err[ERR_NOT_SPD] && !paper && !h.lu) {
         RSD_TRY(promote_failed_fronts(h, d_owner, d_rank, d_tin, d_tout));
         RSD_CUDA_TRY(cudaStreamSynchronize(st));

@@ -14,7 +14,7 @@
 // F_BI) and PU (entries above it, transposed, and F_IB transposed).
 //
 // FP64 levels run in gemm_f64_tc.cu (and diag_f64.cu) unless the arena had no room for its
-// workspace.  Here, left-looking by NB-column blocks k (CUDA cores, FP32 or FP64):
+// workspace or the entries spread too far in scale for its products.  Here, left-looking by NB-column blocks k (CUDA cores, FP32 or FP64):
 //   (a) P[k:N, blk]    -= P[k:N, 0:k]    PU[blk, 0:k]^T   (L and X columns, with the
 //                                                          diagonal block's lower part)
 //   (b) PU[k:N, blk]   -= PU[k:N, 0:k]   P[blk, 0:k]^T    (U^T and Y^T columns, with the

@@ -28,6 +28,24 @@
 // complement that cancels to 1e-7 of its terms is off by half a unit of those terms (rms), by 2 to 5
 // units with FMAs.
 //
+// Scale.  One exponent a row is safe for Cholesky: with K = D K0 D the entries of row i of
+// [L; X] all scale with D_i, and |l_ik| <= sqrt(K_ii).  LU is not like that: with K = Dr K0 Dc
+// an entry of [L; X] scales with Dr_i / Dr_k and one of [U^T; Y^T] with Dr_k Dc_j, so along
+// the columns k of a panel the operands' scales run opposite ways, and what an entry 2^-59
+// below its row's largest loses is not small beside the product.  So column k of [L; X] is
+// split times 2^t_k and column k of [U^T; Y^T] times 2^-t_k (exact, and nothing to undo in
+// the product), t_k the exponent of Dr_k as the pivot u_kk = Dr_k Dc_k gives it: half of its
+// exponent (rows and columns scaled alike, the Galerkin case), all of it (scaled equations) or
+// none of it (scaled unknowns), whichever of the three fits the entries of K best beside its
+// diagonal (lu_scaling).  The operands of the panel solves are scaled to match.
+// No power of two fits every Dr and Dc, so each split row is held against the scale that the
+// same choice gives its diagonal entry of K: rows up to 2^SPREAD_MAX above it keep the
+// error of a product below 2^(2 SPREAD_MAX - 59) Dr_i Dc_j (Cholesky's bound has 0 there); one
+// further up raises ERR_SPREAD, and the setup factors the hierarchy again on the FP64 pipe.
+// Fronts of 300 diagonally dominant unknowns with rows, or rows and columns, scaled over
+// 2^-40 .. 2^40: entries of L wrong by 4e-3 with t_k = 0, now as the unscaled fronts'.  A 37^3
+// convection-diffusion system: 16.41 -> 16.49 ms.
+//
 // Kernel.  A 128 x 64 tile keeps its eight sums in TMEM (8 x 64 columns, all 512).  Digit
 // rows of B are stacked in shared memory, so one MMA of N = 256 multiplies digit i of A by
 // four digits of B and adds into four adjacent sums.  For 64 columns of K the eight digit
@@ -43,6 +61,7 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <climits>
 #include <vector>
 
 #include "rsd_internal.cuh"
@@ -92,6 +111,7 @@ struct F64Front {
     int *ex, *aex, *dex;                     // row exponents of X, A and Dinv_k
     int* sq;                                 // per row of X: sum of digit 4 squared
     float* n2;                               // per row of X: sum of (x 2^-ex)^2
+    int* tk;                                 // nonsymmetric: t_k of the panel's columns
     int nrt;
 };
 
@@ -204,6 +224,66 @@ __device__ __forceinline__ void mark_bad(int node, int* err, int* bad_front) {
     bad_front[node] = 1;
 }
 
+// ---- scale of nonsymmetric fronts ----------------------------------------------------------
+
+constexpr int SPREAD_MAX = 4;                // see above: 2^-51 Dr_i Dc_j in the worst case
+
+// Which power of the diagonal goes to the equations: 0 half of its exponent, 1 all, -1 none.
+// w[q]: how far the largest entry of K lies above its place under q = 0, 1, -1 (in bits).
+__device__ __forceinline__ int lu_scaling(const int* __restrict__ w) {
+    const int w1 = w[1], w2 = w[2];
+    return w[0] > min(w1, w2) + 1 ? (w1 <= w2 ? 1 : -1) : 0;
+}
+// exponents of Dr and Dc for a diagonal entry (or pivot) of exponent e
+__device__ __forceinline__ int lu_row_exp(int q, int e) { return ((1 + q) * e) >> 1; }
+__device__ __forceinline__ int lu_col_exp(int q, int e) { return ((1 - q) * e) >> 1; }
+
+__global__ void k_lu_diag_exp(int n, const int64_t* __restrict__ rowptr, const int* __restrict__ col, const double* __restrict__ val,
+                              int* __restrict__ de) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    int64_t a = rowptr[i], e = rowptr[i + 1];
+    const int64_t end = e;
+    while (a < e) {
+        const int64_t mid = (a + e) >> 1;
+        if (col[mid] < i) a = mid + 1; else e = mid;
+    }
+    int ok = 1;
+    de[i] = a < end && col[a] == i ? exp_above(val[a], &ok) : E_NONE;
+}
+
+// largest exponent of an entry of K above Dr_i Dc_j, for the three choices; a warp a row
+__global__ void __launch_bounds__(256) k_lu_spread(int n, const int64_t* __restrict__ rowptr, const int* __restrict__ col,
+                                                  const double* __restrict__ val, const int* __restrict__ de, int* __restrict__ w) {
+    __shared__ int s_w[3];
+    if (threadIdx.x < 3) s_w[threadIdx.x] = INT_MIN;
+    __syncthreads();
+    const int lane = threadIdx.x & 31, warps = (int)(gridDim.x * (blockDim.x >> 5));
+    int m[3] = {INT_MIN, INT_MIN, INT_MIN};
+    for (int i = (int)(blockIdx.x * (blockDim.x >> 5)) + (threadIdx.x >> 5); i < n; i += warps) {
+        const int di = de[i];
+        if (di == E_NONE) continue;
+        for (int64_t k = rowptr[i] + lane; k < rowptr[i + 1]; k += 32) {
+            int ok = 1;
+            const int e = exp_above(val[k], &ok), dj = de[col[k]];
+            if (e == E_NONE || !ok || dj == E_NONE) continue;
+#pragma unroll
+            for (int h = 0; h < 3; ++h) {
+                const int q = h == 2 ? -1 : h;
+                m[h] = max(m[h], e - lu_row_exp(q, di) - lu_col_exp(q, dj));
+            }
+        }
+    }
+#pragma unroll
+    for (int h = 0; h < 3; ++h) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) m[h] = max(m[h], __shfl_xor_sync(0xffffffffu, m[h], o));
+        if (lane == 0) atomicMax(&s_w[h], m[h]);
+    }
+    __syncthreads();
+    if (threadIdx.x < 3) atomicMax(&w[threadIdx.x], s_w[threadIdx.x]);
+}
+
 // ---- splitting -----------------------------------------------------------------------------
 // Half a warp takes a row and 128 columns, eight adjacent columns (one 16-byte chunk per
 // digit) to a lane.  HBM-bound: 8 bytes read and 16 written per entry.
@@ -242,12 +322,21 @@ __device__ __forceinline__ int store_digits(const double (&x)[8], const int (&e)
     return sq;
 }
 
+// scale of row r of [L; X] (Dr) or of [U^T; Y^T] (Dc), from its diagonal entry of K
+__device__ __forceinline__ int row_scale(const FrontDesc& f, int r, bool upper, int sc, const int* __restrict__ de) {
+    const int d = de[r < f.s ? f.I[r] : f.Bd[r - f.s]];
+    return upper ? lu_col_exp(sc, d) : lu_row_exp(sc, d);
+}
+
 // Operands of the panel solve at block column k: A_ij 2^-s_j (rows below the diagonal
 // block) and Dinv_cj 2^s_j, s_j the exponent of L_jj (a row's entries then compare across
-// columns of different scale).  blockIdx.x < na: SA_ROWS rows of A, else of Dinv.
-// Nonsymmetric fronts, blockIdx.z = 0: P against (U_kk^T)^-1, s_j of U_jj; 1: PU against L_kk^-1.
+// columns of different scale).  blockIdx.x < na: nr rows of A, else of Dinv.
+// Nonsymmetric fronts, blockIdx.z = 0: P against (U_kk^T)^-1, s_j the exponent of Dc_j; 1: PU
+// against L_kk^-1, s_j that of Dr_j, which is the column's t_k too (de, the exponents of K's
+// diagonal, and sw as launch_lu_scale left them; null for symmetric fronts).
 __global__ void __launch_bounds__(256) k_split_a(const FrontDesc* __restrict__ fronts, const F64Front* __restrict__ wk, int k,
-                                                int na, int nr, int* __restrict__ err, int* __restrict__ bad_front) {
+                                                int K0, int na, int nr, const int* __restrict__ de, const int* __restrict__ sw,
+                                                int* __restrict__ err, int* __restrict__ bad_front) {
     __shared__ int sj[NB];
     const FrontDesc f = fronts[blockIdx.y];
     if (f.s <= k) return;
@@ -258,10 +347,16 @@ __global__ void __launch_bounds__(256) k_split_a(const FrontDesc* __restrict__ f
     const F64Front wf = wk[gridDim.z * blockIdx.y + blockIdx.z];
     const bool lu = gridDim.z == 2, upper = blockIdx.z == 1;
     const double* P = (const double*)(upper ? f.PU : f.P);
-    const double* diag = (const double*)(lu && !upper ? f.PU : f.P);
+    const double* diag = (const double*)(lu ? f.PU : f.P);       // u_jj or l_jj
     const double* Dk = (const double*)(lu && !upper ? f.DinvU : f.Dinv) + (int64_t)(k / NB) * NB * NB;
-    int ok = 1;
-    if (threadIdx.x < NB) sj[threadIdx.x] = (int)threadIdx.x < w ? exp_above(diag[(int64_t)(k + threadIdx.x) * f.ldp + k + threadIdx.x], &ok) : 0;
+    const int sc = lu ? lu_scaling(sw) : 0;
+    int ok = 1, spread = 0;
+    if (threadIdx.x < NB) {
+        int e = (int)threadIdx.x < w ? exp_above(diag[(int64_t)(k + threadIdx.x) * f.ldp + k + threadIdx.x], &ok) : 0;
+        if (lu) e = upper ? lu_row_exp(sc, e) : lu_col_exp(sc, e);
+        sj[threadIdx.x] = e;
+        if (lu && upper && blockIdx.x == 0) wf.tk[k - K0 + threadIdx.x] = e;
+    }
     __syncthreads();
 #pragma unroll 1
     for (int r = r0 + (threadIdx.x >> 4); r < r0 + nr; r += 16) {
@@ -284,15 +379,19 @@ __global__ void __launch_bounds__(256) k_split_a(const FrontDesc* __restrict__ f
             store_digits<SLV_DB, SLV_FB>(x, e, dst, (int64_t)(isA ? wf.nrt : 2) * GROUP, r & 63, ch);
             if (ch == 0) (isA ? wf.aex : wf.dex)[r] = top;
         }
+        if (lu && isA && in) spread |= top > row_scale(f, r, upper, sc, de) + SPREAD_MAX;
     }
     if (!ok) mark_bad(f.node, err, bad_front);
+    else if (spread) err[ERR_SPREAD] = 1;
 }
 
 // Digits of the solved rows X of block column k for the updates that follow, the panel's
 // columns K0 .. k + w of a row on one exponent (from the largest entry and the norm):
-// where the new block raises it, the row's earlier blocks are split again.
+// where the new block raises it, the row's earlier blocks are split again.  Nonsymmetric fronts:
+// column c times 2^t_c on side 0, 2^-t_c on side 1.
 __global__ void __launch_bounds__(256) k_split_x(const FrontDesc* __restrict__ fronts, const F64Front* __restrict__ wk, int k,
-                                                int K0, int* __restrict__ err, int* __restrict__ bad_front) {
+                                                int K0, const int* __restrict__ de, const int* __restrict__ sw,
+                                                int* __restrict__ err, int* __restrict__ bad_front) {
     const FrontDesc f = fronts[blockIdx.y];
     if (f.s <= k) return;
     const F64Front wf = wk[gridDim.z * blockIdx.y + blockIdx.z];
@@ -301,19 +400,23 @@ __global__ void __launch_bounds__(256) k_split_x(const FrontDesc* __restrict__ f
     const int r = k + w + (int)blockIdx.x * 16 + (threadIdx.x >> 4);
     const bool in = r < f.N;
     const double* src = (const double*)(blockIdx.z ? f.PU : f.P) + (int64_t)r * f.ldp + j0;
-    int ok = 1, top = E_NONE;
+    const bool lu = gridDim.z == 2;
+    const int sign = blockIdx.z ? -1 : 1;
+    int ok = 1, top = E_NONE, t[8];
     double x[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
         x[q] = in && j0 + q < w ? src[k + q] : 0.0;
-        top = max(top, exp_above(x[q], &ok));
+        t[q] = lu ? sign * wf.tk[k - K0 + j0 + q] : 0;
+        const int ex = exp_above(x[q], &ok);
+        if (ex != E_NONE) top = max(top, ex + t[q]);
     }
     top = half_warp_max(top);
     const int old = in && k > K0 ? wf.ex[r] : E_NONE;
     top = max(top, old);
     float n2 = 0.f;
 #pragma unroll
-    for (int q = 0; q < 8; ++q) n2 += square_scaled(x[q], top);
+    for (int q = 0; q < 8; ++q) n2 += square_scaled(x[q], top - t[q]);
 #pragma unroll
     for (int o = 8; o > 0; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
     if (in && k > K0) n2 += wf.n2[r] * exp2f((float)(2 * max(old - top, -60)));
@@ -322,14 +425,17 @@ __global__ void __launch_bounds__(256) k_split_x(const FrontDesc* __restrict__ f
     if (in) {
         int e[8];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) e[q] = top;
+        for (int q = 0; q < 8; ++q) e[q] = top - t[q];
         const int64_t stride = (int64_t)wf.nrt * GROUP;
         char* dst = wf.XS + (int64_t)(r >> 6) * GROUP;
         sq = store_digits<UPD_DB, UPD_FB>(x, e, dst + (k - K0) / KB * stride, stride, r & 63, ch);
         if (top > old)
             for (int c = K0; c < k; c += NB) {
 #pragma unroll
-                for (int q = 0; q < 8; ++q) x[q] = src[c + q];
+                for (int q = 0; q < 8; ++q) {
+                    x[q] = src[c + q];
+                    e[q] = lu ? top - sign * wf.tk[c - K0 + j0 + q] : top;
+                }
                 sq += store_digits<UPD_DB, UPD_FB>(x, e, dst + (c - K0) / KB * stride, stride, r & 63, ch);
             }
     }
@@ -340,6 +446,7 @@ __global__ void __launch_bounds__(256) k_split_x(const FrontDesc* __restrict__ f
         wf.sq[r] = k > K0 && top == old ? wf.sq[r] + sq : sq;
     }
     if (!ok) mark_bad(f.node, err, bad_front);
+    else if (lu && in && top > row_scale(f, r, blockIdx.z, lu_scaling(sw), de) + SPREAD_MAX) err[ERR_SPREAD] = 1;
 }
 
 // ---- the GEMM ------------------------------------------------------------------------------
@@ -593,7 +700,7 @@ int row_tiles(int N) { return 2 * ((N + BM - 1) / BM); }
 
 size_t front_bytes(int N) {
     const size_t g = (size_t)row_tiles(N) * GROUP;
-    return (WP / KB + 2) * g + 4 * (size_t)GROUP + 4 * al(sizeof(int) * (size_t)N) + al(sizeof(int) * NB);
+    return (WP / KB + 2) * g + 4 * (size_t)GROUP + 4 * al(sizeof(int) * (size_t)N) + al(sizeof(int) * NB) + al(sizeof(int) * WP);
 }
 
 // tiles of W columns covering the task's rows and columns
@@ -607,6 +714,19 @@ int64_t set_tiles(F64Task& t, int W) {
 }
 
 }  // namespace
+
+int launch_lu_scale(Handle& h) {
+    cudaStream_t st = h.stream;
+    const int pi = prof_begin(h, K_ASSEMBLE, st);
+    RSD_CUDA_TRY(cudaMemsetAsync(h.d_lu_scale + h.n, 0x80, sizeof(int) * LU_SCALE_EXTRA, st));       // far below any exponent
+    k_lu_diag_exp<<<(unsigned)((h.n + 255) / 256), 256, 0, st>>>(h.n, h.d_rowptr, h.d_col, h.d_val, h.d_lu_scale);
+    k_lu_spread<<<(unsigned)std::min((h.n + 7) / 8, 8 * h.num_sms), 256, 0, st>>>(h.n, h.d_rowptr, h.d_col, h.d_val, h.d_lu_scale,
+                                                                                h.d_lu_scale + h.n);
+    count_launch(2);
+    prof_end(h, pi, 0.0, 12.0 * h.nnz, st);
+    RSD_CUDA_TRY(cudaGetLastError());
+    return RSD_OK;
+}
 
 // Workspace of a level: the digits of one 512-wide panel of every front at once where that
 // fits the cap (groups of fronts then take turns), of one front at least.  The cap is far
@@ -651,7 +771,8 @@ int factor_level_f64_tc(Handle& h, int li) {
                 w.sq = (int*)p; p += al(sizeof(int) * (size_t)f.N);
                 w.n2 = (float*)p; p += al(sizeof(float) * (size_t)f.N);
                 w.aex = (int*)p; p += al(sizeof(int) * (size_t)f.N);
-                w.dex = (int*)p;
+                w.dex = (int*)p; p += al(sizeof(int) * NB);
+                w.tk = sd ? wk[(size_t)(f0 + g.nf) * sides].tk : (int*)p;      // both sides' columns
                 off += need;
             }
             g.max_s = std::max(g.max_s, f.s);
@@ -775,6 +896,8 @@ int factor_level_f64_tc(Handle& h, int li) {
     for (int few = 0; few < 2; ++few)
         for (int sv = 0; sv < 2; ++sv)
             RSD_CUDA_TRY(cudaFuncSetAttribute(kern[few][sv], cudaFuncAttributeMaxDynamicSharedMemorySize, smem[few]));
+    const int* de = h.lu ? h.d_lu_scale : nullptr;
+    const int* sw = h.lu ? h.d_lu_scale + h.n : nullptr;
     size_t li_ = 0;
     auto run = [&]() -> int {
         const Launch& l = launches[li_++];
@@ -806,12 +929,13 @@ int factor_level_f64_tc(Handle& h, int li) {
             auto split = [&](bool x) -> int {
                 if (!rows) return RSD_OK;
                 const int pi = prof_begin(h, K_COPY16, st);
-                if (x) k_split_x<<<dim3((unsigned)((rows + 15) / 16), (unsigned)g.nf, (unsigned)sides), 256, 0, st>>>(d_fr, d_wk + (size_t)g.f0 * sides, k, K0, h.d_err, h.d_front_bad);
+                if (x) k_split_x<<<dim3((unsigned)((rows + 15) / 16), (unsigned)g.nf, (unsigned)sides), 256, 0, st>>>(
+                           d_fr, d_wk + (size_t)g.f0 * sides, k, K0, de, sw, h.d_err, h.d_front_bad);
                 else {
                     // 64 rows a CTA share the load of s_j; with few CTAs 16, for the shorter chain
                     const int nr = (rows + 63) / 64 * g.nf * sides > h.num_sms ? 64 : 16, na = (rows + nr - 1) / nr;
                     k_split_a<<<dim3((unsigned)(na + NB / nr), (unsigned)g.nf, (unsigned)sides), 256, 0, st>>>(
-                        d_fr, d_wk + (size_t)g.f0 * sides, k, na, nr, h.d_err, h.d_front_bad);
+                        d_fr, d_wk + (size_t)g.f0 * sides, k, K0, na, nr, de, sw, h.d_err, h.d_front_bad);
                 }
                 count_launch();
                 prof_end(h, pi, 0.0, bytes, st);

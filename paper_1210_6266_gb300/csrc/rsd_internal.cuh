@@ -15,7 +15,9 @@ namespace rsd {
 constexpr int NB = 128;
 
 // Device-side error flags (one int array per handle).
-enum ErrSlot { ERR_NOT_SPD = 0, ERR_TIMEOUT = 1, ERR_NOT_SPD_NODE = 2, ERR_SLOTS = 4 };
+// ERR_SPREAD: a nonsymmetric FP64 front's entries spread too far in scale for the split
+// products (gemm_f64_tc.cu); the setup then factors the hierarchy again without them.
+enum ErrSlot { ERR_NOT_SPD = 0, ERR_TIMEOUT = 1, ERR_NOT_SPD_NODE = 2, ERR_SPREAD = 3, ERR_SLOTS = 4 };
 
 #define RSD_CUDA_TRY(expr)                                           \
     do {                                                             \
@@ -228,6 +230,7 @@ struct Handle {
     // the arena only fits without it (those fronts then run on the FP64 pipe)
     char* f64_ws = nullptr;
     size_t f64_ws_bytes = 0;
+    int* d_lu_scale = nullptr;           // nonsymmetric FP64 fronts: see launch_lu_scale
     char* tc_ws = nullptr;               // scratch of a tensor-core level (factor_tc_workspace), or null
     size_t tc_ws_bytes = 0;
     int* d_err = nullptr;
@@ -389,6 +392,10 @@ int launch_diag_f64(Handle& h, int li, int f0, int nf, int k, cudaStream_t st);
 // counts, and the partial Cholesky or LU of the level (needs the handle's f64_ws)
 size_t f64_tc_workspace(const std::vector<int>& rows, bool lu);
 int factor_level_f64_tc(Handle& h, int li);
+// nonsymmetric K: the exponents of its diagonal (n ints) and LU_SCALE_EXTRA more for the
+// choice of the scaling its split products use, to h.d_lu_scale
+constexpr int LU_SCALE_EXTRA = 4;
+int launch_lu_scale(Handle& h);
 // nonsymmetric fronts: assembly, extend-add and LU partial factorisation of level li
 int launch_assemble_fronts_lu(Handle& h, int li, const int64_t* rowptr, const int* col, const double* val,
                               const int* owner, const int* rank, const int* tin, const int* tout);
