@@ -292,6 +292,12 @@ int rsd_solve_adjoint(rsd_handle h, const double* g, double* lam, double tol, rs
  * RSD_ERR_ARG for a bad level or a paper-mode handle.                                  */
 int rsd_inject_drop_sweep_item(rsd_handle h, int32_t level);
 
+/* rsd_inject_setup_timeout -- as above for the factorisation: the next rsd_setup (or
+ * rsd_setup_batched) of the calling thread starts with the timeout flag raised, so that
+ * every wait of its tensor-core GEMMs that is not met at once gives up.  Their CTAs let
+ * what they have in flight land and leave; the CUDA context stays usable.              */
+int rsd_inject_setup_timeout(void);
+
 /* rsd_check -- synchronise the handle's stream and report any device-side error flag
  * (timeout of a bounded wait, failed pivot) raised since setup.                        */
 int rsd_check(rsd_handle h);

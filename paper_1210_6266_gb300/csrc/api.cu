@@ -31,6 +31,9 @@ void set_last_error(const std::string& msg) { g_last_error = msg; }
 
 static std::atomic<long long> g_launches(0);
 
+// rsd_inject_setup_timeout: the calling thread's next rsd_setup (taken by build_handle)
+static thread_local bool t_inject_setup_timeout = false;
+
 // One cached arena per device: rsd_destroy parks its arena here instead of freeing it and
 // the next rsd_setup on that device reuses it when it is large enough (the arena of a
 // factorisation is tens of GB; mapping and unmapping it costs tens of milliseconds).
@@ -755,6 +758,8 @@ static int promote_failed_fronts(Handle& h, int* d_owner, int* d_rank, int* d_ti
 
 // Build the handle's levels, memory plan and device copies from an analysis.
 static int build_handle(Handle& h, Analysis& a, const int64_t* rowptr, const int* col, const double* val) {
+    const bool inject_timeout = t_inject_setup_timeout;
+    t_inject_setup_timeout = false;
     const auto t_plan = std::chrono::steady_clock::now();
     h.n = a.n;
     h.n_nodes = a.n_nodes;
@@ -1122,6 +1127,7 @@ static int build_handle(Handle& h, Analysis& a, const int64_t* rowptr, const int
     RSD_CUDA_TRY(cudaMemcpyAsync(d_gptr, stage_host(h, gptr_all.data(), sizeof(int) * gptr_all.size()), sizeof(int) * gptr_all.size(), cudaMemcpyHostToDevice, st));
     RSD_CUDA_TRY(cudaMemcpyAsync(d_gsrc, stage_host(h, gsrc_all.data(), sizeof(int2) * gsrc_all.size()), sizeof(int2) * gsrc_all.size(), cudaMemcpyHostToDevice, st));
     RSD_CUDA_TRY(cudaMemsetAsync(h.d_err, 0, sizeof(int) * ERR_SLOTS, st));
+    if (inject_timeout) RSD_CUDA_TRY(cudaMemsetAsync(h.d_err + ERR_TIMEOUT, 1, sizeof(int), st));
     RSD_CUDA_TRY(cudaMemsetAsync(h.d_front_bad, 0, sizeof(int) * a.n_nodes, st));
     {
         const int big = 0x7fffffff;
@@ -1665,6 +1671,11 @@ extern "C" int rsd_peak_gemm(int32_t prec, int32_t n, int32_t reps, double secon
 extern "C" int rsd_inject_drop_sweep_item(rsd_handle hh, int32_t level) {
     if (!hh || hh->h.paper || level < 0 || level >= (int)hh->h.levels.size()) return RSD_ERR_ARG;
     hh->h.inject_drop_level = level;
+    return RSD_OK;
+}
+
+extern "C" int rsd_inject_setup_timeout(void) {
+    t_inject_setup_timeout = true;
     return RSD_OK;
 }
 

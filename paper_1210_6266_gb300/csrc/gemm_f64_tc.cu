@@ -528,10 +528,10 @@ k_gemm_f64_tc(const F64Task* __restrict__ tasks, int ntask, int n_tiles, int* __
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tmem_slot;
 
+    bool ok = true;                          // no wait of this thread has given up
     if (warp == 0) {
         if (lane == 0) {
             uint32_t ia = 0, ib = 0;
-            bool ok = true;
             for (int g = blockIdx.x; g < n_tiles && ok; g += gridDim.x) {
                 int tm, tn;
                 const F64Task& t = tasks[f64_tile<W>(tasks, ntask, g, &tm, &tn)];
@@ -561,19 +561,14 @@ k_gemm_f64_tc(const F64Task* __restrict__ tasks, int ntask, int n_tiles, int* __
                     }
                 }
             }
-            if (!ok) {                       // a wait gave up: the copies and MMAs in flight land first
-                const long long t0 = clock64();
-                while (clock64() - t0 < 4000000ll) __nanosleep(1000);
-            }
         }
     } else if (warp == 1) {
         if (lane == 0) {
             uint32_t ia = 0, ib = 0, it = 0;
-            bool ok = true;
             for (int g = blockIdx.x; g < n_tiles && ok; g += gridDim.x, ++it) {
                 int tm, tn;
                 const int nkb = tasks[f64_tile<W>(tasks, ntask, g, &tm, &tn)].nkb;
-                if (!mbar_wait(acc_empty, (it & 1) ^ 1, err)) break;
+                if (!mbar_wait(acc_empty, (it & 1) ^ 1, err)) { ok = false; break; }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 for (int kb = 0; kb < nkb && ok; ++kb, ++ib) {
                     const uint32_t q = ib & 1;
@@ -616,7 +611,7 @@ k_gemm_f64_tc(const F64Task* __restrict__ tasks, int ntask, int n_tiles, int* __
             double* P = t.P + (int64_t)gr * t.ldp;
             double* U = t.U + (int64_t)(gr - s) * t.ldu - s;
             if (!SOLVE && in && c_base >= c_lo) asm volatile("prefetch.global.L2 [%0];" ::"l"(c_base < s ? P + c_base : U + c_base));
-            if (!__all_sync(0xffffffffu, mbar_wait(acc_full, it & 1, err))) break;
+            if (!__all_sync(0xffffffffu, mbar_wait(acc_full, it & 1, err))) { ok = false; break; }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             long long a1[CW];
             uint32_t a0[CW];
@@ -688,8 +683,9 @@ k_gemm_f64_tc(const F64Task* __restrict__ tasks, int ntask, int n_tiles, int* __
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
+    const bool gave_up = __syncthreads_or(!ok);
     if (warp == 1) {
+        if (gave_up) settle_in_flight();
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ND * W) : "memory");
     }

@@ -265,6 +265,7 @@ k_gemm_tc(const TcTask* __restrict__ tasks, const TcTile* __restrict__ tiles,
     grid_dep_wait();
     grid_dep_launch();
 
+    bool ok = true;                          // no wait of this thread has given up
     if (warp == 0) {
         if (lane == 0) {
             const CUtensorMap* ma = maps + tk.map_a;
@@ -272,7 +273,7 @@ k_gemm_tc(const TcTask* __restrict__ tasks, const TcTile* __restrict__ tiles,
             for (int kb = 0; kb < nk; ++kb) {
                 const int s = kb % STAGES;
                 const uint32_t ph = (kb / STAGES) & 1;
-                if (!mbar_wait(bar_empty + 8 * s, ph ^ 1, err)) break;
+                if (!mbar_wait(bar_empty + 8 * s, ph ^ 1, err)) { ok = false; break; }
                 const uint32_t sa = base + s * S::STAGE;
                 const uint32_t sb = sa + S::A_BYTES;
                 mbar_expect_tx(bar_full + 8 * s, S::STAGE);
@@ -286,7 +287,6 @@ k_gemm_tc(const TcTask* __restrict__ tasks, const TcTile* __restrict__ tiles,
     } else if (warp == 1) {
         if (lane == 0) {
             constexpr uint32_t idesc = idesc_tf32(BN);
-            bool ok = true;
             for (int kb = 0; kb < nk && ok; ++kb) {
                 const int s = kb % STAGES;
                 const uint32_t ph = (kb / STAGES) & 1;
@@ -315,13 +315,14 @@ k_gemm_tc(const TcTask* __restrict__ tasks, const TcTile* __restrict__ tiles,
                                             sbase + quarter * 4096, m0 + quarter * 32, n0, lane};
         float4 cur[8];
         ep.fetch(0, cur);
-        const bool ok = mbar_wait(bar_done, 0, err);
+        ok = __all_sync(0xffffffffu, mbar_wait(bar_done, 0, err));      // (what follows is the whole warp's)
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         ep.run(tmem + ((uint32_t)(quarter * 32) << 16), 0, BN, cur, ok);
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     }
-    __syncthreads();
+    const bool gave_up = __syncthreads_or(!ok);
     if (warp == 1) {
+        if (gave_up) settle_in_flight();
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(BN) : "memory");
     }
@@ -373,10 +374,10 @@ k_gemm_tc_persist(const TcTask* __restrict__ tasks, const TcTile* __restrict__ t
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tmem_slot;
 
+    bool ok = true;                          // no wait of this thread has given up
     if (warp == 0) {
         if (lane == 0) {
             uint32_t it = 0;
-            bool ok = true;
             for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
                 const TcTile tl = tiles[t];
                 const TcTask tk = tasks[tl.task];
@@ -402,7 +403,6 @@ k_gemm_tc_persist(const TcTask* __restrict__ tasks, const TcTile* __restrict__ t
         if (lane == 0) {
             constexpr uint32_t idesc = idesc_of(OpT<OP>::FMT, BN);
             uint32_t it = 0, tcount = 0;
-            bool ok = true;
             for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x, ++tcount) {
                 const TcTile tl = tiles[t];
                 const uint32_t buf = tcount & 1, use = (tcount >> 1) & 1;
@@ -442,16 +442,18 @@ k_gemm_tc_persist(const TcTask* __restrict__ tasks, const TcTile* __restrict__ t
                                         sbase + STAGES * S::STAGE + S::EPI + (warp - 2) * 4096, m0 + quarter * 32, n0, lane};
             float4 cur[8];
             ep.fetch(cb, cur);
-            const bool ok = mbar_wait(bar_accf + 8 * buf, use, err);
+            const bool full = __all_sync(0xffffffffu, mbar_wait(bar_accf + 8 * buf, use, err));     // (whole warps below)
+            ok = ok && full;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            ep.run(tmem + buf * BN + ((uint32_t)(quarter * 32) << 16), cb, ce, cur, ok);
+            ep.run(tmem + buf * BN + ((uint32_t)(quarter * 32) << 16), cb, ce, cur, full);
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar_acce + 8 * buf) : "memory");
         }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     }
-    __syncthreads();
+    const bool gave_up = __syncthreads_or(!ok);
     if (warp == 1) {
+        if (gave_up) settle_in_flight();
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * BN) : "memory");
     }

@@ -48,6 +48,13 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* er
     return true;
 }
 
+// End of a GEMM kernel of which a wait gave up: the CTA's own copies and MMAs still in flight
+// land (about 2 ms, a thousand times what one takes) before TMEM is freed and the CTA leaves.
+__device__ __forceinline__ void settle_in_flight() {
+    const long long t0 = clock64();
+    while (clock64() - t0 < 4000000ll) __nanosleep(1000);
+}
+
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
     asm volatile(
         "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
