@@ -218,8 +218,9 @@ typedef struct rsd_handle_s* rsd_handle;
  * node's front from K and its children's Schur contributions, factor the interface block
  * and form the Schur contribution to the ancestors (Eq. 3.2).  All numeric work runs
  * in this library's CUDA kernels on opt->stream; the call returns after the stream has
- * drained and reports RSD_ERR_NOT_SPD if any pivot failed.  The caller may free K,
- * dof_node and T as soon as the call returns.                                         */
+ * drained and reports RSD_ERR_NOT_SPD if any pivot failed, RSD_ERR_TIMEOUT (and no handle)
+ * if a bounded wait of the factorisation gave up.  The caller may free K, dof_node and T
+ * as soon as the call returns.                                                        */
 int rsd_setup(const rsd_csr* K, const int32_t* dof_node, const rsd_tree* T,
               const rsd_options* opt, rsd_handle* out);
 
@@ -295,7 +296,8 @@ int rsd_inject_drop_sweep_item(rsd_handle h, int32_t level);
 /* rsd_inject_setup_timeout -- as above for the factorisation: the next rsd_setup (or
  * rsd_setup_batched) of the calling thread starts with the timeout flag raised, so that
  * every wait of its tensor-core GEMMs that is not met at once gives up.  Their CTAs let
- * what they have in flight land and leave; the CUDA context stays usable.              */
+ * what they have in flight land and leave, the call returns RSD_ERR_TIMEOUT, and the CUDA
+ * context stays usable.                                                               */
 int rsd_inject_setup_timeout(void);
 
 /* rsd_check -- synchronise the handle's stream and report any device-side error flag

@@ -1392,8 +1392,15 @@ static int build_handle(Handle& h, Analysis& a, const int64_t* rowptr, const int
         return RSD_OK;
     };
     RSD_TRY(factor_all());
+    // A wait of the factorisation that gave up leaves tiles undone and no factor to return;
+    // whatever else the flags say may follow from it.
     int err[ERR_SLOTS];
-    RSD_CUDA_TRY(cudaMemcpy(err, h.d_err, sizeof(err), cudaMemcpyDeviceToHost));
+    auto read_flags = [&]() -> int {
+        RSD_CUDA_TRY(cudaMemcpy(err, h.d_err, sizeof(err), cudaMemcpyDeviceToHost));
+        if (err[ERR_TIMEOUT]) set_last_error("a wait of the factorisation gave up");
+        return err[ERR_TIMEOUT] ? RSD_ERR_TIMEOUT : RSD_OK;
+    };
+    RSD_TRY(read_flags());
     if (err[ERR_SPREAD]) {
         // nonsymmetric FP64 fronts whose scales the split products do not fit: everything
         // again, FP64 levels on the FP64 pipe (what depends on their Schur contributions, a
@@ -1403,13 +1410,13 @@ static int build_handle(Handle& h, Analysis& a, const int64_t* rowptr, const int
         RSD_CUDA_TRY(cudaMemcpyAsync(h.d_err, stage_host(h, clear, sizeof(clear)), sizeof(clear), cudaMemcpyHostToDevice, st));
         RSD_CUDA_TRY(cudaMemsetAsync(h.d_front_bad, 0, sizeof(int) * a.n_nodes, st));
         RSD_TRY(factor_all());
-        RSD_CUDA_TRY(cudaMemcpy(err, h.d_err, sizeof(err), cudaMemcpyDeviceToHost));
+        RSD_TRY(read_flags());
     }
     if (err[ERR_NOT_SPD] && !paper && !h.lu) {
         RSD_TRY(promote_failed_fronts(h, d_owner, d_rank, d_tin, d_tout));
         RSD_CUDA_TRY(cudaStreamSynchronize(st));
         stage_reset(h);
-        RSD_CUDA_TRY(cudaMemcpy(err, h.d_err, sizeof(err), cudaMemcpyDeviceToHost));
+        RSD_TRY(read_flags());
     }
     if (err[ERR_NOT_SPD]) {
         h.notspd_node = err[ERR_NOT_SPD_NODE];

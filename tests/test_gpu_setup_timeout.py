@@ -1,5 +1,6 @@
 """Waits of the factorisation's tensor-core GEMMs that give up (rsd_inject_setup_timeout):
-the kernels finish and the CUDA context stays usable."""
+the kernels finish, rsd_setup returns RSD_ERR_TIMEOUT and no handle, and the CUDA context
+stays usable."""
 import numpy as np
 import pytest
 
@@ -33,10 +34,9 @@ def test_waits_of_the_factorisation_that_give_up(rsd, prec, n, depth, lu):
     z_ref = h.apply(prob["b"]).clone()
     h.close()
     assert lib.rsd_inject_setup_timeout() == 0
-    try:
-        setup().close()
-    except rsd.RSDError:
-        pass
+    with pytest.raises(rsd.RSDError) as e:
+        setup()
+    assert e.value.code == _lib.RSD_ERR_TIMEOUT
     torch.cuda.synchronize()                               # the kernels finished
     h = setup()
     assert torch.equal(h.apply(prob["b"]), z_ref)
