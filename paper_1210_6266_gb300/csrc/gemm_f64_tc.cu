@@ -117,20 +117,21 @@ struct F64Front {
 
 // ---- entry <-> digits --------------------------------------------------------------------
 
-constexpr int E_NONE = -1200;                // exponent of a row of zeros
+constexpr int E_NONE = -4000;                // exponent of a row of zeros (below any scaled entry's)
 
-// exponent e of a finite x: |x| < 2^e (E_NONE for zero and subnormals); *ok = 0 otherwise
+// exponent e of a finite x: |x| < 2^e (E_NONE for zero); *ok = 0 otherwise
 __device__ __forceinline__ int exp_above(double x, int* ok) {
-    const int ex = (int)((__double_as_longlong(x) >> 52) & 0x7ff);
+    const long long b = __double_as_longlong(x);
+    const int ex = (int)((b >> 52) & 0x7ff);
     if (ex == 0x7ff) *ok = 0;
-    return ex ? ex - 1022 : E_NONE;
+    return b << 1 ? ex - 1022 : E_NONE;                          // (2^-1022 for all subnormals: 59 bits hold every one)
 }
 
-// (x 2^-e)^2 for finite |x| < 2^e, to FP32 (below 2^-200: 0)
+// (x 2^-e)^2 for finite |x| < 2^e, to FP32 (below 2^-200: 0; a subnormal as 2^-1022 at least)
 __device__ __forceinline__ float square_scaled(double x, int e) {
     const long long b = __double_as_longlong(x);
-    const int f = (int)((b >> 52) & 0x7ff), ex = f - 1023 - e + 127;  // biased FP32 exponent of x 2^-e
-    if (f == 0 || ex <= 0) return 0.f;
+    const int f = max((int)((b >> 52) & 0x7ff), 1), ex = f - 1023 - e + 127;     // biased FP32 exponent of x 2^-e
+    if (!(b << 1) || ex <= 0) return 0.f;
     const float v = __int_as_float((ex << 23) | (int)((b >> 29) & 0x7fffff));
     return v * v;
 }
@@ -139,10 +140,10 @@ __device__ __forceinline__ float square_scaled(double x, int e) {
 template <int FB>
 __device__ __forceinline__ long long to_fixed(double x, int e) {
     const long long b = __double_as_longlong(x);
-    const int ex = (int)((b >> 52) & 0x7ff), sh = ex - 1075 + FB - e;     // |x| = m 2^(ex - 1075)
-    if (ex == 0 || ex == 0x7ff || sh < -54) return 0;
-    const unsigned long long m = ((unsigned long long)b & 0xfffffffffffffull) | 0x10000000000000ull;
-    const unsigned long long f = sh >= 0 ? m << min(sh, FB - 53) : (m + (1ull << (-sh - 1))) >> -sh;
+    const int eb = (int)((b >> 52) & 0x7ff), ex = max(eb, 1), sh = ex - 1075 + FB - e;     // |x| = m 2^(ex - 1075)
+    if (eb == 0x7ff || sh < -54) return 0;
+    const unsigned long long m = ((unsigned long long)b & 0xfffffffffffffull) | (eb ? 0x10000000000000ull : 0ull);
+    const unsigned long long f = sh >= 0 ? m << min(sh, 63) : (m + (1ull << (-sh - 1))) >> -sh;
     return b < 0 ? -(long long)f : (long long)f;
 }
 
@@ -190,7 +191,7 @@ __device__ __forceinline__ uint32_t pack_digits(int lo, int hi) {
     return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-// (a1 2^S + a0) 2^e rounded to FP64, 0 <= a0 < 2^S, |a1| < 2^60; below the normal range: 0
+// (a1 2^S + a0) 2^e rounded to FP64 (halves away from zero), 0 <= a0 < 2^S, |a1| < 2^60
 template <int S>
 __device__ __forceinline__ double from_fixed(long long a1, uint32_t a0, int e) {
     const long long sign = a1 & 0x8000000000000000ll;
@@ -207,10 +208,14 @@ __device__ __forceinline__ double from_fixed(long long a1, uint32_t a0, int e) {
         m <<= z;
         l = 64 + z;
     }
-    m = (m >> 11) + ((m >> 10) & 1);                              // 53 bits, 2^52 <= m <= 2^53
     const int be = 11 + S - l + e + 52 + 1022;                   // biased exponent - 1
-    if (be < 0) return 0.0;
-    if (be > 2044) return __longlong_as_double(sign | 0x7ff0000000000000ll);
+    if (be < 0) {                                                // subnormal: fewer bits
+        const int sh = min(11 - be, 65);
+        m = sh > 64 ? 0 : sh == 64 ? m >> 63 : (m >> sh) + ((m >> (sh - 1)) & 1);
+        return __longlong_as_double(sign | (long long)m);
+    }
+    m = (m >> 11) + ((m >> 10) & 1);                              // 53 bits, 2^52 <= m <= 2^53
+    if (be > 2045) return __longlong_as_double(sign | 0x7ff0000000000000ll);
     return __longlong_as_double(sign | (long long)(((unsigned long long)be << 52) + m));
 }
 
