@@ -306,7 +306,9 @@ int rsd_check(rsd_handle h);
 
 /* rsd_destroy -- release the handle.  Its device arena is kept in a one-slot per-device
  * cache and reused by the next rsd_setup on that device if large enough (the previously
- * cached block, if smaller, is freed); rsd_release_cache() frees the cached blocks.      */
+ * cached block, if smaller, is freed), and so is, from one rsd_setup to the next, the
+ * workspace of its factorisation (4 GiB at most; it gives way when another allocation of
+ * the library needs the room).  rsd_release_cache() frees the cached blocks.             */
 void        rsd_destroy(rsd_handle h);
 void        rsd_release_cache(void);
 const char* rsd_strerror(int code);

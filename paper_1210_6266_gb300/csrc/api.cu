@@ -41,6 +41,27 @@ static thread_local bool t_inject_setup_timeout = false;
 struct ArenaCache { char* ptr = nullptr; size_t bytes = 0; };
 static std::mutex g_cache_mu;
 static ArenaCache g_cache[64];
+// and one factorisation workspace per device (SetupWorkspace below)
+static ArenaCache g_ws_cache[64];
+
+// cudaMalloc on the current device; a parked workspace gives way to it.
+cudaError_t device_malloc(void** p, size_t bytes) {
+    const cudaError_t rc = cudaMalloc(p, bytes);
+    if (rc == cudaSuccess) return rc;
+    cudaGetLastError();
+    int dev = 0;
+    cudaGetDevice(&dev);
+    {
+        std::lock_guard<std::mutex> lk(g_cache_mu);
+        ArenaCache& c = g_ws_cache[dev & 63];
+        if (!c.ptr) return rc;
+        cudaFree(c.ptr);
+        c = ArenaCache{};
+    }
+    const cudaError_t again = cudaMalloc(p, bytes);
+    if (again != cudaSuccess) cudaGetLastError();
+    return again;
+}
 
 static char* arena_take(size_t bytes, int dev, size_t* got) {
     {
@@ -55,7 +76,7 @@ static char* arena_take(size_t bytes, int dev, size_t* got) {
         if (c.ptr) { cudaFree(c.ptr); c = ArenaCache{}; }   // too small: give it back first
     }
     char* p = nullptr;
-    if (cudaMalloc((void**)&p, bytes) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    if (device_malloc((void**)&p, bytes) != cudaSuccess) return nullptr;
     *got = bytes;
     return p;
 }
@@ -168,6 +189,64 @@ static void arena_give(char* p, size_t bytes, int dev) {
     c.ptr = p;
     c.bytes = bytes;
 }
+
+// Workspace of a setup's factorisation: the digits of one panel of FP64 fronts on the tensor
+// cores, the diagonal-block scratch of the TF32 and 16-bit levels (2.3 or 3.3 MB a front).
+// Levels are factored one after another and share it; nothing reads it afterwards.  A
+// setup takes the device's parked block, or a new one, and parks it when it is done with the
+// device (each of several setups at once has a block of its own, and the largest stays):
+// allocating it stream-ordered on each setup stalled the host, 1.8 ms at 512 fronts (setup +
+// solve of 24 grids of 17 to 65 nodes a side 140.1 -> 130.5 ms, of 49^3 elasticity 40.1 -> 37.7
+// ms), and kept in the handle's arena it was up to 4 GB of every hierarchy a program holds.
+// Blocks over PARK_MAX go back to the driver at once.
+struct SetupWorkspace {
+    static constexpr size_t PARK_MAX = (size_t)4 << 30;
+    // room left for the setup's stream-ordered allocations (task lists, uploads)
+    static constexpr size_t HEADROOM = (size_t)256 << 20;
+    Handle& h;
+    char* ptr = nullptr;
+    size_t bytes = 0;
+    explicit SetupWorkspace(Handle& hh) : h(hh) {}
+    SetupWorkspace(const SetupWorkspace&) = delete;
+    SetupWorkspace& operator=(const SetupWorkspace&) = delete;
+
+    bool take(size_t need) {
+        {
+            std::lock_guard<std::mutex> lk(g_cache_mu);
+            ArenaCache& c = g_ws_cache[h.device & 63];
+            if (c.ptr && c.bytes >= need) {
+                ptr = c.ptr;
+                bytes = c.bytes;
+                c = ArenaCache{};
+                return true;
+            }
+            if (c.ptr) { cudaFree(c.ptr); c = ArenaCache{}; }   // too small: give it back first
+        }
+        size_t avail = 0, total = 0;
+        if (cudaMemGetInfo(&avail, &total) != cudaSuccess || avail < need + HEADROOM ||
+            cudaMalloc((void**)&ptr, need) != cudaSuccess) {
+            cudaGetLastError();
+            ptr = nullptr;
+            return false;
+        }
+        bytes = need;
+        return true;
+    }
+    ~SetupWorkspace() {
+        h.f64_ws = h.tc_ws = nullptr;
+        h.f64_ws_bytes = h.tc_ws_bytes = 0;
+        if (!ptr) return;
+        cudaStreamSynchronize(h.stream);              // (an error left work behind)
+        if (h.chain) cudaStreamSynchronize(h.chain);
+        std::lock_guard<std::mutex> lk(g_cache_mu);
+        ArenaCache& c = g_ws_cache[h.device & 63];
+        if (bytes > PARK_MAX || (c.ptr && c.bytes >= bytes)) { cudaFree(ptr); return; }
+        if (c.ptr) cudaFree(c.ptr);
+        c.ptr = ptr;
+        c.bytes = bytes;
+    }
+};
+
 void count_launch(int n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 
 int prof_begin(Handle& h, int cls, cudaStream_t stream) {
@@ -1044,34 +1123,13 @@ static int build_handle(Handle& h, Analysis& a, const int64_t* rowptr, const int
     const size_t o_bad = take(sizeof(int) * a.n_nodes);
     const size_t o_ticket = take(sizeof(int) * 2 * nl + 16);
     const size_t o_lscale = h.lu ? take(sizeof(int) * ((size_t)a.n + LU_SCALE_EXTRA)) : 0;
-    // Workspaces of the factorisation, last in the arena (levels are factored one after
-    // another and share it): the digits of one panel of FP64 fronts factored on the tensor
-    // cores, the diagonal-block scratch of the TF32 and 16-bit levels (2.3 or 3.3 MB a front:
-    // allocating it stream-ordered on each setup stalled the host, 1.8 ms at 512 fronts;
-    // setup + solve of 24 grids of 17 to 65 nodes a side 140.1 -> 130.5 ms, of 49^3
-    // elasticity 40.1 -> 37.7 ms).  Without room for it the FP64 levels run on the FP64 pipe
-    // and the others allocate their scratch.
-    size_t f64_ws = 0, tc_ws = 0;
-    for (int d = 0; d < nl; ++d) {
-        if (tc_level(h.levels[d]) && h.levels[d].factored) tc_ws = std::max(tc_ws, factor_tc_workspace((int)h.levels[d].nodes.size()));
-        if (!is_fp64(h.levels[d].prec) || !h.levels[d].factored) continue;
-        std::vector<int> rows;
-        for (int t : h.levels[d].nodes) rows.push_back(a.I_off[t + 1] - a.I_off[t] + beff(t));
-        f64_ws = std::max(f64_ws, f64_tc_workspace(rows, h.lu));
-    }
-    const size_t o_ws = off;
-    h.arena_bytes = off + std::max(f64_ws, tc_ws);
+    h.arena_bytes = off;
     {
         int dev = 0;
         cudaGetDevice(&dev);
         h.device = dev;
         size_t got = 0;
         h.arena = arena_take(h.arena_bytes, dev, &got);
-        if (!h.arena && (f64_ws || tc_ws)) {
-            f64_ws = tc_ws = 0;
-            h.arena_bytes = off;
-            h.arena = arena_take(h.arena_bytes, dev, &got);
-        }
         if (!h.arena) {
             set_last_error("device arena of " + std::to_string(h.arena_bytes) + " bytes");
             return RSD_ERR_NOMEM;
@@ -1079,14 +1137,6 @@ static int build_handle(Handle& h, Analysis& a, const int64_t* rowptr, const int
         h.arena_capacity = got;
     }
     char* A = h.arena;
-    if (f64_ws) {
-        h.f64_ws = A + o_ws;
-        h.f64_ws_bytes = f64_ws;
-    }
-    if (tc_ws) {
-        h.tc_ws = A + o_ws;
-        h.tc_ws_bytes = tc_ws;
-    }
     h.d_rowptr = (int64_t*)(A + o_rowptr);
     h.d_col = (int*)(A + o_col);
     h.d_val = (double*)(A + o_val);
@@ -1352,6 +1402,22 @@ static int build_handle(Handle& h, Analysis& a, const int64_t* rowptr, const int
     RSD_TRY(static_apply_prepare(h, (FrontDesc*)(A + o_sfronts)));
     // the tensor-core levels need tensor maps over the fronts just placed
     RSD_TRY(gemm_tc_prepare(h));
+    // The workspace comes after the setup's other allocations.  Without room for it the FP64
+    // levels run on the FP64 pipe and the others allocate their scratch.
+    SetupWorkspace ws(h);
+    size_t f64_ws = 0, tc_ws = 0;
+    for (auto& L : h.levels) {
+        if (!L.factored) continue;
+        if (tc_level(L)) tc_ws = std::max(tc_ws, factor_tc_workspace((int)L.fronts.size()));
+        if (!is_fp64(L.prec)) continue;
+        std::vector<int> rows;
+        for (auto& f : L.fronts) rows.push_back(f.N);
+        f64_ws = std::max(f64_ws, f64_tc_workspace(rows, h.lu));
+    }
+    if (std::max(f64_ws, tc_ws) && ws.take(std::max(f64_ws, tc_ws))) {
+        if (f64_ws) { h.f64_ws = ws.ptr; h.f64_ws_bytes = f64_ws; }
+        if (tc_ws) { h.tc_ws = ws.ptr; h.tc_ws_bytes = tc_ws; }
+    }
     h.prof.host_part[5] = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t_plan).count();
     // ---- numeric setup, deepest level first ----
     if (h.lu && h.f64_ws) RSD_TRY(launch_lu_scale(h));
@@ -1467,12 +1533,13 @@ extern "C" void rsd_release_cache(void) {
     std::lock_guard<std::mutex> lk(g_cache_mu);
     int cur = 0;
     cudaGetDevice(&cur);
-    for (int d = 0; d < 64; ++d) {
-        if (!g_cache[d].ptr) continue;
-        cudaSetDevice(d);
-        cudaFree(g_cache[d].ptr);
-        g_cache[d] = ArenaCache{};
-    }
+    for (int d = 0; d < 64; ++d)
+        for (ArenaCache* c : {&g_cache[d], &g_ws_cache[d]}) {
+            if (!c->ptr) continue;
+            cudaSetDevice(d);
+            cudaFree(c->ptr);
+            *c = ArenaCache{};
+        }
     cudaSetDevice(cur);
 }
 

@@ -13,7 +13,7 @@
 // Before factorisation F is spread over P (entries on or below the diagonal of F_II, and
 // F_BI) and PU (entries above it, transposed, and F_IB transposed).
 //
-// FP64 levels run in gemm_f64_tc.cu (and diag_f64.cu) unless the arena had no room for its
+// FP64 levels run in gemm_f64_tc.cu (and diag_f64.cu) unless there was no room for its
 // workspace or the entries spread too far in scale for its products.  Here, left-looking by NB-column blocks k (CUDA cores, FP32 or FP64):
 //   (a) P[k:N, blk]    -= P[k:N, 0:k]    PU[blk, 0:k]^T   (L and X columns, with the
 //                                                          diagonal block's lower part)

@@ -639,10 +639,10 @@ int gemm_tc_prepare(Handle& h) {
             if (L.op16 != TC_OP_TF32) RSD_TRY(encode_2d(&maps[tc_map_panel16(f.node)], f.P16, f.s, f.N, f.ldp, L.op16));
         }
     }
-    RSD_CUDA_TRY(cudaMalloc((void**)&st->d_maps, maps.size() * sizeof(CUtensorMap)));
+    RSD_CUDA_TRY(device_malloc((void**)&st->d_maps, maps.size() * sizeof(CUtensorMap)));
     st->ws_slots = 2 * h.num_sms;
     for (auto& b : st->buf)
-        RSD_CUDA_TRY(cudaMalloc((void**)&b.d_ws, (size_t)st->ws_slots * BM * 256 * sizeof(float)));
+        RSD_CUDA_TRY(device_malloc((void**)&b.d_ws, (size_t)st->ws_slots * BM * 256 * sizeof(float)));
     RSD_CUDA_TRY(cudaMemcpy(st->d_maps, maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice));
     return RSD_OK;
 }
@@ -1070,10 +1070,10 @@ int gemm_tc_autotune(const char* path, cudaStream_t stream, int num_sms, double*
     RSD_TRY(encode_2d(&maps[tc_map_panel16(0)], buf + o_a16, Kmax, Mmax, Kmax, TC_OP_F16));
     RSD_TRY(encode_2d(&maps[tc_map_panel(1)], B, Kmax, Nn, Kmax));
     RSD_TRY(encode_2d(&maps[tc_map_panel16(1)], buf + o_b16, Kmax, Nn, Kmax, TC_OP_F16));
-    RSD_CUDA_TRY(cudaMalloc((void**)&st->d_maps, maps.size() * sizeof(CUtensorMap)));
+    RSD_CUDA_TRY(device_malloc((void**)&st->d_maps, maps.size() * sizeof(CUtensorMap)));
     RSD_CUDA_TRY(cudaMemcpy(st->d_maps, maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice));
     st->ws_slots = 2 * num_sms;
-    for (auto& b : st->buf) RSD_CUDA_TRY(cudaMalloc((void**)&b.d_ws, (size_t)st->ws_slots * BM * 256 * sizeof(float)));
+    for (auto& b : st->buf) RSD_CUDA_TRY(device_malloc((void**)&b.d_ws, (size_t)st->ws_slots * BM * 256 * sizeof(float)));
     auto time_one = [&](const GemmTask& t, int op, float* best) -> int {
         *best = 1e30f;
         for (int rep = 0; rep < 3; ++rep) {

@@ -35,6 +35,7 @@ enum ErrSlot { ERR_NOT_SPD = 0, ERR_TIMEOUT = 1, ERR_NOT_SPD_NODE = 2, ERR_SPREA
     } while (0)
 
 void set_last_error(const std::string& msg);
+cudaError_t device_malloc(void** p, size_t bytes);   // cudaMalloc; parked workspaces give way to it
 
 inline int elem_bytes(int prec) { return prec == RSD_PREC_FP64 ? 8 : 4; }
 inline bool is_fp64(int prec) { return prec == RSD_PREC_FP64; }
@@ -226,12 +227,12 @@ struct Handle {
     size_t arena_bytes = 0;
     size_t arena_capacity = 0;          // bytes of the block actually held (cache reuse)
     int device = 0;
-    // digits of FP64 fronts on the tensor cores (gemm_f64_tc.cu), in the arena; null when
-    // the arena only fits without it (those fronts then run on the FP64 pipe)
+    // during rsd_setup only: digits of FP64 fronts on the tensor cores (gemm_f64_tc.cu; null
+    // when there is no room for them: those fronts then run on the FP64 pipe)
     char* f64_ws = nullptr;
     size_t f64_ws_bytes = 0;
     int* d_lu_scale = nullptr;           // nonsymmetric FP64 fronts: see launch_lu_scale
-    char* tc_ws = nullptr;               // scratch of a tensor-core level (factor_tc_workspace), or null
+    char* tc_ws = nullptr;               // and scratch of a tensor-core level (factor_tc_workspace), or null
     size_t tc_ws_bytes = 0;
     int* d_err = nullptr;
     int* d_front_bad = nullptr;          // per node: a pivot of its factorisation failed
