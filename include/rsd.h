@@ -300,6 +300,12 @@ int rsd_inject_drop_sweep_item(rsd_handle h, int32_t level);
  * context stays usable.                                                               */
 int rsd_inject_setup_timeout(void);
 
+/* rsd_inject_workspace_limit -- the next rsd_setup (or rsd_setup_batched) of the calling
+ * thread finds room for at most `bytes` of factorisation workspace: FP64 fronts are then
+ * factored fewer at a time, or on CUDA cores when one front's does not fit, and TF32 and
+ * 16-bit levels allocate their scratch as they go.  RSD_ERR_ARG if bytes < 0.           */
+int rsd_inject_workspace_limit(int64_t bytes);
+
 /* rsd_check -- synchronise the handle's stream and report any device-side error flag
  * (timeout of a bounded wait, failed pivot) raised since setup.                        */
 int rsd_check(rsd_handle h);

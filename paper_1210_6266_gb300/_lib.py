@@ -43,7 +43,8 @@ EXPORTS = [
     "rsd_profile", "rsd_launch_count", "rsd_apply_static", "rsd_last_error_detail",
     "rsd_release_cache", "rsd_setup_batched", "rsd_solve_adjoint", "rsd_grid_exp",
     "rsd_grid_coef_grad", "rsd_profile_trace", "rsd_peak_gemm",
-    "rsd_inject_drop_sweep_item", "rsd_inject_setup_timeout", "rsd_grid_elastic_sizes", "rsd_grid_elastic_assemble",
+    "rsd_inject_drop_sweep_item", "rsd_inject_setup_timeout", "rsd_inject_workspace_limit",
+    "rsd_grid_elastic_sizes", "rsd_grid_elastic_assemble",
     "rsd_grid_elastic_load", "rsd_grid_elastic_partition", "rsd_autotune", "rsd_tune_load",
     "rsd_front_factor_upper",
 ]
@@ -114,6 +115,7 @@ def load() -> C.CDLL:
             "rsd_check": (C.c_int, [P]),
             "rsd_inject_drop_sweep_item": (C.c_int, [P, C.c_int32]),
             "rsd_inject_setup_timeout": (C.c_int, []),
+            "rsd_inject_workspace_limit": (C.c_int, [C.c_int64]),
             "rsd_destroy": (None, [P]),
             "rsd_strerror": (C.c_char_p, [C.c_int]),
             "rsd_last_error_detail": (C.c_char_p, []),

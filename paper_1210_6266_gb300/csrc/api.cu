@@ -33,6 +33,8 @@ static std::atomic<long long> g_launches(0);
 
 // rsd_inject_setup_timeout: the calling thread's next rsd_setup (taken by build_handle)
 static thread_local bool t_inject_setup_timeout = false;
+// rsd_inject_workspace_limit: the same, < 0 for none (taken by its SetupWorkspace)
+static thread_local int64_t t_inject_workspace_limit = -1;
 
 // One cached arena per device: rsd_destroy parks its arena here instead of freeing it and
 // the next rsd_setup on that device reuses it when it is large enough (the arena of a
@@ -206,11 +208,13 @@ struct SetupWorkspace {
     Handle& h;
     char* ptr = nullptr;
     size_t bytes = 0;
-    explicit SetupWorkspace(Handle& hh) : h(hh) {}
+    int64_t limit;                                    // rsd_inject_workspace_limit
+    explicit SetupWorkspace(Handle& hh) : h(hh), limit(t_inject_workspace_limit) { t_inject_workspace_limit = -1; }
     SetupWorkspace(const SetupWorkspace&) = delete;
     SetupWorkspace& operator=(const SetupWorkspace&) = delete;
 
     bool take(size_t need) {
+        if (limit >= 0 && need > (size_t)limit) return false;
         {
             std::lock_guard<std::mutex> lk(g_cache_mu);
             ArenaCache& c = g_ws_cache[h.device & 63];
@@ -1402,22 +1406,25 @@ static int build_handle(Handle& h, Analysis& a, const int64_t* rowptr, const int
     RSD_TRY(static_apply_prepare(h, (FrontDesc*)(A + o_sfronts)));
     // the tensor-core levels need tensor maps over the fronts just placed
     RSD_TRY(gemm_tc_prepare(h));
-    // The workspace comes after the setup's other allocations.  Without room for it the FP64
-    // levels run on the FP64 pipe and the others allocate their scratch.
+    // The workspace comes after the setup's other allocations.  Where there is no room for all
+    // of it, FP64 fronts take turns on what there is, one at a time at least (the tensor cores
+    // are 18 times as fast as the FP64 pipe at 57^3); without room for one front the FP64
+    // levels run on the FP64 pipe.  TF32 and 16-bit levels it does not hold allocate theirs.
     SetupWorkspace ws(h);
-    size_t f64_ws = 0, tc_ws = 0;
+    size_t f64_ws = 0, f64_min = 0, tc_ws = 0;
     for (auto& L : h.levels) {
         if (!L.factored) continue;
         if (tc_level(L)) tc_ws = std::max(tc_ws, factor_tc_workspace((int)L.fronts.size()));
         if (!is_fp64(L.prec)) continue;
         std::vector<int> rows;
         for (auto& f : L.fronts) rows.push_back(f.N);
-        f64_ws = std::max(f64_ws, f64_tc_workspace(rows, h.lu));
+        f64_ws = std::max(f64_ws, f64_tc_workspace(rows, h.lu, &f64_min));
     }
-    if (std::max(f64_ws, tc_ws) && ws.take(std::max(f64_ws, tc_ws))) {
-        if (f64_ws) { h.f64_ws = ws.ptr; h.f64_ws_bytes = f64_ws; }
-        if (tc_ws) { h.tc_ws = ws.ptr; h.tc_ws_bytes = tc_ws; }
-    }
+    size_t want = std::max(f64_ws, tc_ws);
+    while (want && !ws.take(want))                       // (the other levels' scratch goes first)
+        want = want > f64_ws ? f64_ws : want > f64_min ? std::max(f64_min, want / 2) : 0;
+    if (f64_ws && want >= f64_min) { h.f64_ws = ws.ptr; h.f64_ws_bytes = std::min(want, f64_ws); }
+    if (tc_ws && want >= tc_ws) { h.tc_ws = ws.ptr; h.tc_ws_bytes = tc_ws; }
     h.prof.host_part[5] = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t_plan).count();
     // ---- numeric setup, deepest level first ----
     if (h.lu && h.f64_ws) RSD_TRY(launch_lu_scale(h));
@@ -1750,6 +1757,12 @@ extern "C" int rsd_inject_drop_sweep_item(rsd_handle hh, int32_t level) {
 
 extern "C" int rsd_inject_setup_timeout(void) {
     t_inject_setup_timeout = true;
+    return RSD_OK;
+}
+
+extern "C" int rsd_inject_workspace_limit(int64_t bytes) {
+    if (bytes < 0) return RSD_ERR_ARG;
+    t_inject_workspace_limit = bytes;
     return RSD_OK;
 }
 

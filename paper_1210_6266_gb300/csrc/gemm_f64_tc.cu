@@ -732,10 +732,11 @@ int launch_lu_scale(Handle& h) {
 // Workspace of a level: the digits of one 512-wide panel of every front at once where that
 // fits the cap (groups of fronts then take turns), of one front at least.  The cap is far
 // above what fills the chip: 4 GiB hold over 100 fronts of 4000 rows, thousands of tiles.
-size_t f64_tc_workspace(const std::vector<int>& rows, bool lu) {
+size_t f64_tc_workspace(const std::vector<int>& rows, bool lu, size_t* least) {
     const size_t cap = (size_t)4 << 30;
     size_t sum = 0, most = 0;
     for (int N : rows) { sum += (lu ? 2 : 1) * front_bytes(N); most = std::max(most, (lu ? 2 : 1) * front_bytes(N)); }
+    *least = std::max(*least, most);
     return std::min(sum, std::max(cap, most));
 }
 

@@ -390,8 +390,9 @@ int run_factor_level(Handle& h, int li);
 // fronts [f0, f0 + nf) of level li (diag_f64.cu)
 int launch_diag_f64(Handle& h, int li, int f0, int nf, int k, cudaStream_t st);
 // FP64 level on the tensor cores (gemm_f64_tc.cu): workspace for fronts of the given row
-// counts, and the partial Cholesky or LU of the level (needs the handle's f64_ws)
-size_t f64_tc_workspace(const std::vector<int>& rows, bool lu);
+// counts (*least is raised to what the largest one alone needs), and the partial Cholesky or LU
+// of the level (needs the handle's f64_ws)
+size_t f64_tc_workspace(const std::vector<int>& rows, bool lu, size_t* least);
 int factor_level_f64_tc(Handle& h, int li);
 // nonsymmetric K: the exponents of its diagonal (n ints) and LU_SCALE_EXTRA more for the
 // choice of the scaling its split products use, to h.d_lu_scale
