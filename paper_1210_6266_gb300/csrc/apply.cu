@@ -16,6 +16,7 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <atomic>
 #include <climits>
 #include <mutex>
 
@@ -1322,7 +1323,7 @@ void launch_bwd(int gd, bool h16, int grid, cudaStream_t st, const FrontDesc* fr
 // Clusters of the cluster sweeps resident at once on the current device (the persistent
 // grid), looked up once per device.
 int cl_grid(int n_items, int* out) {
-    static int max_cl[64] = {};
+    static std::atomic<int> max_cl[64];          // (threads that ask at once store the same count)
     int dev = 0;
     RSD_CUDA_TRY(cudaGetDevice(&dev));
     if (dev < 0 || dev >= 64) return RSD_ERR_ARG;
@@ -1338,13 +1339,13 @@ int cl_grid(int n_items, int* out) {
         RSD_CUDA_TRY(cudaOccupancyMaxActiveClusters(&n2, (void*)k_bwd_sweep_cl, &cfg));
         max_cl[dev] = std::max(1, std::min(n1, n2));
     }
-    *out = std::max(1, std::min(n_items, max_cl[dev]));
+    *out = std::max(1, std::min(n_items, max_cl[dev].load()));
     return RSD_OK;
 }
 
 // Clusters of the FP64 cluster sweeps resident at once on the current device.
 int f64_cl_grid(int n_items, int* out) {
-    static int max_cl[64] = {};
+    static std::atomic<int> max_cl[64];          // (threads that ask at once store the same count)
     int dev = 0;
     RSD_CUDA_TRY(cudaGetDevice(&dev));
     if (dev < 0 || dev >= 64) return RSD_ERR_ARG;
@@ -1357,7 +1358,7 @@ int f64_cl_grid(int n_items, int* out) {
         RSD_CUDA_TRY(cudaOccupancyMaxActiveClusters(&n2, (void*)k_bwd_sweep_f64, &cfg));
         max_cl[dev] = std::max(1, std::min(n1, n2));
     }
-    *out = std::max(1, std::min(n_items, max_cl[dev]));
+    *out = std::max(1, std::min(n_items, max_cl[dev].load()));
     return RSD_OK;
 }
 

@@ -20,6 +20,7 @@
 // L fills the lower triangle of a 128 x 129 array, X (transposed, one column further
 // right) its upper triangle.
 #include <algorithm>
+#include <atomic>
 
 #include "cluster.cuh"
 #include "rsd_internal.cuh"
@@ -516,13 +517,14 @@ int launch_cl(DiagKernel kern, int CL, size_t smem, const FrontDesc* d_fronts, i
 
 }  // namespace
 
-// How many clusters of 16 (more than the portable 8) the current device holds at once; 0
-// where it takes none.
-static int wide_clusters(DiagKernel kern, size_t smem) {
-    static int known[64][2] = {};
+// How many clusters of 16 (more than the portable 8) of the Cholesky or the LU kernel the
+// current device holds at once; 0 where it takes none.  (Threads that ask at once store the
+// same count.)
+static int wide_clusters(DiagKernel kern, size_t smem, bool lu) {
+    static std::atomic<int> known[64][2];
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) { cudaGetLastError(); return 0; }
-    int& n = known[dev][smem == LU_SMEM];
+    int n = known[dev][lu].load(std::memory_order_relaxed);
     if (!n) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(16 * 16);
@@ -542,6 +544,7 @@ static int wide_clusters(DiagKernel kern, size_t smem) {
             m = 0;
         }
         n = m + 1;
+        known[dev][lu].store(n, std::memory_order_relaxed);
     }
     return n - 1;
 }
@@ -568,7 +571,7 @@ int launch_diag_f64(Handle& h, int li, int f0, int nf, int k, cudaStream_t st) {
         {k_lu_diag_f64<1>, k_lu_diag_f64<2>, k_lu_diag_f64<4>, k_lu_diag_f64<8>, k_lu_diag_f64<16>}};
     const size_t smem = h.lu ? LU_SMEM : DIAG_SMEM;
     int lg = alive * 8 <= h.num_sms ? 3 : alive * 4 <= h.num_sms ? 2 : alive * 2 <= h.num_sms ? 1 : 0;
-    if (lg == 3 && alive <= wide_clusters(kern[h.lu][4], smem)) lg = 4;
+    if (lg == 3 && alive <= wide_clusters(kern[h.lu][4], smem, h.lu)) lg = 4;
     const int rc = launch_cl(kern[h.lu][lg], 1 << lg, smem, fr, nf, k, h.d_err, h.d_front_bad, st);
     prof_end(h, pi, flops, bytes, st);
     return rc;
