@@ -1045,7 +1045,11 @@ k_bwd_sweep_cl(const FrontDesc* __restrict__ fronts, const int* __restrict__ ite
 // Work items, their order and the waits are those of the per-CTA kernels.
 constexpr int F64_CL = 8;
 constexpr int F64_R = NB / F64_CL;               // rows per CTA of a block
-constexpr int F64_CL_FRONTS = 16;               // levels of at most this many fronts
+// levels of at most this many fronts: one application of 1, 8, 12, 16, 24, 32, 48, 63 problems of
+// 17^3 in one hierarchy, their roots on CTAs of their own 224 249 277 308 375 445 580 709 us, on
+// clusters 118 217 220 253 332 416 588 743; of 33^3, 1.26 3.00 4.11 5.20 7.50 9.83 14.5 19.0 ms
+// against 0.67 3.14 3.89 5.06 7.46 9.85 14.7 19.2 (the 8's with their 64 leaves, the 1's with 8)
+constexpr int F64_CL_FRONTS = 16;
 constexpr int F64_AHEAD = 4;                     // blocks whose factor entries are loaded before their wait
 static_assert(F64_R == 2 * AW, "two rows per warp");
 

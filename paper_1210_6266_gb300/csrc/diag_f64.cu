@@ -39,7 +39,7 @@ __device__ __forceinline__ void cl_st_f64(uint32_t a, double v) {
 }
 
 // 1 / sqrt(d) for d > 0: an FP32 estimate y of the reduced argument (2^-21) and one
-// third-order Householder step, y + y e (1/2 + 3/8 e) with e = 1 - d y^2.
+// third-order Householder step, y + y e (1/2 + 3/8 e) with e = 1 - d y^2 (1.5 roundings).
 __device__ __forceinline__ double rsqrt_chain(double d) {
     const long long b = __double_as_longlong(d);
     const int ex = (int)(b >> 52) - 1023;
@@ -52,8 +52,10 @@ __device__ __forceinline__ double rsqrt_chain(double d) {
     return fma(y * e, fma(0.375, e, 0.5), y);
 }
 
-// 1 / d for finite d != 0: an FP32 estimate y (2^-22) and y + y (e + e^2), e = 1 - d y: three
-// FMAs deep on the chain from pivot to pivot (about 260 clocks; 1.0 / d takes 360).
+// 1 / d for finite d != 0: an FP32 estimate y (2^-22) and the third-order hyperpower step
+// (Altman, "An optimum cubically convergent iterative method of inverting a linear bounded
+// operator", 1960) y + y (e + e^2), e = 1 - d y: three FMAs deep on the chain from pivot to pivot
+// (about 260 clocks; 1.0 / d takes 360).  One rounding of 1 / d.
 __device__ __forceinline__ double rcp_chain(double d) {
     const long long b = __double_as_longlong(d);
     const int ex = (int)((b >> 52) & 0x7ff) - 1023;
