@@ -131,7 +131,9 @@ typedef struct {
     int32_t restart;     /* FGMRES restart length (<= 0: 30)                                */
     const char* tune_cache; /* path of a table written by rsd_autotune (host string, read at
                             setup): the tile width and split-K count of the tensor-core
-                            updates by size bucket; NULL = built-in rules                  */
+                            Schur and outer panel updates by size bucket (the short products
+                            of the diagonal blocks' chain take fixed tiles); NULL =
+                            built-in rules                                                 */
     int32_t nonsymmetric;/* nonzero: K is not symmetric (its sparsity pattern must be): every
                             front is factored F_II = L U without pivoting (Eqs. 3.2-3.3 with
                             K_IL != K_LI^T, as the two-variable systems of Sec. 4, Eqs.
@@ -313,7 +315,7 @@ int rsd_check(rsd_handle h);
 /* rsd_destroy -- release the handle.  Its device arena is kept in a one-slot per-device
  * cache and reused by the next rsd_setup on that device if large enough (the previously
  * cached block, if smaller, is freed), and so is, from one rsd_setup to the next, the
- * workspace of its factorisation (4 GiB at most; it gives way when another allocation of
+ * workspace of its factorisation (16 GiB at most; it gives way when another allocation of
  * the library needs the room).  rsd_release_cache() frees the cached blocks.             */
 void        rsd_destroy(rsd_handle h);
 void        rsd_release_cache(void);

@@ -200,9 +200,10 @@ static void arena_give(char* p, size_t bytes, int dev) {
 // allocating it stream-ordered on each setup stalled the host, 1.8 ms at 512 fronts (setup +
 // solve of 24 grids of 17 to 65 nodes a side 140.1 -> 130.5 ms, of 49^3 elasticity 40.1 -> 37.7
 // ms), and kept in the handle's arena it was up to 4 GB of every hierarchy a program holds.
-// Blocks over PARK_MAX go back to the driver at once.
+// Blocks over PARK_MAX (6 % of the device) go back to the driver at once: 4096 TF32 leaves need
+// 9.7 GB, and 65^3 in as many took 30.5 ms a setup + solve without a parked block, 25.6 with.
 struct SetupWorkspace {
-    static constexpr size_t PARK_MAX = (size_t)4 << 30;
+    static constexpr size_t PARK_MAX = (size_t)16 << 30;
     // room left for the setup's stream-ordered allocations (task lists, uploads)
     static constexpr size_t HEADROOM = (size_t)256 << 20;
     Handle& h;
@@ -1633,7 +1634,7 @@ extern "C" int rsd_setup(const rsd_csr* K, const int32_t* dof_node, const rsd_tr
         const int ps[3] = {o.prec_leaf, o.prec_mid, o.prec_root};
         for (int p : ps)
             if (p != RSD_PREC_FP64 && p != RSD_PREC_FP32) {
-                set_last_error("nonsymmetric fronts (LU) are factored in FP64 or FP32 on CUDA cores");
+                set_last_error("nonsymmetric fronts (LU) are factored in FP64 or FP32");
                 return RSD_ERR_ARG;
             }
         if (o.krylov == RSD_KRYLOV_PCG || (o.mode == RSD_MODE_PAPER && o.gamma == 0)) {
