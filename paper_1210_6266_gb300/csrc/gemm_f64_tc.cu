@@ -22,9 +22,13 @@
 // updated with one FP64 subtraction.  The pairs left out (d = 8 and beyond) are of
 // either sign but for the squares of digit 4 on C's diagonal (X X^T): those are summed per
 // row and added (without them every pivot is biased one way).
-// Error of a 57^3 log-normal diffusion solve against the assembled system's solution
-// refined in extended precision: 0.9e-15 this way, 3.8e-15 with FMAs on the FP64 pipe (with
-// exponents fixed by sqrt(K_ii), most entries of a row being far smaller, 1e-11).  A Schur
+// Error of 57^3 log-normal diffusion solves (three loads) against the assembled system's
+// solution, refined with extended-precision residuals: 9.0, 5.0 and 5.3e-16 this way, 37.6, 18.5
+// and 16.0e-16 with FMAs on the FP64 pipe (of 37^3 convection-diffusion, LU: 4.9, 4.3, 5.9 against
+// 6.7, 6.2, 7.0).  A plain FP64 CG on the unassembled operator is itself 46, 25 and 18e-16 from
+// that solution and lies nearer to the FMA form's answers (17, 14, 12 against 53, 26, 18): a
+// comparison with one says more about the two roundings' likeness than about either error.
+// (With exponents fixed by sqrt(K_ii), most entries of a row being far smaller, 1e-11.)  A Schur
 // complement that cancels to 1e-7 of its terms is off by half a unit of those terms (rms), by 2 to 5
 // units with FMAs.
 //
