@@ -12,7 +12,7 @@ Metric: DOF / (t_setup + t_solve) per step, mixed form against the plain FP64 fo
 The default run prints one JSON line: the mixed form (factor entries rounded to TF32, the
 long Schur updates on FP16 operand copies, FP16 sweeps, FP64 PCG) on the 129^3 workload
 (K timed steps after W warm-up steps) as the headline, and, in the same line, the plain
-FP64 form of the same workload (one timed step: it takes over a minute), the 256-problem
+FP64 form of the same workload (one timed step of about 3 s), the 256-problem
 batched workload in both forms (BF16 operands; the FP64 form on its first 64 problems),
 paper mode with gamma = 8 inner GMRES iterations and FGMRES, the measured peaks of the
 library's own GEMM kernels, and the oracle's CPU baseline.
@@ -497,7 +497,7 @@ def main() -> None:
                                      f"trilinear hex, E per leaf log-uniform [1, 1e3], nu = {ELASTIC_NU}, "
                                      f"{8 ** ework['depth']} leaves (depth {ework['depth']})"),
                            n_dof=eprob["n_dof"], steps=2, warmup=1,
-                           fp64_form="not timed: about 3.5e14 flops of FP64 factorisation, some 5 minutes")
+                           fp64_form="not timed: about 3.5e14 flops of FP64 factorisation")
         del eprob
     paper_rec = None
     if single and not args.no_paper and not batched and args.mode == "exact" and args.form == "mixed":
