@@ -7,9 +7,10 @@
 // so 36 exact FP16 products per FP64 product are over fifty times cheaper.
 //
 // Digits.  Row i of an operand has an exponent e_i with |entry| < 2^e_i, taken from its
-// entries in the columns of the product (128 for a panel solve, up to 512 for an update).  An entry is rounded to a multiple of 2^(e_i - FB) and written as eight balanced
-// digits of DB bits, x = 2^(e_i - FB) sum_k d_k 2^(DB (7 - k)), stored as FP16 integers of
-// magnitude at most 1024.  Products: C = the sum over digit pairs with i + j = d <= 7 of
+// entries in the columns of the product (128 for a panel solve, up to 512 for an update).
+// An entry is rounded to a multiple of 2^(e_i - FB) and written as eight balanced digits of DB
+// bits, x = 2^(e_i - FB) sum_k d_k 2^(DB (7 - k)), stored as FP16 integers of magnitude at
+// most 1024.  Products: C = the sum over digit pairs with i + j = d <= 7 of
 // 2^(DB (14 - d)) (D_i D_j^T); a sum over pairs and K columns that stays below 2^24 is exact in FP32,
 // whatever its order:
 //   updates, K <= 512: DB = 7, FB = 59 (|d_k| <= 64), and e_i such that a row's sum of
@@ -47,8 +48,9 @@
 // error of a product below 2^(2 SPREAD_MAX - 59) Dr_i Dc_j (Cholesky's bound has 0 there); one
 // further up raises ERR_SPREAD, and the setup factors the hierarchy again on the FP64 pipe.
 // Fronts of 300 diagonally dominant unknowns with rows, or rows and columns, scaled over
-// 2^-40 .. 2^40: entries of L wrong by 4e-3 with t_k = 0, now as the unscaled fronts'.  A 37^3
-// convection-diffusion system: 16.41 -> 16.49 ms.
+// 2^-40 .. 2^40: entries of L wrong by 4e-3 with t_k = 0, now as the unscaled fronts'.  37^3
+// convection-diffusion, setup + solve: 16.45 -> 16.65 ms with the scales and the subnormals below
+// (57^3 FP64, for those: 61.6 -> 62.1).
 //
 // Kernel.  A 128 x 64 tile keeps its eight sums in TMEM (8 x 64 columns, all 512).  Digit
 // rows of B are stacked in shared memory, so one MMA of N = 256 multiplies digit i of A by
